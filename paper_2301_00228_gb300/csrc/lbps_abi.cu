@@ -164,6 +164,21 @@ int build_boundary(const lbps_params* p, const uint8_t* node_type, const double*
             if (!body(i + DX[d], j + DY[d])) return true;
         return false;
     };
+    // difference stencils of point (i, j) (already in the lattice): x in bits 0, 1, y in bits 2, 3
+    auto kinds_at = [&](int i, int j) {
+        auto kind = [&](int dx, int dy) {
+            const bool hp = body(i + dx, j + dy), hm = body(i - dx, j - dy);
+            return hp && hm ? lbps::DIFF_CENTRAL : hp ? lbps::DIFF_FORWARD : lbps::DIFF_BACKWARD;
+        };
+        return (int)kind(1, 0) | (int)kind(0, 1) << 2;
+    };
+    // ... and of its body neighbours E, N, W, S, 4 bits each above them (BNode::kinds)
+    auto kinds_of = [&](int i, int j) {
+        int k = kinds_at(i, j);
+        for (int d = 0; d < 4; ++d)
+            if (body(i + DX[d], j + DY[d])) k |= kinds_at((i + DX[d] + nx) % nx, (j + DY[d] + ny) % ny) << (4 + 4 * d);
+        return k;
+    };
     auto bvalue = [&](size_t k, double& bx, double& by) {
         bx = bc_value ? bc_value[2 * k] : 0.0;
         by = bc_value ? bc_value[2 * k + 1] : 0.0;
@@ -203,6 +218,7 @@ int build_boundary(const lbps_params* p, const uint8_t* node_type, const double*
                 node.smask = smask;
                 node.bx = bx;
                 node.by = by;
+                node.kinds = kinds_of(i, j);
                 out.bn[q] = node;
             }
         }
@@ -262,6 +278,7 @@ int build_boundary(const lbps_params* p, const uint8_t* node_type, const double*
                 }
                 node.inv_m = 1.0 / (p->rho * vol);
             }
+            node.kinds = kinds_of(i, j);
             out.bn.push_back(node);
         }
     }
@@ -846,6 +863,10 @@ int lbps_create_cells(const lbps_params* params, const uint8_t* node_type, const
     c.a[1] = lat->a_psi;
     c.a0[0] = params->a0_phi;
     c.a0[1] = lat->a0_psi;
+    c.two_mu = 2.0 * mu;
+    c.half_dh = 0.5 * dh;
+    c.dt2 = dt + dt;
+    c.quarter_dh = 0.25 * dh;
     c.two_dt2 = 2.0 / (dt * dt);
     c.two_dt = 2.0 / dt;
     c.inv_rho_dh2 = 1.0 / (rho * dh * dh);

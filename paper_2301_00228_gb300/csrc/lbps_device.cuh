@@ -35,6 +35,19 @@ __device__ __forceinline__ bool chk_ok(const P* p, int line) {
         g_chk_addr = reinterpret_cast<unsigned long long>(c);
     return ok;
 }
+// Each translation unit of kernels has its own copy of the table.
+static inline cudaError_t upload_check_table(const char* const* los, const char* const* his, int n) {
+    cudaError_t e = cudaSuccess;
+    if (n > 0) e = cudaMemcpyToSymbol(g_chk_lo, los, n * sizeof(const char*));
+    if (e == cudaSuccess && n > 0) e = cudaMemcpyToSymbol(g_chk_hi, his, n * sizeof(const char*));
+    if (e == cudaSuccess) e = cudaMemcpyToSymbol(g_chk_n, &n, sizeof(n));
+    return e;
+}
+static inline int read_check_report(unsigned long long out[2]) {
+    if (cudaMemcpyFromSymbol(&out[0], g_chk_line, sizeof(out[0])) != cudaSuccess) return -1;
+    if (cudaMemcpyFromSymbol(&out[1], g_chk_addr, sizeof(out[1])) != cudaSuccess) return -1;
+    return 1;
+}
 #define LBPS_LDG(p) (::lbps::chk_ok((p), __LINE__) ? __ldg(p) : decltype(__ldg(p))(0))
 #define LBPS_LD(p) (::lbps::chk_ok((p), __LINE__) ? *(p) : decltype(+*(p))(0))
 #define LBPS_ST(p, v)                                      \
@@ -45,6 +58,21 @@ __device__ __forceinline__ bool chk_ok(const P* p, int line) {
 #define LBPS_LDG(p) __ldg(p)
 #define LBPS_LD(p) (*(p))
 #define LBPS_ST(p, v) (*(p) = (v))
+#endif
+// A load of data that other blocks of the same launch may have written (NC =
+// false: an ordinary load, which sees them after the launch's barrier) or of
+// data nothing in the launch writes (NC = true: the read-only path).
+#ifdef LBPS_CHECKED
+#define LBPS_LDX(NC, p) ((NC) ? LBPS_LDG(p) : LBPS_LD(p))
+#else
+template <bool NC, typename T>
+__device__ __forceinline__ T load_nc(const T* p) {
+    if constexpr (NC)
+        return __ldg(p);
+    else
+        return *p;
+}
+#define LBPS_LDX(NC, p) ::lbps::load_nc<NC>(p)
 #endif
 
 // Lattice geometry.  Planes are pitched: row j of a plane starts at j * px.
@@ -79,6 +107,9 @@ struct Consts {
     double load_hold[2];        // t_hold: the factor is min(t, t_hold) / t_ramp
     int bc_feq_mode;            // Eq. LBE_mod reading
     int bc_j_mode;              // J of Eq. correction-f: 0 stored, 1 partial LBE update
+    double two_mu;              // 2 mu
+    double half_dh, quarter_dh; // dh / 2, dh / 4
+    double dt2;                 // 2 Delta t
 };
 
 // Time factor of the boundary data of one kind (0 Neumann, 1 Dirichlet) at
@@ -127,8 +158,13 @@ struct BNode {
     double inv_m;    // 1 / (rho V_C) of the cell (general geometry)
     double l[4];     // in-body lengths of the cell's sides E, N, W, S (general geometry)
     int nbmask;      // bit d: the neighbour in direction d is in the body (general geometry)
-    int pad;
+    int kinds;       // difference stencils (DIFF_*), 2 bits each: the point's own along x (bits 0, 1) and
+                     // y (2, 3), then x and y at its body neighbours E, N, W, S (bits 4 + 4 d ..)
 };
+
+// Second-order difference stencils along an axis (reading R4): central, or
+// one-sided three-point towards larger / smaller indices.
+enum { DIFF_CENTRAL = 0, DIFF_FORWARD = 1, DIFF_BACKWARD = 2 };
 
 enum { NEUMANN = 1, DIRICHLET = 2, VOID = 3 };
 
@@ -256,6 +292,33 @@ __device__ inline double ddy(const double* __restrict__ g, size_t stride, int i,
     return mul_rn(acc, inv2h);
 }
 
+// FP32 -> FP64 exactly by integer operations only (the conversion
+// instruction runs on the FP64 pipe, which the update keeps busy): the
+// binary32 sign, exponent and fraction placed in binary64's fields.  Normal
+// numbers: exponent rebased from 127 to 1023, fraction shifted up 29 bits.
+// Zero: zero.  Subnormals m 2^-149 (m < 2^23, leading one at bit k):
+// exponent k - 149 + 1023, the bits below the leading one as the fraction.
+// Infinity and NaN: exponent 2047, the fraction (a NaN's payload) kept.
+__device__ __forceinline__ double widen(double x) { return x; }
+__device__ __forceinline__ double widen(float f) {
+    const unsigned u = __float_as_uint(f);
+    const unsigned e = (u >> 23) & 0xffu;
+    unsigned hi = ((u >> 3) & 0x0fffffffu) + (896u << 20), lo = u << 29;
+    if (e - 1u >= 254u) {   // zero, subnormal, infinity, NaN
+        unsigned m = u & 0x7fffffu, E = 0u;
+        if (e == 255u) {
+            E = 2047u;
+        } else if (m != 0u) {
+            const unsigned k = 31u - (unsigned)__clz(m);   // bit of the leading one, 0..22
+            E = k + 874u;
+            m = (m << (23u - k)) & 0x7fffffu;
+        }
+        hi = (E << 20) | (m >> 3);
+        lo = m << 29;
+    }
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)lo);
+}
+
 // Interior acceleration, Eq. navier: a = c_d^2 grad(phi) - c_s^2 curl(psi e_z)
 // with central differences of the neighbours' moments.  Evaluated in the
 // population type T and widened to FP64 for the Newmark update.
@@ -267,13 +330,15 @@ __device__ __forceinline__ void accel_interior_v(T phiW, T phiE, T phiS, T phiN,
     ax = fma_rn(k.cd2h, dphix, -mul_rn(k.cs2h, dpsiy));
     ay = fma_rn(k.cd2h, dphiy, mul_rn(k.cs2h, dpsix));
 }
-template <typename T>
+// INT: widened with integer operations (fewer FP64 instructions, more
+// registers).
+template <typename T, bool INT>
 __device__ __forceinline__ void accel_interior(T phiW, T phiE, T phiS, T phiN, T psiW, T psiE, T psiS,
                                                T psiN, const KC<T>& k, double& ax, double& ay) {
     T x, y;
     accel_interior_v<T>(phiW, phiE, phiS, phiN, psiW, psiE, psiS, psiN, k, x, y);
-    ax = (double)x;
-    ay = (double)y;
+    ax = INT ? widen(x) : (double)x;
+    ay = INT ? widen(y) : (double)y;
 }
 
 // Eq. integration (explicit Newmark as printed).
@@ -289,37 +354,10 @@ __device__ __forceinline__ void newmark(double u, double v, double a, const Cons
 // and 16-bit storages, as the accelerations themselves), so u and v take 3
 // FP64 fused multiply-adds each instead of 6; they differ from two calls of
 // newmark by rounding only.
-// FP32 -> FP64 exactly by integer operations only (the conversion
-// instruction runs on the FP64 pipe, which the update keeps busy): the
-// binary32 sign, exponent and fraction placed in binary64's fields.  Normal
-// numbers: exponent rebased from 127 to 1023, fraction shifted up 29 bits.
-// Zero: zero.  Subnormals m 2^-149 (m < 2^23, leading one at bit k):
-// exponent k - 149 + 1023, the bits below the leading one as the fraction.
-// Infinity and NaN: exponent 2047, the fraction (a NaN's payload) kept.
-__device__ __forceinline__ double widen(double x) { return x; }
-__device__ __forceinline__ double widen(float f) {
-    const unsigned u = __float_as_uint(f);
-    const unsigned e = (u >> 23) & 0xffu;
-    unsigned m = u & 0x7fffffu, E;
-    if (e == 255u) {
-        E = 2047u;
-    } else if (e != 0u) {
-        E = e + 896u;
-    } else if (m != 0u) {
-        const unsigned k = 31u - (unsigned)__clz(m);   // bit of the leading one, 0..22
-        E = k + 874u;
-        m = (m << (23u - k)) & 0x7fffffu;
-    } else {
-        E = 0u;
-    }
-    const unsigned hi = (u & 0x80000000u) | (E << 20) | (m >> 3);
-    return __hiloint2double((int)hi, (int)(m << 29));
-}
-
 template <typename T>
 __device__ __forceinline__ void newmark2(double u, double v, T a0, T a1, const Consts& c, double& u2, double& v2) {
     const double sa = widen(fma_rn((T)3, a0, a1)), sb = widen(add_rn(a0, a1));
-    u2 = fma_rn(c.half_dt2, sa, fma_rn(c.dt + c.dt, v, u));
+    u2 = fma_rn(c.half_dt2, sa, fma_rn(c.dt2, v, u));
     v2 = fma_rn(c.dt, sb, v);
 }
 
@@ -364,12 +402,13 @@ struct PopDirect {
     struct Raw {
         T f[2][5];
     };
+    template <bool NC = true>
     __device__ __forceinline__ static void load_raw(const T* __restrict__ f, size_t plane, size_t p, bool ok,
                                                     Raw& r) {
 #pragma unroll
         for (int s = 0; s < 2; ++s)
 #pragma unroll
-            for (int q = 0; q < 5; ++q) r.f[s][q] = ok ? LBPS_LDG(f + (size_t)(s * 5 + q) * plane + p) : (T)0;
+            for (int q = 0; q < 5; ++q) r.f[s][q] = ok ? LBPS_LDX(NC, f + (size_t)(s * 5 + q) * plane + p) : (T)0;
     }
     __device__ __forceinline__ static void decode(const Raw& r, int s, const KC<T>&, T (&x)[5]) {
 #pragma unroll
@@ -405,12 +444,12 @@ struct PopDirect {
             for (int q = 0; q < 5; ++q) r.f[s][q] = x[s][q];
     }
     // Equilibria of Eq. feq of both sets at lattice offset p for s[set] and
-    // the lattice first moments (jx[set], jy[set]) (FP64 in), in stored form.
+    // the lattice first moments (jx[set], jy[set]), in stored form.
     // FP32 storage evaluates them in FP32 (from a and a_0 of the FP32
     // constants); FP64 storage in FP64.
-    __device__ __forceinline__ static void eq_raw(size_t, const Consts& c, const double (&sv)[2],
-                                                  const double (&jx)[2], const double (&jy)[2], const KC<T>& k,
-                                                  Raw& r) {
+    template <typename J>
+    __device__ __forceinline__ static void eq_raw(size_t, const Consts& c, const double (&sv)[2], const J (&jx)[2],
+                                                  const J (&jy)[2], const KC<T>& k, Raw& r) {
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             if constexpr (sizeof(T) == 4) {
@@ -560,15 +599,16 @@ struct PopNeq16 {
         asm("" : "+r"(x));
         return x + k.key4;
     }
+    template <bool NC = true>
     __device__ __forceinline__ static void load_raw(const float* __restrict__ f, size_t plane, size_t p, bool ok,
                                                     Raw& r) {
         const unsigned* w = words(f, plane);
 #pragma unroll
         for (int s = 0; s < 2; ++s)
 #pragma unroll
-            for (int q = 0; q < 3; ++q) r.m[s][q] = ok ? LBPS_LDG(f + (size_t)(s * 3 + q) * plane + p) : 0.0f;
+            for (int q = 0; q < 3; ++q) r.m[s][q] = ok ? LBPS_LDX(NC, f + (size_t)(s * 3 + q) * plane + p) : 0.0f;
 #pragma unroll
-        for (int q = 0; q < 2; ++q) r.w[q] = ok ? LBPS_LDG(w + (size_t)q * plane + p) : 0u;
+        for (int q = 0; q < 2; ++q) r.w[q] = ok ? LBPS_LDX(NC, w + (size_t)q * plane + p) : 0u;
     }
     __device__ __forceinline__ static void decode(const Raw& r, int s, const KC<float>& k, float (&x)[5]) {
         expand_pairs(r.m[s][0], r.m[s][1], r.m[s][2], half_of(r.w[0], s, k), half_of(r.w[1], s, k), k.r[s], x);
@@ -673,9 +713,9 @@ struct PopNeq16 {
     // Equilibria of Eq. feq of both sets at lattice offset p (the rounding key),
     // in FP32 and in stored form: J = (jx, jy) and the pair sums' deviation
     // 2 a s - 2 r f^0 from the stored f^0 (zero up to rounding), scaled.
-    __device__ __forceinline__ static void eq_raw(size_t p, const Consts&, const double (&sv)[2],
-                                                  const double (&jx)[2], const double (&jy)[2],
-                                                  const KC<float>& k, Raw& r) {
+    template <typename J>
+    __device__ __forceinline__ static void eq_raw(size_t p, const Consts&, const double (&sv)[2], const J (&jx)[2],
+                                                  const J (&jy)[2], const KC<float>& k, Raw& r) {
         unsigned w = 0;
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
@@ -777,15 +817,16 @@ struct PopBfp13 {
     __device__ __forceinline__ static unsigned enc_set(const float (&x)[5], float r, float scale) {
         return bfp13_encode(scaled_n(add_rn(x[1], x[3]), x[0], r, scale), scaled_n(add_rn(x[2], x[4]), x[0], r, scale));
     }
+    template <bool NC = true>
     __device__ __forceinline__ static void load_raw(const float* __restrict__ f, size_t plane, size_t p, bool ok,
                                                     Raw& r) {
         const unsigned* w = words(f, plane);
 #pragma unroll
         for (int s = 0; s < 2; ++s)
 #pragma unroll
-            for (int q = 0; q < 3; ++q) r.m[s][q] = ok ? LBPS_LDG(f + (size_t)(s * 3 + q) * plane + p) : 0.0f;
+            for (int q = 0; q < 3; ++q) r.m[s][q] = ok ? LBPS_LDX(NC, f + (size_t)(s * 3 + q) * plane + p) : 0.0f;
 #pragma unroll
-        for (int q = 0; q < 2; ++q) r.w[q] = ok ? LBPS_LDG(w + (size_t)q * plane + p) : 0u;
+        for (int q = 0; q < 2; ++q) r.w[q] = ok ? LBPS_LDX(NC, w + (size_t)q * plane + p) : 0u;
     }
     __device__ __forceinline__ static void decode(const Raw& r, int s, const KC<float>& k, float (&x)[5]) {
         float nx, ny;
@@ -905,9 +946,9 @@ struct PopBfp13 {
     }
     // Equilibria of Eq. feq of both sets, in FP32 and in stored form (as
     // PopNeq16::eq_raw; p unused, no rounding keys).
-    __device__ __forceinline__ static void eq_raw(size_t, const Consts&, const double (&sv)[2],
-                                                  const double (&jx)[2], const double (&jy)[2],
-                                                  const KC<float>& k, Raw& r) {
+    template <typename J>
+    __device__ __forceinline__ static void eq_raw(size_t, const Consts&, const double (&sv)[2], const J (&jx)[2],
+                                                  const J (&jy)[2], const KC<float>& k, Raw& r) {
 #pragma unroll
         for (int s = 0; s < 2; ++s) {
             const float sf = (float)sv[s];
