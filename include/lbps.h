@@ -39,8 +39,9 @@ extern "C" {
 #define LBPS_ERR_OOM (-2)       /* device allocation failed / block too small */
 #define LBPS_ERR_CUDA (-3)      /* a CUDA runtime call or launch failed       */
 #define LBPS_ERR_NONFINITE (-4) /* the state became non-finite (instability)  */
-#define LBPS_ERR_TIMEOUT (-5)   /* reserved: no kernel waits on the device, so
-                                   no call returns it                        */
+#define LBPS_ERR_TIMEOUT (-5)   /* a barrier inside a launch of many steps ran
+                                   out (the blocks were not all running); the
+                                   state is undefined until the next init    */
 #define LBPS_ERR_STATE (-6)     /* call out of order (e.g. step before init)  */
 
 /* Node types of the boundary mask (Sec. 2, Fig. 1). */
@@ -452,7 +453,11 @@ int lbps_check_report(uint64_t out[2]);
  * Defaults: variant 0 (variant 2 for FP64 storage, which needs more
  * registers, and 4 for BFP13, whose codec does); 32 rows, or 16 or 8 on lattices too small to give the
  * interior kernel 16384 warps at 32 (below about 4096^2); 16 rows from
- * 640000 to 2000000 points and 4 rows below 640000 (measured best). */
+ * 640000 to 2000000 points and 4 rows below 640000 (measured best).  A
+ * lattice whose launch shape was set takes its single steps as launches of
+ * that shape; otherwise lattices up to 1200000 points take many steps in one
+ * cooperative launch (the same bits; not while lbps_profile records or the
+ * stream is being captured). */
 int lbps_set_tuning(lbps_lattice* lat, int32_t variant, int32_t rows_per_warp);
 
 /* Steps per CUDA graph of lbps_step: k even, 2..64 (LBPS_ERR_INVALID
@@ -460,7 +465,7 @@ int lbps_set_tuning(lbps_lattice* lat, int32_t variant, int32_t rows_per_warp);
  * starting state copy and replays them; what is left of n (or a block a
  * synchronisation would split) runs as pairs from a 2-step graph or as
  * direct launches.  Results do not depend on it; a larger k saves launch
- * time on small lattices. */
+ * time.  Lattices that take many steps in one launch use no graphs. */
 int lbps_set_graph_steps(lbps_lattice* lat, int32_t k);
 
 /* Two time steps per sweep of the interior (on != 0) or one (0, the default).

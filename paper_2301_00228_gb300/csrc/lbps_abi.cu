@@ -574,6 +574,46 @@ int step_graph(lbps_lattice* lat, int k, cudaGraphExec_t* out, int* end_cur) {
     return LBPS_OK;
 }
 
+// Lattices up to this many points take their single steps many to a launch
+// (launch_fused); above it the phases of a step are long and the launches of a
+// replayed graph cost no more than the barriers.  Measured, us a step, one
+// launch against graphs of 32 steps: 64^2 FP64 10.9 / 15.7, 128 x 96 7.2 / 9.1,
+// 300^2 8.7 / 10.2 (BF16 11.5 / 13.3, BFP13 13.9 / 16.2), 389 x 1171 15.7 /
+// 18.1, 800^2 19.6 / 21.8, 1024^2 27.4 / 29.2 (BF16 33.7 / 33.6, with a hole
+// 41.8 / 45.7), 1536^2 71 / 59.
+constexpr int64_t kFusedMaxPoints = 1200000;
+// Steps per launch at most (tens of milliseconds at the largest size).
+constexpr int64_t kFusedMaxSteps = 1024;
+
+bool fused_ok(const lbps_lattice* lat) {
+    return !lat->fused_off && !lat->prof && !lat->tuned && !pair_ok(lat) &&
+           (int64_t)lat->L.g.nx * lat->L.g.ny <= kFusedMaxPoints;
+}
+
+// m steps in one launch (launch_fused); *done = false where the device
+// refuses the cooperative launch (the steps then run as separate launches).
+int run_fused(lbps_lattice* lat, int m, bool* done) {
+    const int a = lat->cur, b = a ^ 1;
+    cudaError_t e = lbps::with_policy(lat->p.storage, [&](auto pol) {
+        using P = decltype(pol);
+        return lbps::launch_fused<P>(lat->L.g, lat->c, lat->kc<P>(), lat->view<P>(a), lat->view<P>(b), lat->bn(),
+                                     lat->L.nb, lat->flag(), lat->tstep(), lat->bar(), m, lat->st);
+    });
+    *done = e == cudaSuccess;
+    if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+        cudaGetLastError();
+        lat->fused_off = true;
+        return LBPS_OK;
+    }
+    if (e != cudaSuccess) {
+        lat->last_cuda = (int)e;
+        return LBPS_ERR_CUDA;
+    }
+    lat->cur ^= m & 1;
+    lat->steps += m;
+    return LBPS_OK;
+}
+
 int run_sync(lbps_lattice* lat) {
     cudaError_t e = lbps::with_policy(lat->p.storage, [&](auto pol) {
         using P = decltype(pol);
@@ -657,8 +697,8 @@ int stage_u(lbps_lattice* lat, const double* ux0, const double* uy0, const doubl
 // (and the 16-bit scale choice before it).
 int init_staged(lbps_lattice* lat) {
     lat->cur ^= 1;
-    // the non-finite flag and the step counter beside it
-    if (cudaMemsetAsync(lat->flag(), 0, 16, lat->st) != cudaSuccess) return LBPS_ERR_CUDA;
+    // the non-finite flag and, beside it, the step counter and the barrier word
+    if (cudaMemsetAsync(lat->flag(), 0, kAlign, lat->st) != cudaSuccess) return LBPS_ERR_CUDA;
     if (lat->neq16()) {
         int rc = choose_scale(lat);
         if (rc != LBPS_OK) return rc;
@@ -1017,7 +1057,30 @@ int lbps_step_async(lbps_lattice* lat, int64_t n) {
         return lbps_batch_step(lat->solo, n);
     }
     const int l = lat->p.sync_every;
+    bool fused = fused_ok(lat);
+    if (fused) {
+        // a capturing stream gets the plain launches of single steps
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(lat->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+            cudaGetLastError();
+            fused = false;
+        }
+    }
     for (int64_t s = 0; s < n;) {
+        if (fused) {
+            int64_t m = std::min(n - s, kFusedMaxSteps);
+            if (l > 0) m = std::min<int64_t>(m, l - lat->steps % l);
+            const int rc = run_fused(lat, (int)m, &fused);
+            if (rc != LBPS_OK) return rc;
+            if (fused) {
+                s += m;
+                if (l > 0 && lat->steps % l == 0) {
+                    const int rs = run_sync(lat);
+                    if (rs != LBPS_OK) return rs;
+                }
+            }
+            continue;
+        }
         // graph_k steps at once from a graph, else 2, unless per-kernel timing
         // is on or a synchronisation falls after one of the first k - 1 of them
         int k = 0;
@@ -1062,6 +1125,7 @@ int lbps_check(lbps_lattice* lat) {
         lat->last_cuda = (int)e;
         return LBPS_ERR_CUDA;
     }
+    if (flag & lbps::kFlagTimeout) return LBPS_ERR_TIMEOUT;
     return flag ? LBPS_ERR_NONFINITE : LBPS_OK;
 }
 
@@ -1288,6 +1352,7 @@ int lbps_set_tuning(lbps_lattice* lat, int32_t variant, int32_t rows_per_warp) {
         return LBPS_ERR_INVALID;
     lat->tuning.variant = variant;
     lat->tuning.rows_per_warp = rows_per_warp;
+    lat->tuned = true;
     lat->gen += 1;  // captured step graphs use the old launch shape
     return LBPS_OK;
 }

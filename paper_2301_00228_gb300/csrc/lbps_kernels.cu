@@ -634,6 +634,7 @@ cudaError_t set_check_range(const void* base, size_t bytes, cudaStream_t st) {
     const int n = (int)ranges.size();
     cudaError_t e = cudaStreamSynchronize(st);  // no kernel in flight sees a half-written table
     if (e == cudaSuccess) e = upload_check_table(los.data(), his.data(), n);
+    if (e == cudaSuccess) e = fused_check_table(los.data(), his.data(), n);
     return e;
 #else
     (void)base;
@@ -646,7 +647,9 @@ cudaError_t set_check_range(const void* base, size_t bytes, cudaStream_t st) {
 int check_report(unsigned long long out[2]) {
 #ifdef LBPS_CHECKED
     if (cudaDeviceSynchronize() != cudaSuccess) return -1;
-    return read_check_report(out);
+    int rc = read_check_report(out);
+    if (rc > 0 && out[0] == 0) rc = fused_check_report(out);
+    return rc;
 #else
     out[0] = out[1] = 0;
     return 0;

@@ -82,6 +82,25 @@ template <typename P>
 cudaError_t launch_norms(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, int field, const double* ref,
                          double* partials, double* out4, cudaStream_t st);
 
+// ---- many steps in one launch (lbps_fused.cu)
+
+// Advances copy A (current) by `steps` time steps in one cooperative launch:
+// the odd steps write B, the even ones A.  Every step is the interior strips
+// and the boundary Newmark pass, a barrier over the grid, the boundary reset
+// and another barrier.  bar: the barrier's word (zero at creation).  A wait
+// that runs out sets kFlagTimeout in *flag.  Returns
+// cudaErrorCooperativeLaunchTooLarge (nothing launched) where the grid cannot
+// be resident at once.
+constexpr unsigned kFlagNonfinite = 1u, kFlagTimeout = 2u;
+template <typename P>
+cudaError_t launch_fused(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, View<P> B, const BNode* bn,
+                         int nb, unsigned* flag, unsigned long long* tstep, unsigned* bar, int steps,
+                         cudaStream_t st);
+#ifdef LBPS_CHECKED
+cudaError_t fused_check_table(const char* const* los, const char* const* his, int n);
+int fused_check_report(unsigned long long out[2]);
+#endif
+
 // ---- batches: many lattices advanced by one launch of each kernel per step
 
 // Everything the kernels need about one lattice of a batch.  v[cur] holds the

@@ -94,6 +94,8 @@ struct lbps_lattice {
     // batch of this one lattice (lbps_step_async)
     lbps_batch* solo = nullptr;
     lbps::Tuning tuning;  // bulk-kernel launch shape
+    bool tuned = false;   // set by the caller (lbps_set_tuning): the steps then run in that shape
+    bool fused_off = false;  // the device refused a cooperative launch
     int last_cuda = 0;    // cudaError_t of the last failing CUDA call
     int64_t steps;
     bool initialised;
@@ -130,6 +132,8 @@ struct lbps_lattice {
     unsigned* flag() const { return reinterpret_cast<unsigned*>(mem + L.off_flag); }
     // device step counter (time of the boundary data), beside the flag
     unsigned long long* tstep() const { return reinterpret_cast<unsigned long long*>(mem + L.off_flag + 8); }
+    // the grid barrier's word of launch_fused, in the same 256 bytes
+    unsigned* bar() const { return reinterpret_cast<unsigned*>(mem + L.off_flag + 128); }
     double* partials() const { return reinterpret_cast<double*>(mem + L.off_part); }
     double* out4() const { return reinterpret_cast<double*>(mem + L.off_out); }
     double* staging() const { return reinterpret_cast<double*>(mem + L.off_staging); }
