@@ -664,25 +664,34 @@ def bulk_roofline(prof, d, args, seconds, geometry, peak, peak_kind, wname):
             "boundary_newmark_pass": "beside the interior kernel on a second stream, not timed"}
 
 
+def sweep_steps(prof, steps):
+    """Steps per sweep of the timed window (4 for FP32 lattices of 3 M points
+    and more, else 2), from the number of sweep launches."""
+    return 4 if steps > 2.5 * max(float(prof[1]), 1.0) else 2
+
+
 def pair_roofline(prof, d, args, seconds, peak, peak_kind, wname):
-    """The two-step kernel: it reads the state of the points at least 3 from
-    every edge once and writes it once per launch, for two steps of updates
-    (events around every launch), with u, du/dt integrated over both steps
-    in one composed Newmark update."""
+    """The sweep kernel (K = 2 or 4 steps): it reads the state of the points
+    at least K + 1 from every edge once and writes it once per launch, for K
+    steps of updates (events around every launch), with u, du/dt integrated
+    over two steps at a time in one composed Newmark update."""
     pair_ms, pair_n = float(prof[0]), float(prof[1])
-    deep = (d.nx - 6) * (d.ny - 6)
+    K = sweep_steps(prof, args.steps)
+    deep = (d.nx - 2 * K - 2) * (d.ny - 2 * K - 2)
     alg_bytes = deep * BYTES_PER_UPDATE[args.storage]
     avg_s = pair_ms / max(pair_n, 1) / 1000.0
     achieved = alg_bytes / avg_s / 1e9
-    return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
-            "traffic": ncu_traffic(wname, args.storage, kernel="pair_kernel"), "kernel": "pair_kernel",
+    return {"bound": "hbm" if K == 2 else "fp64 pipe", "achieved": achieved, "peak": peak, "unit": "GB/s",
+            "frac": achieved / peak,
+            "traffic": ncu_traffic(wname, args.storage, kernel="sweep_kernel"), "kernel": "sweep_kernel",
             "peak_source": peak_kind, "alg_bytes_per_launch": alg_bytes, "avg_launch_ms": avg_s * 1000.0,
-            "steps_per_launch": 2, "updates_per_launch": 2 * deep,
-            "bytes_per_update": alg_bytes / (2 * deep),
-            "limiter": "latency at 20 warps/SM with the FP64 pipe about 2/3 busy (one composed Newmark update of u, du/dt per point per launch)",
+            "steps_per_launch": K, "updates_per_launch": K * deep,
+            "bytes_per_update": alg_bytes / (K * deep),
+            "limiter": "FP64 pipe (12 FP64 instructions per row of a warp for 4 steps, 64 cycles each)" if K == 4
+            else "issue slots of the storage codec, then HBM",
             "share_of_step_time": pair_ms / (1000.0 * seconds),
-            "kernel_timing": "CUDA events around every two-step launch of the timed steps",
-            "frame_and_boundary_passes": "beside the two-step kernel on a second stream of greatest priority, "
+            "kernel_timing": "CUDA events around every sweep launch of the timed steps",
+            "frame_and_boundary_passes": "beside the sweep on a second stream of greatest priority, "
                                           "not timed; they run on SM slots the kernel's retiring blocks free, so "
                                           "the kernel's launch time includes them"}
 
@@ -802,11 +811,11 @@ def run_gpu(args):
     peak, peak_kind = measured_peaks()
     if pairs:
         roofline = pair_roofline(prof, d, args, seconds, peak, peak_kind, wname)
-        # per pair of steps: the two-step kernel; beside it the boundary
-        # Newmark and reset of each step and two frame passes of four launches
-        # (BFP13 storage: one more launch per reset, its y streams)
+        # per sweep its kernel; beside it, per step, the boundary Newmark pass,
+        # the frame and the reset (BFP13 storage: one more launch per reset,
+        # its y streams); an odd last step is a single one (three launches)
         split = 1 if args.storage == "bfp13" else 0
-        gpu_launches = (args.steps // 2) * (13 + 2 * split) + (args.steps % 2) * (3 + split)
+        gpu_launches = int(prof[1]) + args.steps * (3 + split)
         single = single_step_window(lbps, lat, d, args, points, peak, stream)
     else:
         roofline = bulk_roofline(prof, d, args, seconds, geometry, peak, peak_kind, wname)
@@ -878,7 +887,7 @@ def run_gpu(args):
                            "replicas_per_gpu": 1, **({"tuning": args.tuning} if args.tuning else {})},
                 "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "gpu_launches": gpu_launches,
                 "clocks": clock}
-        line["config"]["steps_per_sweep"] = 2 if pairs else 1
+        line["config"]["steps_per_sweep"] = sweep_steps(prof, args.steps) if pairs else 1
         if single is not None:
             line["single_step"] = single
         if precision is not None:

@@ -480,16 +480,17 @@ int lbps_set_graph_steps(lbps_lattice* lat, int32_t k);
  * bits as single steps between synchronisations, u and du/dt the same up to
  * rounding.  Allocates the scratch copy (cudaMalloc, the
  * size of one state copy; LBPS_ERR_OOM if that fails) and frees it when
- * turned off or at lbps_destroy.  A synchronisation point that falls between
- * the two steps of a pair makes that pair two single steps.  With
- * lbps_profile on, the events of each pair bracket the two-step kernel only.
- * Below 12 x 2^20 points (and without per-kernel timing or synchronisation)
- * the pairs run as a batch of this one lattice (lbps_batch_set_step_pairs:
- * four launches a pair), from there on as the two-step kernel beside a chain
- * of boundary and frame launches on a second stream of greatest priority;
- * both give the same bits.  It pays from about 1700^2 points (FP32: 8192^2
- * 75.1 against 43.2 GLUPS; 4096^2 68.8 against 41.9; 2048^2 46.3 against
- * 37.1; 1536^2 32.5 against 33.6). */
+ * turned off or at lbps_destroy.  FP32 lattices of at least 3000000 points and
+ * 64 points a side advance the points at least 5 from the edges four steps per
+ * sweep (two of those updates), which takes a second scratch copy; without
+ * memory for it, or for the last 2 or 3 steps, they take two.  A
+ * synchronisation point that falls between the steps of a sweep makes it
+ * shorter sweeps or single steps.  With
+ * lbps_profile on, the events of each sweep bracket its kernel only.
+ * The sweep runs beside a chain
+ * of boundary and frame launches on a second stream of greatest priority.
+ * It pays from about 800^2 points (FP32, us a step against single steps:
+ * 8192^2 576 / 1563; 4096^2 159 / 400; 2047 x 1533 36 / 85). */
 int lbps_set_step_pairs(lbps_lattice* lat, int32_t on);
 
 /* 1 if lbps_step takes two steps per sweep on this lattice (turned on and

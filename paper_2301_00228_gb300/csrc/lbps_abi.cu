@@ -431,25 +431,6 @@ bool pair_ok(const lbps_lattice* lat) {
            lat->L.nb > 0;
 }
 
-// Below this many points a lattice takes its pairs of steps as a batch of
-// itself (lbps_batch_set_step_pairs): four launches a pair, the two-step
-// strips and the first step's frame strips in one persistent kernel, where
-// run_pair's concurrent chain on the second stream costs thirteen launches.
-// Measured (FP32 pulses, CUDA graphs, run_pair's second stream at the
-// greatest priority): 2048^2 46.3 against 37.9 GLUPS, 3072^2 56.8 against
-// 56.9; from 4096^2 run_pair is faster (68.8 against 63.0).
-constexpr int64_t kSoloPairsMaxPoints = 12ll << 20;
-
-bool solo_pairs(const lbps_lattice* lat) {
-    return pair_ok(lat) && !lat->prof && lat->p.sync_every == 0 &&
-           (int64_t)lat->L.g.nx * (int64_t)lat->L.g.ny < kSoloPairsMaxPoints;
-}
-
-void drop_solo(lbps_lattice* lat) {
-    if (lat->solo) lbps_batch_destroy(lat->solo);
-    lat->solo = nullptr;
-}
-
 // Steps n and n + 1 in one sweep of the interior.  Copy A (current) holds
 // step n, copy B receives step n + 2, the scratch copy X step n + 1 where the
 // boundary rules need it:
@@ -457,8 +438,8 @@ void drop_solo(lbps_lattice* lat) {
 //   from the edges, A -> X; reset(n) A, X -> X; Newmark(n + 1) X -> B; the
 //   interior kernel on the points 1..2 from the edges, X -> B; reset(n + 1)
 //   X, B -> B (the order of two single steps, on X and B);
-//   main stream, beside it: pair_kernel, A -> B, the points at least 3 from
-//   the edges.
+//   main stream, beside it: the sweep, A -> B, the points at least 3 from the
+//   edges.
 // The two streams write disjoint parts of X and B and read A, X, B only where
 // the other does not write, so they run concurrently; the join ends the pair.
 int run_pair(lbps_lattice* lat) {
@@ -473,7 +454,14 @@ int run_pair(lbps_lattice* lat) {
             // per-kernel timing: events around the two-step kernel (the passes
             // beside it are not timed, as the Newmark pass of a single step)
             cudaError_t r = prof_mark(lat);
-            if (r == cudaSuccess) r = lbps::launch_pair<P>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st, 32);
+            if (r == cudaSuccess) {
+                if constexpr (sizeof(typename P::V) == 8)
+                    r = lbps::launch_pair<P>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st, 32);
+                else
+                    r = lbps::launch_sweep<P, 2>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st);
+                if (r == cudaErrorNotSupported)   // a driver without tensor maps
+                    r = lbps::launch_pair<P>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st, 32);
+            }
             if (r == cudaSuccess) r = prof_mark(lat);
             if (r == cudaSuccess && lat->prof) lat->ev_kind.push_back(0);
             auto bnd = [&](lbps::View<P> s, lbps::View<P> d, int pass) {
@@ -499,11 +487,72 @@ int run_pair(lbps_lattice* lat) {
     return LBPS_OK;
 }
 
-// k steps: pairs in one sweep where they apply, else single steps
+// Four steps per sweep: FP32 storage (the others' codecs bind four steps: BFP13
+// 4096^2 263 us a step against 201 with two) from the size at which the binding
+// turns sweeps on by itself (2047 x 1533: 35.6 us a step against 54 with two).
+constexpr int64_t kQuadMinPoints = 3000000;
+constexpr int32_t kQuadMinSide = 64;
+
+bool quad_ok(const lbps_lattice* lat) { return lat->ymem && pair_ok(lat); }
+
+// Four steps, n .. n + 3, in one sweep of the interior, as run_pair: copy A
+// (current) holds step n, copy B receives step n + 4, and the scratch copies X
+// and Y hold steps n + 1, n + 3 and n + 2 where the boundary rules need them.
+// Step n + q + 1 is computed beside the sweep on the points 1 .. 7 - q from
+// the edges (each step reads one point further than it writes); the sweep
+// writes the points at least 5 from every edge.
+int run_quad(lbps_lattice* lat) {
+    const int a = lat->cur, b = lat->cur ^ 1;
+    cudaError_t e = cudaEventRecord(lat->fork, lat->st);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(lat->side, lat->fork, 0);
+    if (e == cudaSuccess)
+        e = lbps::with_policy(lat->p.storage, [&](auto pol) {
+            using P = decltype(pol);
+            const auto& g = lat->L.g;
+            const lbps::View<P> copy[4] = {lat->view<P>(a), lat->copy_view<P>(lat->xmem), lat->copy_view<P>(lat->ymem),
+                                           lat->view<P>(b)};
+            cudaError_t r = prof_mark(lat);
+            if constexpr (std::is_same<P, lbps::PolF32>::value) {
+                if (r == cudaSuccess)
+                    r = lbps::launch_sweep<P, 4>(g, lat->c, lat->kc<P>(), copy[0], copy[3], lat->flag(), lat->st);
+            } else {
+                r = cudaErrorNotSupported;   // other storages have no second scratch copy
+            }
+            if (r == cudaSuccess) r = prof_mark(lat);
+            if (r == cudaSuccess && lat->prof) lat->ev_kind.push_back(0);
+            const int order[5] = {0, 1, 2, 1, 3};   // A, X, Y, X, B
+            for (int q = 0; q < 4 && r == cudaSuccess; ++q) {
+                const lbps::View<P> &S = copy[order[q]], &D = copy[order[q + 1]];
+                auto bnd = [&](int pass) {
+                    return lbps::launch_boundary<P>(g, lat->c, lat->kc<P>(), S, D, lat->bn(), lat->L.nb, lat->flag(),
+                                                    lat->tstep(), lat->side, pass, pass + 1);
+                };
+                r = bnd(1);
+                if (r == cudaSuccess)
+                    r = lbps::launch_frame<P>(g, lat->c, lat->kc<P>(), S, D, lat->flag(), lat->side, 7 - q);
+                if (r == cudaSuccess) r = bnd(2);
+            }
+            return r;
+        });
+    if (e == cudaSuccess) e = cudaEventRecord(lat->join, lat->side);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(lat->st, lat->join, 0);
+    if (e != cudaSuccess) {
+        lat->last_cuda = (int)e;
+        return LBPS_ERR_CUDA;
+    }
+    lat->cur = b;
+    lat->steps += 4;
+    return LBPS_OK;
+}
+
+// k steps: four or two in one sweep where they apply, else single steps
 int run_steps(lbps_lattice* lat, int k) {
     int rc = LBPS_OK;
     for (int s = 0; s < k && rc == LBPS_OK;) {
-        if (k - s >= 2 && pair_ok(lat)) {
+        if (k - s >= 4 && quad_ok(lat)) {
+            rc = run_quad(lat);
+            s += 4;
+        } else if (k - s >= 2 && pair_ok(lat)) {
             rc = run_pair(lat);
             s += 2;
         } else {
@@ -1044,18 +1093,6 @@ int lbps_step_async(lbps_lattice* lat, int64_t n) {
     lbps::NvtxRange nvtx("lbps_step_async");
     if (!lat || n < 0) return LBPS_ERR_INVALID;
     if (!lat->initialised) return LBPS_ERR_STATE;
-    if (n >= 2 && solo_pairs(lat)) {
-        if (!lat->solo) {
-            lbps_lattice* one = lat;
-            int rc = lbps_batch_create(&one, 1, lat->st, &lat->solo);
-            if (rc == LBPS_OK) rc = lbps_batch_set_step_pairs(lat->solo, 1);
-            if (rc != LBPS_OK) {
-                drop_solo(lat);
-                return rc;
-            }
-        }
-        return lbps_batch_step(lat->solo, n);
-    }
     const int l = lat->p.sync_every;
     bool fused = fused_ok(lat);
     if (fused) {
@@ -1084,8 +1121,10 @@ int lbps_step_async(lbps_lattice* lat, int64_t n) {
         // graph_k steps at once from a graph, else 2, unless per-kernel timing
         // is on or a synchronisation falls after one of the first k - 1 of them
         int k = 0;
-        for (int c : {lat->graph_k, 2})
-            if (k == 0 && n - s >= c && !lat->prof && !(l > 0 && l - lat->steps % l < c)) k = c;
+        const bool quad = n - s >= 4 && quad_ok(lat) && !(l > 0 && l - lat->steps % l < 4);
+        for (int c : {lat->graph_k, quad ? 0 : 2}) {
+            if (k == 0 && c > 0 && n - s >= c && !lat->prof && !(l > 0 && l - lat->steps % l < c)) k = c;
+        }
         if (k > 0) {
             cudaGraphExec_t g = nullptr;
             int end_cur = lat->cur;
@@ -1099,6 +1138,10 @@ int lbps_step_async(lbps_lattice* lat, int64_t n) {
             lat->steps += k;
             lat->cur = end_cur;
             s += k;
+        } else if (quad) {
+            int rc = run_quad(lat);
+            if (rc != LBPS_OK) return rc;
+            s += 4;
         } else if (n - s >= 2 && pair_ok(lat) && !(l > 0 && (lat->steps + 1) % l == 0)) {
             int rc = run_pair(lat);
             if (rc != LBPS_OK) return rc;
@@ -1361,7 +1404,6 @@ int lbps_set_step_pairs(lbps_lattice* lat, int32_t on) {
     if (!lat || on < 0 || on > 1) return LBPS_ERR_INVALID;
     if ((on != 0) == (lat->xmem != nullptr)) return LBPS_OK;
     if (cudaStreamSynchronize(lat->st) != cudaSuccess) return LBPS_ERR_CUDA;
-    drop_solo(lat);
     if (on) {
         void* x = nullptr;
         if (cudaMalloc(&x, lat->L.copy_bytes) != cudaSuccess) {
@@ -1376,7 +1418,23 @@ int lbps_set_step_pairs(lbps_lattice* lat, int32_t on) {
             return LBPS_ERR_CUDA;
         }
         lat->xmem = static_cast<char*>(x);
+        // the second scratch copy of four steps per sweep; without it the
+        // lattice takes two
+        if (lat->p.storage == LBPS_STORAGE_F32 && (int64_t)lat->p.nx * lat->p.ny >= kQuadMinPoints &&
+            std::min(lat->p.nx, lat->p.ny) >= kQuadMinSide && cudaMalloc(&x, lat->L.copy_bytes) == cudaSuccess) {
+            if (cudaMemset(x, 0, lat->L.copy_bytes) == cudaSuccess &&
+                lbps::set_check_range(x, lat->L.copy_bytes, lat->st) == cudaSuccess)
+                lat->ymem = static_cast<char*>(x);
+            else
+                cudaFree(x);
+        }
+        cudaGetLastError();
     } else {
+        if (lat->ymem) {
+            lbps::set_check_range(lat->ymem, 0, lat->st);
+            cudaFree(lat->ymem);
+            lat->ymem = nullptr;
+        }
         lbps::set_check_range(lat->xmem, 0, lat->st);
         cudaFree(lat->xmem);
         lat->xmem = nullptr;
@@ -1522,7 +1580,6 @@ int lbps_set_stream(lbps_lattice* lat, void* cuda_stream) {
 
 void lbps_destroy(lbps_lattice* lat) {
     if (!lat) return;
-    drop_solo(lat);
     drop_graphs(lat);
     if (lat->cap) cudaStreamDestroy(lat->cap);
     if (lat->side) {
@@ -1532,6 +1589,11 @@ void lbps_destroy(lbps_lattice* lat) {
     if (lat->fork) cudaEventDestroy(lat->fork);
     if (lat->join) cudaEventDestroy(lat->join);
     if (lat->mem) lbps::set_check_range(lat->mem, 0, lat->st);  // checked builds: the block is no longer live
+    if (lat->ymem) {
+        lbps::set_check_range(lat->ymem, 0, lat->st);
+        cudaStreamSynchronize(lat->st);
+        cudaFree(lat->ymem);
+    }
     if (lat->xmem) {
         lbps::set_check_range(lat->xmem, 0, lat->st);
         cudaStreamSynchronize(lat->st);

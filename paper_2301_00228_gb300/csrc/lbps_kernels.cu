@@ -183,19 +183,26 @@ __global__ void __launch_bounds__(128, MINB) bulk_kernel(Geo g, Consts c, KCof<P
 
 // ------------------------------------------------- two steps per sweep
 
-// The interior kernel restricted to the window w: strips s0 .. s0 + nstrips - 1,
-// rows [jb, je) in chunks of `rows` (the frame passes of a two-step sweep).
+// The interior kernel on the points 1 .. fw from the edges only (the frame
+// passes of sweeps of several steps): the bottom, top, left and right band in
+// turn, each cut into blocks of kWarpsPerBlock strips and chunks of `rows`.
+// Everything but the strip is uniform over a block, so that it needs no
+// registers of the strip's.
+struct alignas(16) Bands {
+    Win w[4];
+    int s0[4], strips[4], blocks_x[4], first[4];   // first: its first block
+};
 template <typename P, int MINB, int UVD>
 __global__ void __launch_bounds__(128, MINB) frame_kernel(Geo g, Consts c, KCof<P> k, View<P> A, View<P> B,
-                                                          unsigned* flag, int s0, int nstrips, int jb, int je,
-                                                          int rows, Win w) {
-    const int warp = blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-    if (warp >= nstrips) return;  // whole warp
-    const int xs = (s0 + warp) * kStripCols;
-    const int j0 = jb + blockIdx.y * rows;
-    const int j1 = min(j0 + rows, je);
-    if (j0 >= j1) return;
-    const bool bad = bulk_strip<P, UVD, true>(g, c, k, A, B, xs, j0, j1, w);
+                                                          unsigned* flag, int rows, Bands bands) {
+    const int q = blockIdx.x;
+    const int band = (q >= bands.first[1]) + (q >= bands.first[2]) + (q >= bands.first[3]);
+    const int chunk = (q - bands.first[band]) / bands.blocks_x[band];
+    const int warp = (q - bands.first[band] - chunk * bands.blocks_x[band]) * kWarpsPerBlock + (threadIdx.x >> 5);
+    if (warp >= bands.strips[band]) return;  // whole warp
+    const int j0 = bands.w[band].y0 + chunk * rows;
+    const int j1 = min(j0 + rows, bands.w[band].y1);
+    const bool bad = bulk_strip<P, UVD, true>(g, c, k, A, B, (bands.s0[band] + warp) * kStripCols, j0, j1, bands.w[band]);
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, 1u);
 }
 
@@ -731,25 +738,23 @@ cudaError_t launch_frame(const Geo& g, const Consts& c, const KCof<P>& k, View<P
     // BFP13 fits 6 blocks with u prefetched one row ahead, not two
     constexpr int minb = sizeof(typename P::V) == 8 ? 4 : 6;
     constexpr int uvd = std::is_same<P, PopBfp13>::value ? 1 : 2;
-    auto kern = frame_kernel<P, minb, uvd>;
-    const int nx = g.nx, ny = g.ny, rows = 32;
-    const int all = (nx + kStripCols - 1) / kStripCols;
-    const dim3 blk(32 * kWarpsPerBlock);
-    auto blocks = [](int strips) { return (strips + kWarpsPerBlock - 1) / kWarpsPerBlock; };
-    // top and bottom bands: every strip, fw rows
-    kern<<<dim3(blocks(all), 1), blk, 0, st>>>(g, c, k, A, B, flag, 0, all, 1, 1 + fw, fw,
-                                                Win{1, nx - 1, 1, 1 + fw});
-    kern<<<dim3(blocks(all), 1), blk, 0, st>>>(g, c, k, A, B, flag, 0, all, ny - 1 - fw, ny - 1, fw,
-                                                Win{1, nx - 1, ny - 1 - fw, ny - 1});
-    // left and right bands between them: the strips holding columns 1 .. fw and
-    // nx - 1 - fw .. nx - 2
-    const int jb = 1 + fw, je = ny - 1 - fw, chunks = (je - jb + rows - 1) / rows;
-    const int ls0 = 1 / kStripCols, ls1 = fw / kStripCols;
-    const int rs0 = (nx - 1 - fw) / kStripCols, rs1 = (nx - 2) / kStripCols;
-    kern<<<dim3(blocks(ls1 - ls0 + 1), chunks), blk, 0, st>>>(g, c, k, A, B, flag, ls0, ls1 - ls0 + 1, jb, je, rows,
-                                                             Win{1, 1 + fw, jb, je});
-    kern<<<dim3(blocks(rs1 - rs0 + 1), chunks), blk, 0, st>>>(g, c, k, A, B, flag, rs0, rs1 - rs0 + 1, jb, je, rows,
-                                                             Win{nx - 1 - fw, nx - 1, jb, je});
+    // rows per chunk: short, since each launch waits for the one before and a
+    // warp's march is a chain of loads
+    constexpr int rows = 8;
+    const int nx = g.nx, ny = g.ny, all = (nx + kStripCols - 1) / kStripCols;
+    const int jb = 1 + fw, je = ny - 1 - fw, r0 = (nx - 1 - fw) / kStripCols;
+    Bands bands = {{Win{1, nx - 1, 1, 1 + fw}, Win{1, nx - 1, ny - 1 - fw, ny - 1}, Win{1, 1 + fw, jb, je},
+                    Win{nx - 1 - fw, nx - 1, jb, je}},
+                   {0, 0, 0, r0},
+                   {all, all, fw / kStripCols + 1, (nx - 2) / kStripCols - r0 + 1},
+                   {}, {}};
+    int blocks = 0;
+    for (int q = 0; q < 4; ++q) {
+        bands.first[q] = blocks;
+        bands.blocks_x[q] = (bands.strips[q] + kWarpsPerBlock - 1) / kWarpsPerBlock;
+        blocks += bands.blocks_x[q] * ((bands.w[q].y1 - bands.w[q].y0 + rows - 1) / rows);
+    }
+    frame_kernel<P, minb, uvd><<<blocks, 32 * kWarpsPerBlock, 0, st>>>(g, c, k, A, B, flag, rows, bands);
     return cudaGetLastError();
 }
 

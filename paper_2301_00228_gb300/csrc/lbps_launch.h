@@ -66,6 +66,11 @@ template <typename P>
 cudaError_t launch_frame(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, View<P> B, unsigned* flag,
                          cudaStream_t st, int fw);
 
+// K steps (2 or 4) of the points at least K + 1 from every edge, A -> B.
+template <typename P, int K>
+cudaError_t launch_sweep(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, View<P> B, unsigned* flag,
+                         cudaStream_t st);
+
 template <typename P>
 cudaError_t launch_sync(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, cudaStream_t st);
 

@@ -90,9 +90,8 @@ struct lbps_lattice {
     // holds step n + 1 on the boundary and the points up to 3 from it
     // (cudaMalloc'd, copy_bytes), null when off
     char* xmem = nullptr;
-    // pairs of steps of a lattice below lbps_solo_pairs_max points run as a
-    // batch of this one lattice (lbps_step_async)
-    lbps_batch* solo = nullptr;
+    // four steps per sweep (large lattices): a second scratch copy
+    char* ymem = nullptr;
     lbps::Tuning tuning;  // bulk-kernel launch shape
     bool tuned = false;   // set by the caller (lbps_set_tuning): the steps then run in that shape
     bool fused_off = false;  // the device refused a cooperative launch

@@ -382,8 +382,9 @@ struct Win {
 // (from i - 1), 2 f^3 (from i + 1), 4 f^2 (from j - 1), 8 f^4 (from j + 1).
 // A rectangle's boundary points are its non-periodic edges; a general
 // geometry marks them in its node-type plane.
+template <bool RECT>
 __device__ __forceinline__ int streamed_in(const Geo& g, int i, int j, size_t p) {
-    if (!g.general) {
+    if (RECT || !g.general) {
         int m = 0;
         if (!g.periodic_x) m |= (i == 1 ? 1 : 0) | (i == g.nx - 2 ? 2 : 0);
         if (!g.periodic_y) m |= (j == 1 ? 4 : 0) | (j == g.ny - 2 ? 8 : 0);
@@ -403,7 +404,8 @@ __device__ __forceinline__ int streamed_in(const Geo& g, int i, int j, size_t p)
 // Returns true in lanes that produced a non-finite value.  All 32 lanes of
 // the warp must call it together (warp shuffles).  UVD: how many rows ahead u
 // and du/dt are prefetched (1 or 2; the populations always 2).  WIN: writes
-// only points inside the window w (the frame passes of a two-step sweep).
+// only columns [w.x0, w.x1) of its rows, which lie inside the window (the
+// frame passes of sweeps of several steps).
 // NC = false: copy A may have been written earlier in the same launch (the
 // many-step kernel, which is bound by FP64 instructions and has registers to
 // spare: it widens the accelerations with integer operations).
@@ -467,7 +469,8 @@ __device__ __forceinline__ bool bulk_strip(const Geo& g, const Consts& c, const 
             Nm[s] = add_rn(add_rn(Nf[s][1], Nf[s][2]), add_rn(Nf[s][3], Nf[s][4]));
             Ns[s] = add_rn(Nf[s][0], Nm[s]);
         }
-        const bool row_interior = (g.periodic_y || (j > 0 && j < g.ny - 1)) && (!WIN || (j >= w.y0 && j < w.y1));
+        // (a window's rows are interior ones of the lattice: j0 .. j1 lie in it)
+        const bool row_interior = g.periodic_y || (j > 0 && j < g.ny - 1);
         if (row_interior) {  // warp-uniform
             V sW[2], sE[2], out[2][5];
 #pragma unroll
@@ -488,14 +491,14 @@ __device__ __forceinline__ bool bulk_strip(const Geo& g, const Consts& c, const 
             const size_t p = at(j);
             // general geometry: only interior points (boundary and void points
             // are the boundary passes' or stay zero)
-            if (out_lane && (!g.general || LBPS_LDG(&g.type[p]) == 0)) {
+            if (out_lane && (WIN || !g.general || LBPS_LDG(&g.type[p]) == 0)) {
                 double ax, ay;
                 accel_interior<V, !NC>(sW[0], sE[0], Ps[0], Ns[0], sW[1], sE[1], Ps[1], Ns[1], k, ax, ay);
                 double u1[4];
                 newmark(Cu[0], Cu[2], ax, c, u1[0], u1[2]);
                 newmark(Cu[1], Cu[3], ay, c, u1[1], u1[3]);
                 if constexpr (P::kSplitStream)
-                    P::store_point_pins(B.f, PL, p, out, k, streamed_in(g, col, j, p));
+                    P::store_point_pins(B.f, PL, p, out, k, streamed_in<WIN>(g, col, j, p));
                 else
                     P::store_point(B.f, PL, p, out, k);
 #pragma unroll

@@ -1,0 +1,359 @@
+// Several time steps of the deep interior of a rectangle in one sweep.
+//
+// A point at least K + 1 from every edge depends, K steps later, only on
+// interior points that the boundary reset of the steps between leaves alone
+// (the reset of a step changes the points at most 1 from an edge, and that
+// reaches one point further each step).  So a sweep that reads the state once
+// and writes it once advances those points by K steps; the boundary rules and
+// the points up to K from the edges run step by step beside it.
+//
+// Each warp marches down a strip of 32 columns, K pipeline stages deep: a row
+// enters as state n, each iteration moves every stage one row on, and the row
+// K - 1 above leaves as state n + K.  A stage keeps the row before (moment,
+// f^4) and its own row; x neighbours come by shuffles, so each step costs a
+// column on both sides (32 - 2 K columns come out).  Every step rounds to the
+// stored form, so the populations are the bits of single steps.  u, du/dt wait
+// in shared memory until their row leaves and then take two steps at a time
+// (newmark2).
+#include <cstring>
+
+#include <cuda.h>
+
+#include "lbps_steps.cuh"
+
+namespace lbps {
+
+namespace {
+
+// Polls of an mbarrier before a warp gives up (a second or more).
+constexpr int kMaxWaits = 1 << 22;
+
+__device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void mbar_init(unsigned long long* bar) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar)) : "memory");
+}
+
+__device__ __forceinline__ void mbar_expect(unsigned long long* bar, unsigned bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity) {
+    for (int n = 0; n < kMaxWaits; ++n) {
+        unsigned ok;
+        asm volatile(
+            "{\n.reg .pred p;\n"
+            "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+            "selp.u32 %0, 1, 0, p;\n}\n"
+            : "=r"(ok)
+            : "r"(smem_addr(bar)), "r"(parity)
+            : "memory");
+        if (ok) return true;
+    }
+    return false;
+}
+
+__device__ __forceinline__ void tma_load(void* dst, const CUtensorMap* map, int x, int y, unsigned long long* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+        "[%5];" ::"r"(smem_addr(dst)),
+        "l"(map), "r"(x), "r"(y), "r"(0), "r"(smem_addr(bar))
+        : "memory");
+}
+
+template <typename P>
+constexpr bool kHashed = false;
+template <typename H>
+constexpr bool kHashed<PopNeq16<H>> = true;
+
+// Ends a warp's reads of a slot before a copy into it is issued: orders every
+// lane's earlier shared-memory loads before later asynchronous copies (without
+// it ptxas may move a load whose value is needed late past the copy's issue),
+// then waits for every lane.
+__device__ __forceinline__ void release_slot() {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    __syncwarp();
+}
+
+// Shape of a sweep of K steps over 4-byte population planes.  A warp's lanes
+// are 32 columns, of which the inner OUT come out K steps later.  A slot of
+// the warp's ring holds two rows: the box of the populations ([plane][2][BOX]
+// words, from column xs - SKIP - K, a multiple of 4) and the box of u, du/dt
+// of the rows that leave the pipeline with them ([4][2][OUT] doubles).
+template <typename P, int K>
+struct Sweep {
+    static constexpr int OUT = 32 - 2 * K;
+    static constexpr int SKIP = (4 - K % 4) % 4;
+    static constexpr int BOX = (32 + SKIP + 3) / 4 * 4;
+    static constexpr int PLANES = P::kBytesPerPoint / 4;
+    static constexpr int F_BYTES = PLANES * 2 * BOX * 4;
+    static constexpr int U_OFF = (F_BYTES + 127) / 128 * 128;
+    static constexpr int U_BYTES = 4 * 2 * OUT * 8;
+    static constexpr int SLOT = U_OFF + (U_BYTES + 127) / 128 * 128;
+    static constexpr int DEPTH = K == 4 ? 4 : 2;   // slots; 16 or 9.5 KB a warp
+    // blocks per SM: FP16 and BF16 spill at 96 registers (8192^2 FP16: 743 us
+    // a step at 4 blocks, 830 at 5)
+    static constexpr int MINB = K == 4 ? 3 : kHashed<P> ? 4 : 5;
+    static constexpr int DEEP = K + 1;   // distance from the edges of the points a sweep writes
+    static constexpr size_t kSmem = (size_t)kWarpsPerBlock * DEPTH * SLOT;
+};
+
+// What a row keeps of its accelerations until its last step: the sums of each
+// pair of steps that newmark2 takes, or the first acceleration of a pair.
+template <typename V>
+struct Acc {
+    V a[2];        // the acceleration of a pair's first step
+    V sa[2], sb[2];  // 3 a0 + a1 and a0 + a1 of the pair before
+};
+
+template <typename P, int K>
+__device__ __forceinline__ bool sweep_strip(const Geo& g, const Consts& c, const KCof<P>& k,
+                                            const CUtensorMap* mf, const CUtensorMap* mu, const View<P>& B, char* ring,
+                                            unsigned long long* bars, int xs, int j0, int j1, bool& timeout) {
+    using V = typename P::V;
+    using S = Sweep<P, K>;
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int col = xs - K + lane;
+    const bool out_lane = lane >= K && lane < 32 - K && col >= S::DEEP && col < g.nx - S::DEEP;
+    const size_t PL = g.plane;
+    const int nq = j1 - j0 + 2 * K, ngroups = (nq + 1) / 2;   // rows read, and pairs of them
+    const int nit = nq - 2;
+
+    auto issue = [&](int q) {   // lane 0
+        char* slot = ring + (q % S::DEPTH) * S::SLOT;
+        unsigned long long* bar = bars + q % S::DEPTH;
+        // rows j0 - K + 2q, + 1 of the populations; the rows that leave while they enter
+        mbar_expect(bar, S::F_BYTES + (q >= K ? S::U_BYTES : 0));
+        tma_load(slot, mf, xs - K - S::SKIP, j0 - K + 2 * q, bar);
+        if (q >= K) tma_load(slot + S::U_OFF, mu, xs, j0 + 2 * (q - K), bar);
+    };
+    if (lane == 0) {
+        for (int q = 0; q < S::DEPTH; ++q) mbar_init(bars + q);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        for (int q = 0; q < S::DEPTH && q < ngroups; ++q) issue(q);
+    }
+    __syncwarp();
+
+    auto read_row = [&](const char* slot, int half, V (&f)[2][5]) {
+        const unsigned* w = reinterpret_cast<const unsigned*>(slot) + half * S::BOX + S::SKIP + lane;
+        unsigned words[S::PLANES];
+#pragma unroll
+        for (int q = 0; q < S::PLANES; ++q) words[q] = w[q * 2 * S::BOX];
+        typename P::Raw r;
+        static_assert(sizeof(r) == sizeof(words), "a point's words are its planes in order");
+        memcpy(&r, words, sizeof(r));
+        decode_row<P>(r, k, f);
+    };
+
+    // per stage: the row before (moment, f^4) and the row itself
+    V Ps[K][2] = {}, P4[K][2] = {}, Cf[K][2][5] = {}, Cm[K][2] = {};
+    Acc<V> hist[K] = {};
+    bool bad = false;
+
+    auto iterate = [&](const char* slot, int half, int it) {
+        V N[2][5];
+        read_row(slot, half, N);
+        Acc<V> from = {};   // of the row that enters this stage, from the stage before
+        V out[2][5];
+        V ax = 0, ay = 0;
+#pragma unroll
+        for (int s = 0; s < K; ++s) {
+            V Nm[2], Ns[2], Cs[2], sW[2], sE[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                Nm[q] = add_rn(add_rn(N[q][1], N[q][2]), add_rn(N[q][3], N[q][4]));
+                Ns[q] = add_rn(N[q][0], Nm[q]);
+                Cs[q] = add_rn(Cf[s][q][0], Cm[s][q]);
+                sW[q] = __shfl_up_sync(FULL, Cs[q], 1);
+                sE[q] = __shfl_down_sync(FULL, Cs[q], 1);
+                const V f3W = __shfl_up_sync(FULL, Cf[s][q][3], 1);
+                const V f1E = __shfl_down_sync(FULL, Cf[s][q][1], 1);
+                out[q][0] = add_rn(Cf[s][q][0], fma_rn(k.two_a0[q], Cm[s][q], -mul_rn(k.eight_a[q], Cf[s][q][0])));
+                out[q][1] = fma_rn(k.two_a[q], sW[q], -f3W);
+                out[q][3] = fma_rn(k.two_a[q], sE[q], -f1E);
+                out[q][2] = fma_rn(k.two_a[q], Ps[s][q], -P4[s][q]);
+                out[q][4] = fma_rn(k.two_a[q], Ns[q], -N[q][2]);
+            }
+            accel_interior_v<V>(sW[0], sE[0], Ps[s][0], Ns[0], sW[1], sE[1], Ps[s][1], Ns[1], k, ax, ay);
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                Ps[s][q] = Cs[q];
+                P4[s][q] = Cf[s][q][4];
+                Cm[s][q] = Nm[q];
+#pragma unroll
+                for (int d = 0; d < 5; ++d) Cf[s][q][d] = N[q][d];
+            }
+            if (s + 1 < K) {
+                const Acc<V> keep = hist[s];
+                hist[s] = from;
+                if (s & 1) {   // the second step of a pair: its sums
+                    hist[s].sa[0] = fma_rn((V)3, from.a[0], ax);
+                    hist[s].sa[1] = fma_rn((V)3, from.a[1], ay);
+                    hist[s].sb[0] = add_rn(from.a[0], ax);
+                    hist[s].sb[1] = add_rn(from.a[1], ay);
+                } else {
+                    hist[s].a[0] = ax;
+                    hist[s].a[1] = ay;
+                }
+                from = keep;
+                // as stored at this stage's row and read back
+                typename P::Raw raw;
+                P::pack((size_t)(j0 - K + 1 + it - s) * (size_t)g.px + (size_t)col, out, k, raw);
+                decode_row<P>(raw, k, N);
+            }
+        }
+        if (it >= 2 * K - 2 && out_lane) {   // the first test is uniform over the warp
+            const int e = it - (2 * K - 2);
+            const size_t p = (size_t)(j0 + e) * (size_t)g.px + (size_t)col;
+            const double* us = reinterpret_cast<const double*>(slot + S::U_OFF) + half * S::OUT + lane - K;
+            double u[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) u[q] = us[q * 2 * S::OUT];
+            if constexpr (K == 4) {
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const double sa = widen(from.sa[q]), sb = widen(from.sb[q]);
+                    u[q] = fma_rn(c.half_dt2, sa, fma_rn(c.dt2, u[2 + q], u[q]));
+                    u[2 + q] = fma_rn(c.dt, sb, u[2 + q]);
+                }
+            }
+            newmark2(u[0], u[2], from.a[0], ax, c, u[0], u[2]);
+            newmark2(u[1], u[3], from.a[1], ay, c, u[1], u[3]);
+            P::store_point(B.f, PL, p, out, k);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) LBPS_ST(&B.u[(size_t)q * PL + p], u[q]);
+            bad |= !isfinite(out[0][0] + out[1][0]);
+        }
+    };
+
+    // rows 0 and 1: the window of the first stage
+    if (!mbar_wait(bars, 0)) {
+        timeout = true;
+        return false;
+    }
+    {
+        V t[2][5];
+        read_row(ring, 0, t);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            Ps[0][q] = sum5(t[q][0], t[q][1], t[q][2], t[q][3], t[q][4]);
+            P4[0][q] = t[q][4];
+        }
+        read_row(ring, 1, Cf[0]);
+#pragma unroll
+        for (int q = 0; q < 2; ++q)
+            Cm[0][q] = add_rn(add_rn(Cf[0][q][1], Cf[0][q][2]), add_rn(Cf[0][q][3], Cf[0][q][4]));
+    }
+    release_slot();
+    if (lane == 0 && S::DEPTH < ngroups) issue(S::DEPTH);
+    int slot_i = 1;
+    unsigned parity = 0;
+    for (int q = 1; q < ngroups; ++q) {
+        char* slot = ring + slot_i * S::SLOT;
+        if (!mbar_wait(bars + slot_i, parity)) {
+            timeout = true;
+            return bad;
+        }
+        iterate(slot, 0, 2 * q - 2);
+        if (2 * q - 1 < nit) iterate(slot, 1, 2 * q - 1);
+        release_slot();
+        if (lane == 0 && q + S::DEPTH < ngroups) issue(q + S::DEPTH);
+        if (++slot_i == S::DEPTH) {
+            slot_i = 0;
+            parity ^= 1;
+        }
+    }
+    return bad;
+}
+
+// What bounds it: K = 4 in FP32, the FP64 pipe (12 instructions of 64 cycles a
+// row and warp; 79 % busy on 3072^2, issue 54 %, DRAM 53 %, 320 us for 4 steps);
+// K = 2 in the 16-bit formats, the issue slots their codec takes (BFP13 76 %,
+// FP64 49 %, DRAM 69 %, 220 us for 2 steps; K = 4 takes 556 us for 4).  The
+// rows come by TMA, two at a time and DEPTH pairs ahead, so no registers hold
+// rows in flight: the kernel this replaced loaded them through registers, one
+// row ahead, and waited on them (8192^2, two steps: FP32 1784 us, FP16 1632;
+// now FP32 two steps 1626, four steps 2304; FP16 1443).  Blocks per SM: what
+// the registers allow without spilling in earnest (K = 4 at 128 registers
+// spills 314 bytes and takes 3340 us).
+template <typename P, int K, int MINB>
+__global__ void __launch_bounds__(128, MINB) sweep_kernel(Geo g, Consts c, KCof<P> k,
+                                                          const __grid_constant__ CUtensorMap mf,
+                                                          const __grid_constant__ CUtensorMap mu, View<P> B,
+                                                          unsigned* flag, int rows) {
+    using S = Sweep<P, K>;
+    extern __shared__ __align__(128) char smem[];
+    __shared__ unsigned long long bars[kWarpsPerBlock * S::DEPTH];
+    const int wid = threadIdx.x >> 5;
+    const int xs = (blockIdx.x * kWarpsPerBlock + wid) * S::OUT;
+    const int j0 = S::DEEP + blockIdx.y * rows, j1 = min(j0 + rows, g.ny - S::DEEP);
+    if (xs >= g.nx - S::DEEP || j0 >= j1) return;   // whole warp
+    bool timeout = false;
+    const bool bad = sweep_strip<P, K>(g, c, k, &mf, &mu, B, smem + wid * (S::DEPTH * S::SLOT),
+                                       bars + wid * S::DEPTH, xs, j0, j1, timeout);
+    if (timeout) atomicOr(flag, kFlagTimeout);
+    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, kFlagNonfinite);
+}
+
+using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                              const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
+                              CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+cudaError_t encode(CUtensorMap* m, CUtensorMapDataType type, int elem, void* base, const Geo& g, int planes, int box_x) {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
+    if (e != cudaSuccess) return e;
+    if (found != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
+    const cuuint64_t dims[3] = {(cuuint64_t)g.px, (cuuint64_t)g.ny, (cuuint64_t)planes};
+    const cuuint64_t strides[2] = {(cuuint64_t)g.px * elem, (cuuint64_t)g.plane * elem};
+    const cuuint32_t box[3] = {(cuuint32_t)box_x, 2, (cuuint32_t)planes}, one[3] = {1, 1, 1};
+    const CUresult r = reinterpret_cast<EncodeFn>(fn)(m, type, 3, base, dims, strides, box, one,
+                                                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+                                                      CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                                                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+}  // namespace
+
+template <typename P, int K>
+cudaError_t launch_sweep(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, View<P> B, unsigned* flag,
+                         cudaStream_t st) {
+    using S = Sweep<P, K>;
+    CUtensorMap mf, mu;
+    cudaError_t e = encode(&mf, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, A.f, g, S::PLANES, S::BOX);
+    if (e == cudaSuccess) e = encode(&mu, CU_TENSOR_MAP_DATA_TYPE_UINT64, 8, A.u, g, 4, S::OUT);
+    if (e != cudaSuccess) return e;
+    auto kern = sweep_kernel<P, K, S::MINB>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
+    if (e != cudaSuccess) return e;
+    const int strips = (g.nx - S::DEEP + S::OUT - 1) / S::OUT;
+    const int height = g.ny - 2 * S::DEEP, blocks_x = (strips + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    // Rows per chunk.  Tall chunks recompute fewer rows around them; short ones
+    // end more often, so that the boundary launches beside the sweep find room
+    // on the SMs, and fill the last wave.  Measured, us a step: K = 4 FP32 2047
+    // x 1533 41.8 / 43.0 / 35.6 / 46.1 with 32 / 64 / 96 / 128 rows, 8192^2
+    // 601 / 578 / 576 / 578; K = 2 FP16 2047 x 1533 48.1 / 49.2 / 71.1 with 16 /
+    // 32 / 64 rows, 4096^2 204 / 201 / -, BFP13 4096^2 206 / 201 / 211.
+    const int rows = K == 4 ? 96 : (long long)g.nx * g.ny < (6ll << 20) ? 16 : 32;
+    const dim3 grid(blocks_x, (height + rows - 1) / rows);
+    kern<<<grid, 32 * kWarpsPerBlock, S::kSmem, st>>>(g, c, k, mf, mu, B, flag, rows);
+    return cudaGetLastError();
+}
+
+#define LBPS_INSTANTIATE(P)                                                                                       \
+    template cudaError_t launch_sweep<P, 2>(const Geo&, const Consts&, const KCof<P>&, View<P>, View<P>, unsigned*, \
+                                            cudaStream_t);
+
+LBPS_INSTANTIATE(PopDirect<float>)
+LBPS_INSTANTIATE(PopNeq16<__nv_bfloat16>)
+LBPS_INSTANTIATE(PopNeq16<__half>)
+LBPS_INSTANTIATE(PopBfp13)
+template cudaError_t launch_sweep<PopDirect<float>, 4>(const Geo&, const Consts&, const KC<float>&,
+                                                       View<PopDirect<float>>, View<PopDirect<float>>, unsigned*,
+                                                       cudaStream_t);
+
+}  // namespace lbps

@@ -1,0 +1,55 @@
+"""Four time steps per sweep (FP32 lattices of 3 M points and more) against
+single steps: the populations and step counts are the same bits, u and du/dt
+agree up to the rounding of the composed Newmark update (one FP32 rounding of
+the acceleration sums per pair of steps: 1e-7 of the field's largest magnitude
+over some tens of steps), on sides that leave every remainder of the 24-column
+strips and of the row chunks, at the smallest side, with step counts that leave
+0 to 3 steps over and synchronisation points that cut sweeps short."""
+import numpy as np
+import pytest
+
+from paper_2301_00228_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+FIELDS = ("ux", "uy", "vx", "vy", "f_phi", "f_psi")
+
+
+@pytest.fixture(scope="module")
+def L():
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    from paper_2301_00228_gb300 import lbps
+    return lbps
+
+
+def run(L, nx, ny, pairs, chunks, sync=0, load=False):
+    lat = L.Lattice.rectangle(nx, ny, 1.5, 1.0, (2, 1, 1, 2), np.linspace(-2e-4, 2e-4, 8), a0_phi=0.99,
+                              sync_every=sync, step_pairs=pairs)
+    if load:
+        lat.set_load(L.LBPS_NEUMANN, 20 * lat.dt, 45 * lat.dt)
+    y, x = (torch.arange(n, dtype=torch.float64, device="cuda") for n in (ny, nx))
+    u = [1e-3 * torch.sin(a * x)[None, :] * torch.cos(b * y)[:, None] for a, b in ((0.05, 0.03), (0.02, 0.07))]
+    v = [1e-2 * q.flip(0).contiguous() for q in u]
+    lat.init(*u, *v)
+    for n in chunks:
+        lat.step(n)
+    assert lat.check() == 0
+    out = {k: lat.read_device(k) for k in FIELDS}
+    steps = lat.steps
+    lat.close()
+    return out, steps
+
+
+@pytest.mark.parametrize("size", [(2003, 1501), (64, 46900), (46877, 65), (1733, 1741)])
+@pytest.mark.parametrize("chunks,sync", [((4, 7, 34, 1), 0), ((41,), 7)])
+def test_four_steps_per_sweep_equal_single_steps(L, size, chunks, sync):
+    want, n0 = run(L, *size, False, chunks, sync, load=True)
+    got, n1 = run(L, *size, True, chunks, sync, load=True)
+    assert n0 == n1 == sum(chunks)
+    for k in FIELDS:
+        if k.startswith("f_") and not sync:
+            assert torch.equal(got[k], want[k]), (size, k)
+        else:
+            err = float((got[k] - want[k]).abs().max()) / float(want[k].abs().max())
+            assert err <= 1e-7, (size, k, err)
