@@ -127,6 +127,50 @@ struct Boundary {
     std::vector<BNode> bn;
 };
 
+// Whether a point (wrapped along periodic axes) belongs to the body, and whether
+// a body point has a neighbour that does not.  Inlined: build_boundary asks
+// several times for every point of a general geometry.
+struct BodyMap {
+    const lbps_params* p;
+    const uint8_t* node_type;
+    __forceinline__ bool operator()(int i, int j) const {
+        const int nx = p->nx, ny = p->ny;
+        if (i < 0 || i >= nx) {
+            if (!p->periodic_x) return false;
+            i = (i + nx) % nx;
+        }
+        if (j < 0 || j >= ny) {
+            if (!p->periodic_y) return false;
+            j = (j + ny) % ny;
+        }
+        return !node_type || node_type[(size_t)j * nx + i] != LBPS_VOID;
+    }
+    __forceinline__ bool boundary(int i, int j) const {
+        return (*this)(i, j) &&
+               !((*this)(i + 1, j) && (*this)(i, j + 1) && (*this)(i - 1, j) && (*this)(i, j - 1));
+    }
+};
+
+// Difference stencils of the boundary points and their body neighbours
+// (BNode::kinds).
+void set_kinds(const lbps_params* p, const uint8_t* node_type, std::vector<BNode>& bn) {
+    const int nx = p->nx, ny = p->ny;
+    const int DX[4] = {1, 0, -1, 0}, DY[4] = {0, 1, 0, -1};
+    const BodyMap body{p, node_type};
+    auto kind = [&](int i, int j, int dx, int dy) {
+        const bool hp = body(i + dx, j + dy), hm = body(i - dx, j - dy);
+        return (int)(hp && hm ? lbps::DIFF_CENTRAL : hp ? lbps::DIFF_FORWARD : lbps::DIFF_BACKWARD);
+    };
+    for (BNode& q : bn) {
+        q.kinds = kind(q.i, q.j, 1, 0) | kind(q.i, q.j, 0, 1) << 2;
+        for (int d = 0; d < 4; ++d) {
+            if (!body(q.i + DX[d], q.j + DY[d])) continue;
+            const int i = (q.i + DX[d] + nx) % nx, j = (q.j + DY[d] + ny) % ny;
+            q.kinds |= (kind(i, j, 1, 0) | kind(i, j, 0, 1) << 2) << (4 + 4 * d);
+        }
+    }
+}
+
 // Rectangle (no void points, no cells): the outer ring in perimeter order,
 // cells by reading R6 (computed in the kernel from the indices).  General
 // geometry (reading R14): every body point with a neighbour outside the body,
@@ -147,38 +191,8 @@ int build_boundary(const lbps_params* p, const uint8_t* node_type, const double*
     const int DX[4] = {1, 0, -1, 0};
     const int DY[4] = {0, 1, 0, -1};
     auto type_at = [&](int i, int j) { return node_type ? node_type[(size_t)j * nx + i] : (uint8_t)LBPS_INTERIOR; };
-    auto body = [&](int i, int j) {
-        if (i < 0 || i >= nx) {
-            if (!p->periodic_x) return false;
-            i = (i + nx) % nx;
-        }
-        if (j < 0 || j >= ny) {
-            if (!p->periodic_y) return false;
-            j = (j + ny) % ny;
-        }
-        return type_at(i, j) != 3;
-    };
-    auto boundary = [&](int i, int j) {
-        if (!body(i, j)) return false;
-        for (int d = 0; d < 4; ++d)
-            if (!body(i + DX[d], j + DY[d])) return true;
-        return false;
-    };
-    // difference stencils of point (i, j) (already in the lattice): x in bits 0, 1, y in bits 2, 3
-    auto kinds_at = [&](int i, int j) {
-        auto kind = [&](int dx, int dy) {
-            const bool hp = body(i + dx, j + dy), hm = body(i - dx, j - dy);
-            return hp && hm ? lbps::DIFF_CENTRAL : hp ? lbps::DIFF_FORWARD : lbps::DIFF_BACKWARD;
-        };
-        return (int)kind(1, 0) | (int)kind(0, 1) << 2;
-    };
-    // ... and of its body neighbours E, N, W, S, 4 bits each above them (BNode::kinds)
-    auto kinds_of = [&](int i, int j) {
-        int k = kinds_at(i, j);
-        for (int d = 0; d < 4; ++d)
-            if (body(i + DX[d], j + DY[d])) k |= kinds_at((i + DX[d] + nx) % nx, (j + DY[d] + ny) % ny) << (4 + 4 * d);
-        return k;
-    };
+    const BodyMap body{p, node_type};
+    auto boundary = [&](int i, int j) { return body.boundary(i, j); };
     auto bvalue = [&](size_t k, double& bx, double& by) {
         bx = bc_value ? bc_value[2 * k] : 0.0;
         by = bc_value ? bc_value[2 * k + 1] : 0.0;
@@ -218,7 +232,6 @@ int build_boundary(const lbps_params* p, const uint8_t* node_type, const double*
                 node.smask = smask;
                 node.bx = bx;
                 node.by = by;
-                node.kinds = kinds_of(i, j);
                 out.bn[q] = node;
             }
         }
@@ -231,6 +244,13 @@ int build_boundary(const lbps_params* p, const uint8_t* node_type, const double*
             size_t k = (size_t)j * nx + i;
             int t = type_at(i, j);
             if (t == 3) continue;
+            // the points that have all four neighbours inside the lattice and the
+            // body: interior ones, central differences
+            if (node_type && !pairs16 && i > 0 && i < nx - 1 && j > 0 && j < ny - 1 && node_type[k - 1] != 3 &&
+                node_type[k + 1] != 3 && node_type[k - nx] != 3 && node_type[k + nx] != 3) {
+                if (t != LBPS_INTERIOR) return LBPS_ERR_INVALID;
+                continue;
+            }
             for (int ax = 0; ax < 2; ++ax) {  // a difference stencil along x and y
                 int dx = ax == 0, dy = ax == 1;
                 bool hp = body(i + dx, j + dy), hm = body(i - dx, j - dy);
@@ -278,7 +298,6 @@ int build_boundary(const lbps_params* p, const uint8_t* node_type, const double*
                 }
                 node.inv_m = 1.0 / (p->rho * vol);
             }
-            node.kinds = kinds_of(i, j);
             out.bn.push_back(node);
         }
     }
@@ -907,6 +926,7 @@ int lbps_create_cells(const lbps_params* params, const uint8_t* node_type, const
     Boundary bd;
     rc = build_boundary(params, node_type, bc_value, cell, bd);
     if (rc != LBPS_OK) return rc;
+    if (bd.general) set_kinds(params, node_type, bd.bn);   // a rectangle's follow from the indices
     Layout L = make_layout(params, bd.general, (int)bd.bn.size());
     const std::vector<BNode>& bn = bd.bn;
     lbps_lattice* lat = new (std::nothrow) lbps_lattice();

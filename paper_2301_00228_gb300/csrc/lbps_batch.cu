@@ -41,7 +41,9 @@ struct lbps_batch {
     // two steps per sweep (lbps_batch_set_step_pairs): the task lists of the
     // two stages of a pair, stage 1 then stage 2, in their own device block
     bool pairs = false;
-    char* pmem = nullptr;
+    char* pmem = nullptr;         // tensor maps (with tma) | tasks
+    size_t off_ptask = 0;
+    bool tma = false;             // stage 1 takes its strips by TMA (not FP64 storage)
     int np1 = 0, np2 = 0;
 };
 
@@ -129,8 +131,8 @@ size_t max_bulk_tasks(const lbps_batch* b) {
 
 // The tasks of one stage of a pair of steps (two steps per sweep), as
 // run_pair runs them on a single lattice: stage 1 the two-step strips
-// (pair_kernel's 28 columns by 32 rows over the points at least 3 from every
-// edge) and the frame strips on the points 1..3 from the edges; stage 2 the
+// (28 columns by 32 rows over the points at least 3 from every
+// edge, the columns counted from 0 where the strips come by TMA) and the frame strips on the points 1..3 from the edges; stage 2 the
 // frame strips on the points 1..2 from the edges (frame_kernel's bands);
 // both with the Newmark pass of every boundary point spread evenly among them.
 std::vector<PairTask> pair_stage_tasks(const lbps_batch* b, int stage) {
@@ -144,7 +146,7 @@ std::vector<PairTask> pair_stage_tasks(const lbps_batch* b, int stage) {
         nbnd += b->lats[d]->L.nb;
         if (stage == 1)
             for (int j0 = kDeep; j0 < ny - kDeep; j0 += kRows)
-                for (int xs = kDeep; xs < nx - kDeep; xs += kPairCols)
+                for (int xs = b->tma ? 0 : kDeep; xs < nx - kDeep; xs += kPairCols)
                     work.push_back(PairTask{d, lbps::kPairStrip, xs, j0, std::min(j0 + kRows, ny - kDeep), 0, 0, 0, 0});
         const int all = (nx + kCols - 1) / kCols;
         for (int q = 0; q < all; ++q) {   // top and bottom bands, fw rows each
@@ -153,12 +155,10 @@ std::vector<PairTask> pair_stage_tasks(const lbps_batch* b, int stage) {
                                     ny - 1});
         }
         const int jb = 1 + fw, je = ny - 1 - fw;   // left and right bands between them
-        for (int j0 = jb; j0 < je; j0 += kRows) {
-            const int j1 = std::min(j0 + kRows, je);
-            for (int q = 1 / kCols; q <= fw / kCols; ++q)
-                work.push_back(PairTask{d, lbps::kFrameStrip, q * kCols, j0, j1, 1, 1 + fw, jb, je});
-            for (int q = (nx - 1 - fw) / kCols; q <= (nx - 2) / kCols; ++q)
-                work.push_back(PairTask{d, lbps::kFrameStrip, q * kCols, j0, j1, nx - 1 - fw, nx - 1, jb, je});
+        for (int j0 = jb; j0 < je; j0 += lbps::kSideTaskRows) {
+            const int j1 = std::min(j0 + lbps::kSideTaskRows, je);
+            work.push_back(PairTask{d, lbps::kSideStrip, 0, j0, j1, 1, 1 + fw, 0, 0});
+            work.push_back(PairTask{d, lbps::kSideStrip, nx - 8, j0, j1, nx - 1 - fw, nx - 1, 0, 0});
         }
     }
     const size_t nn = (size_t)(nbnd + 31) / 32;
@@ -235,14 +235,23 @@ cudaError_t launch_step(lbps_batch* b, int parity) {
 // the reset of the second (x, v[a ^ 1] -> v[a ^ 1]).
 cudaError_t launch_pair_step(lbps_batch* b, int parity) {
     const BndTask* bt = reinterpret_cast<const BndTask*>(b->mem + b->off_bnd);
-    const PairTask* p1 = reinterpret_cast<const PairTask*>(b->pmem);
+    const PairTask* p1 = reinterpret_cast<const PairTask*>(b->pmem + b->off_ptask);
     const PairTask* p2 = p1 + b->np1;
     return lbps::with_policy(b->storage, [&](auto pol) {
         using P = decltype(pol);
         const DomDesc<P>* dd = reinterpret_cast<const DomDesc<P>*>(b->mem);
         unsigned* next = reinterpret_cast<unsigned*>(b->mem + b->off_next) + 1;   // the two stages' counters
         cudaError_t e = cudaMemsetAsync(next, 0, 2 * sizeof(unsigned), b->st);
-        if (e == cudaSuccess) e = lbps::launch_pair_batch<P>(dd, p1, b->np1, bt, parity, 1, next, b->st);
+        if (e == cudaSuccess) {
+            bool done = false;
+            if constexpr (sizeof(typename P::V) == 4)
+                if (b->tma) {
+                    e = lbps::launch_sweep_batch<P>(dd, reinterpret_cast<const lbps::SweepMaps*>(b->pmem), p1, b->np1,
+                                                    bt, parity, next, b->st);
+                    done = true;
+                }
+            if (!done) e = lbps::launch_pair_batch<P>(dd, p1, b->np1, bt, parity, 1, next, b->st);
+        }
         if (e == cudaSuccess) e = lbps::launch_boundary_batch<P>(dd, bt, b->nbnd, parity, 2, 3, b->st, 1);
         if (e == cudaSuccess) e = lbps::launch_pair_batch<P>(dd, p2, b->np2, bt, parity, 2, next + 1, b->st);
         if (e == cudaSuccess) e = lbps::launch_boundary_batch<P>(dd, bt, b->nbnd, parity, 2, 3, b->st, 2);
@@ -427,6 +436,8 @@ int lbps_batch_check(lbps_batch* b) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
     if (e != cudaSuccess) return fail(b, e);
     for (unsigned f : flags)
+        if (f & lbps::kFlagTimeout) return LBPS_ERR_TIMEOUT;
+    for (unsigned f : flags)
         if (f) return LBPS_ERR_NONFINITE;
     return LBPS_OK;
 }
@@ -457,15 +468,36 @@ int lbps_batch_set_step_pairs(lbps_batch* b, int32_t on) {
         const int rc = lbps_set_step_pairs(l, 1);
         if (rc != LBPS_OK) return rc;
     }
+    // the tensor maps of every lattice's copies; without them (FP64 storage, a
+    // driver that has none) the strips load through registers
+    std::vector<lbps::SweepMaps> maps(b->lats.size());
+    b->tma = lbps::with_policy(b->storage, [&](auto pol) {
+        using P = decltype(pol);
+        if constexpr (sizeof(typename P::V) == 8) {
+            return false;
+        } else {
+            for (size_t d = 0; d < b->lats.size(); ++d) {
+                const lbps_lattice* l = b->lats[d];
+                if (lbps::make_sweep_maps<P>(l->L.g, l->view<P>(0), l->view<P>(1), &maps[d]) != cudaSuccess) return false;
+            }
+            return true;
+        }
+    });
+    cudaGetLastError();
+    b->off_ptask = b->tma ? maps.size() * sizeof(lbps::SweepMaps) : 0;
     const std::vector<PairTask> t1 = pair_stage_tasks(b, 1), t2 = pair_stage_tasks(b, 2);
-    if (cudaMalloc(&b->pmem, (t1.size() + t2.size()) * sizeof(PairTask)) != cudaSuccess) {
+    if (cudaMalloc(&b->pmem, b->off_ptask + (t1.size() + t2.size()) * sizeof(PairTask)) != cudaSuccess) {
         cudaGetLastError();
         b->pmem = nullptr;
         return LBPS_ERR_OOM;
     }
-    cudaError_t e = cudaMemcpyAsync(b->pmem, t1.data(), t1.size() * sizeof(PairTask), cudaMemcpyHostToDevice, b->st);
+    cudaError_t e = cudaSuccess;
+    if (b->tma) e = cudaMemcpyAsync(b->pmem, maps.data(), b->off_ptask, cudaMemcpyHostToDevice, b->st);
+    char* tasks = b->pmem + b->off_ptask;
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(b->pmem + t1.size() * sizeof(PairTask), t2.data(), t2.size() * sizeof(PairTask),
+        e = cudaMemcpyAsync(tasks, t1.data(), t1.size() * sizeof(PairTask), cudaMemcpyHostToDevice, b->st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(tasks + t1.size() * sizeof(PairTask), t2.data(), t2.size() * sizeof(PairTask),
                             cudaMemcpyHostToDevice, b->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
     if (e != cudaSuccess) return fail(b, e);

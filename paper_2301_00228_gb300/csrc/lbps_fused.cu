@@ -58,7 +58,9 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned& phase, uns
     return *alive != 0;
 }
 
-template <typename P, int THREADS, int UVD>
+// GEN: general geometry (a template so that the code of rectangles does not
+// carry it).
+template <typename P, int THREADS, int UVD, bool GEN>
 __global__ void __launch_bounds__(THREADS, 1) fused_kernel(Geo g, Consts c, KCof<P> k, View<P> A0, View<P> B0,
                                                            const BNode* __restrict__ bn, int nb, unsigned* flag,
                                                            unsigned long long* tstep, unsigned* bar, int steps,
@@ -102,8 +104,8 @@ __global__ void __launch_bounds__(THREADS, 1) fused_kernel(Geo g, Consts c, KCof
                 const int q = s0 + t - nbp, strip = q / chunks;
                 const int j0 = (q - strip * chunks) * rows, j1 = min(j0 + rows, g.ny);
                 // rows of a hole: nothing to write, nothing an interior point reads
-                if (g.gap && j0 >= LBPS_LD(&g.gap[2 * strip]) && j1 <= LBPS_LD(&g.gap[2 * strip + 1])) continue;
-                bad |= bulk_strip<P, UVD, false, false>(g, c, k, A, B, strip * kStripCols, j0, j1);
+                if (GEN && g.gap && j0 >= LBPS_LD(&g.gap[2 * strip]) && j1 <= LBPS_LD(&g.gap[2 * strip + 1])) continue;
+                bad |= bulk_strip<P, UVD, false, false, GEN>(g, c, k, A, B, strip * kStripCols, j0, j1);
             }
         }
         if (nb > 0) {
@@ -114,7 +116,7 @@ __global__ void __launch_bounds__(THREADS, 1) fused_kernel(Geo g, Consts c, KCof
                 if (t & 1)
                     neighbour_stresses(g, c, B.u, B.u + g.plane, table, nb, B.s, b);
                 else
-                    bad |= boundary_reset(g, c, k, A, B, table, b);
+                    bad |= boundary_reset<P>(g, c, k, A, B, table, nb, b);
             }
             if (P::kSplitStream) {
                 if (!grid_barrier(bar, phase, flag, &alive)) return;
@@ -161,9 +163,12 @@ cudaError_t launch_fused(const Geo& g, const Consts& c, const KCof<P>& k, View<P
     int blocks = (int)std::min<long long>(sms, std::max<long long>(nst, 2 * nbt));
     const int warps = (int)std::min<long long>(
         warps_max, (nst + blocks - 1) / blocks + 2 * ((nbt + blocks - 1) / blocks));
-    const void* kern = reinterpret_cast<const void*>(fused_kernel<P, 512, 1>);
+    const void* kern = reinterpret_cast<const void*>(g.general ? fused_kernel<P, 512, 1, true>
+                                                               : fused_kernel<P, 512, 1, false>);
     if constexpr (!wide)
-        if (threads_max == 640) kern = reinterpret_cast<const void*>(fused_kernel<P, 640, 1>);
+        if (threads_max == 640)
+            kern = reinterpret_cast<const void*>(g.general ? fused_kernel<P, 640, 1, true>
+                                                           : fused_kernel<P, 640, 1, false>);
     Geo ga = g;
     Consts ca = c;
     KCof<P> ka = k;

@@ -136,9 +136,15 @@ __global__ void __launch_bounds__(128, 6) boundary_reset_kernel(Geo g, Consts c,
                                                              const BNode* __restrict__ bn, int nb, unsigned* flag,
                                                              unsigned long long* tstep) {
     int b = blockIdx.x * blockDim.x + threadIdx.x;
-    if (b < nb && blockIdx.y + 1 == gridDim.y) neighbour_stresses(g, c, B.u, B.u + g.plane, bn, nb, B.s, b);
-    if (blockIdx.y != 0) return;
-    if (b < nb && boundary_reset(g, c, k, A, B, bn, b)) atomicOr(flag, 1u);
+    if (blockIdx.y == 1) {
+        if (b < nb) neighbour_stresses(g, c, B.u, B.u + g.plane, bn, nb, B.s, b);
+        return;
+    }
+    bool bad = false;
+    if (b < nb)
+        bad = gridDim.y == 2 ? boundary_reset<P>(g, c, k, A, B, bn, nb, b)
+                             : boundary_reset<P, true>(g, c, k, A, B, bn, nb, b);
+    if (bad) atomicOr(flag, 1u);
     if (b == 0) LBPS_ST(tstep, LBPS_LD(tstep) + 1ull);
 }
 
@@ -184,26 +190,40 @@ __global__ void __launch_bounds__(128, MINB) bulk_kernel(Geo g, Consts c, KCof<P
 // ------------------------------------------------- two steps per sweep
 
 // The interior kernel on the points 1 .. fw from the edges only (the frame
-// passes of sweeps of several steps): the bottom, top, left and right band in
-// turn, each cut into blocks of kWarpsPerBlock strips and chunks of `rows`.
-// Everything but the strip is uniform over a block, so that it needs no
-// registers of the strip's.
-struct alignas(16) Bands {
-    Win w[4];
-    int s0[4], strips[4], blocks_x[4], first[4];   // first: its first block
-};
+// passes of sweeps of several steps).  Blocks 0 .. bands - 1: the bottom and the
+// top band, strips of rows; then the left and right bands between them, a side
+// strip a warp, groups of W lanes (W >= fw + 2).
+template <typename P, int UVD, int W>
+__device__ __forceinline__ void frame(const Geo& g, const Consts& c, const KCof<P>& k, const View<P>& A,
+                                      const View<P>& B, unsigned* flag, int fw, int bands) {
+    bool bad;
+    const int wid = threadIdx.x >> 5;
+    if (blockIdx.x < (unsigned)bands) {
+        const int per = bands / 2, top = blockIdx.x >= (unsigned)per;
+        const int xs = ((blockIdx.x - top * per) * kWarpsPerBlock + wid) * kStripCols;
+        if (xs >= g.nx) return;  // whole warp
+        const int j0 = top ? g.ny - 1 - fw : 1;
+        bad = bulk_strip<P, UVD, true>(g, c, k, A, B, xs, j0, j0 + fw, Win{1, g.nx - 1, j0, j0 + fw});
+    } else {
+        const int t = (blockIdx.x - bands) * kWarpsPerBlock + wid;
+        const int j0 = 1 + fw + (t >> 1) * (32 / W * kSideRows), je = g.ny - 1 - fw;
+        if (j0 >= je) return;  // whole warp
+        const bool right = t & 1;
+        bad = side_strip<P, W>(g, c, k, A, B, right ? g.nx - W : 0, right ? g.nx - 1 - fw : 1, right ? g.nx - 1 : 1 + fw,
+                               j0, je, kSideRows);
+    }
+    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, 1u);
+}
+
 template <typename P, int MINB, int UVD>
 __global__ void __launch_bounds__(128, MINB) frame_kernel(Geo g, Consts c, KCof<P> k, View<P> A, View<P> B,
-                                                          unsigned* flag, int rows, Bands bands) {
-    const int q = blockIdx.x;
-    const int band = (q >= bands.first[1]) + (q >= bands.first[2]) + (q >= bands.first[3]);
-    const int chunk = (q - bands.first[band]) / bands.blocks_x[band];
-    const int warp = (q - bands.first[band] - chunk * bands.blocks_x[band]) * kWarpsPerBlock + (threadIdx.x >> 5);
-    if (warp >= bands.strips[band]) return;  // whole warp
-    const int j0 = bands.w[band].y0 + chunk * rows;
-    const int j1 = min(j0 + rows, bands.w[band].y1);
-    const bool bad = bulk_strip<P, UVD, true>(g, c, k, A, B, (bands.s0[band] + warp) * kStripCols, j0, j1, bands.w[band]);
-    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, 1u);
+                                                          unsigned* flag, int fw, int bands) {
+    frame<P, UVD, 8>(g, c, k, A, B, flag, fw, bands);
+}
+template <typename P, int MINB, int UVD>
+__global__ void __launch_bounds__(128, MINB) frame_wide_kernel(Geo g, Consts c, KCof<P> k, View<P> A, View<P> B,
+                                                               unsigned* flag, int fw, int bands) {
+    frame<P, UVD, 16>(g, c, k, A, B, flag, fw, bands);
 }
 
 template <typename P, int MINB>
@@ -242,9 +262,13 @@ __global__ void __launch_bounds__(128) boundary_batch_kernel(const DomDesc<P>* _
     else if (pass == 3)
         boundary_stream_y(d.g, d.c, d.k, S, D, d.bn, tk.b);
     else {
-        if (blockIdx.y + 1 == gridDim.y) neighbour_stresses(d.g, d.c, D.u, D.u + d.g.plane, d.bn, d.nb, D.s, tk.b);
-        if (blockIdx.y != 0) return;
-        if (boundary_reset(d.g, d.c, d.k, S, D, d.bn, tk.b)) atomicOr(d.flag, 1u);
+        if (blockIdx.y == 1) {
+            neighbour_stresses(d.g, d.c, D.u, D.u + d.g.plane, d.bn, d.nb, D.s, tk.b);
+            return;
+        }
+        const bool bad = gridDim.y == 2 ? boundary_reset<P>(d.g, d.c, d.k, S, D, d.bn, d.nb, tk.b)
+                                        : boundary_reset<P, true>(d.g, d.c, d.k, S, D, d.bn, d.nb, tk.b);
+        if (bad) atomicOr(d.flag, 1u);
         if (tk.b == 0) LBPS_ST(d.tstep, LBPS_LD(d.tstep) + 1ull);
     }
 }
@@ -300,8 +324,9 @@ __global__ void __launch_bounds__(128, MINB) bulk_batch_kernel(const DomDesc<P>*
     }
 }
 
-// Two steps per sweep for every lattice of a batch: one stage of a pair (see
-// launch_pair_batch).  The tasks are those of pair_kernel, frame_kernel and
+// Two steps per sweep for every lattice of a batch: stage 1 of a pair (see
+// launch_pair_batch) with the strips' rows loaded through registers (FP64
+// storage; the others take them by TMA, lbps_sweep.cu).  The tasks are those of pair_kernel, frame_kernel and
 // boundary_newmark_kernel on each lattice, so each lattice gets the same bits
 // as run on its own with two steps per sweep.  Frame strips take the shape
 // that loads u one row ahead (the results do not depend on it).
@@ -309,7 +334,7 @@ template <typename P, int MINB>
 __global__ void __launch_bounds__(128, MINB) pair_batch_kernel(const DomDesc<P>* __restrict__ dd,
                                                                const PairTask* __restrict__ tasks, int ntasks,
                                                                const BndTask* __restrict__ btasks, int parity,
-                                                               int stage, unsigned* next) {
+                                                               unsigned* next) {
     __shared__ DomDesc<P> sd[kWarpsPerBlock];
     const unsigned FULL = 0xffffffffu;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -325,11 +350,9 @@ __global__ void __launch_bounds__(128, MINB) pair_batch_kernel(const DomDesc<P>*
                 const BndTask bt = btasks[tk.xs + lane];
                 const DomDesc<P>& d = dd[bt.dom];
                 const int a = d.cur ^ parity;
-                const View<P>& S = stage == 2 ? d.x : d.v[a];
-                const View<P>& D = stage == 1 ? d.x : d.v[a ^ 1];
                 const double n = (double)LBPS_LD(d.tstep);
-                boundary_newmark(d.g, d.c, S, D, d.bn, d.nb, S.s, n, bt.b, 0);
-                boundary_newmark(d.g, d.c, S, D, d.bn, d.nb, S.s, n, bt.b, 1);
+                boundary_newmark(d.g, d.c, d.v[a], d.x, d.bn, d.nb, d.v[a].s, n, bt.b, 0);
+                boundary_newmark(d.g, d.c, d.v[a], d.x, d.bn, d.nb, d.v[a].s, n, bt.b, 1);
             }
             continue;
         }
@@ -346,13 +369,50 @@ __global__ void __launch_bounds__(128, MINB) pair_batch_kernel(const DomDesc<P>*
         bool bad;
         if (tk.kind == kPairStrip) {
             bad = pair_strip<P>(d.g, d.c, d.k, d.v[a], d.v[a ^ 1], tk.xs, tk.j0, tk.j1);
+        } else if (tk.kind == kSideStrip) {
+            bad = side_strip<P, 8>(d.g, d.c, d.k, d.v[a], d.x, tk.xs, tk.x0, tk.x1, tk.j0, tk.j1, kSideRows);
         } else {
-            const View<P>& S = stage == 2 ? d.x : d.v[a];
-            const View<P>& D = stage == 1 ? d.x : d.v[a ^ 1];
-            bad = bulk_strip<P, 1, true>(d.g, d.c, d.k, S, D, tk.xs, tk.j0, tk.j1, Win{tk.x0, tk.x1, tk.y0, tk.y1});
+            bad = bulk_strip<P, 1, true>(d.g, d.c, d.k, d.v[a], d.x, tk.xs, tk.j0, tk.j1, Win{tk.x0, tk.x1, tk.y0, tk.y1});
         }
         if (__any_sync(FULL, bad) && lane == 0) atomicOr(d.flag, 1u);
     }
+}
+
+// Stage 2 of a pair, one task a warp: the frame strips and Newmark tasks only,
+// so 5 blocks fit on an SM.  Every task is a chain of scattered loads; what
+// counts is how many run at once (256 lattices: as a persistent grid of the
+// stage-1 kernel's 4 blocks per SM 156 us).
+template <typename P>
+__global__ void __launch_bounds__(128, sizeof(typename P::V) == 8 ? 3 : 5)
+    edge_batch_kernel(const DomDesc<P>* __restrict__ dd, const PairTask* __restrict__ tasks, int ntasks,
+                      const BndTask* __restrict__ btasks, int parity) {
+    __shared__ DomDesc<P> sd[kWarpsPerBlock];
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int t = blockIdx.x * kWarpsPerBlock + wid;
+    if (t >= ntasks) return;  // whole warp
+    const PairTask tk = tasks[t];
+    if (tk.kind == kNewmarkTask) {
+        if (lane < tk.j1) {
+            const BndTask bt = btasks[tk.xs + lane];
+            const DomDesc<P>& d = dd[bt.dom];
+            const View<P>& D = d.v[d.cur ^ parity ^ 1];
+            const double n = (double)LBPS_LD(d.tstep);
+            boundary_newmark(d.g, d.c, d.x, D, d.bn, d.nb, d.x.s, n, bt.b, 0);
+            boundary_newmark(d.g, d.c, d.x, D, d.bn, d.nb, d.x.s, n, bt.b, 1);
+        }
+        return;
+    }
+    const unsigned* src = reinterpret_cast<const unsigned*>(dd + tk.dom);
+    unsigned* dst = reinterpret_cast<unsigned*>(sd + wid);
+    for (int q = lane; q < (int)(sizeof(DomDesc<P>) / 4); q += 32) dst[q] = src[q];
+    __syncwarp();
+    const DomDesc<P>& d = sd[wid];
+    const View<P>& D = d.v[d.cur ^ parity ^ 1];
+    const bool bad = tk.kind == kSideStrip
+                         ? side_strip<P, 8>(d.g, d.c, d.k, d.x, D, tk.xs, tk.x0, tk.x1, tk.j0, tk.j1, kSideRows)
+                         : bulk_strip<P, 1, true>(d.g, d.c, d.k, d.x, D, tk.xs, tk.j0, tk.j1,
+                                                  Win{tk.x0, tk.x1, tk.y0, tk.y1});
+    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(d.flag, 1u);
 }
 
 // ------------------------------------------------------------------ sync
@@ -588,12 +648,17 @@ template <typename P>
 cudaError_t launch_pair_batch(const DomDesc<P>* dd, const PairTask* tasks, int ntasks, const BndTask* btasks,
                               int parity, int stage, unsigned* next, cudaStream_t st) {
     if (ntasks <= 0) return cudaGetLastError();
+    if (stage == 2) {
+        edge_batch_kernel<P><<<(ntasks + kWarpsPerBlock - 1) / kWarpsPerBlock, 32 * kWarpsPerBlock, 0, st>>>(
+            dd, tasks, ntasks, btasks, parity);
+        return cudaGetLastError();
+    }
     // 4 blocks per SM (at 5 the two kinds of strips together spill)
     auto kern = pair_batch_kernel<P, sizeof(typename P::V) == 8 ? 2 : 4>;
     int blocks = resident_blocks(kern);
     if (blocks < 0) return cudaGetLastError();
     blocks = min(blocks, (ntasks + kWarpsPerBlock - 1) / kWarpsPerBlock);
-    kern<<<blocks, 32 * kWarpsPerBlock, 0, st>>>(dd, tasks, ntasks, btasks, parity, stage, next);
+    kern<<<blocks, 32 * kWarpsPerBlock, 0, st>>>(dd, tasks, ntasks, btasks, parity, next);
     return cudaGetLastError();
 }
 
@@ -738,23 +803,17 @@ cudaError_t launch_frame(const Geo& g, const Consts& c, const KCof<P>& k, View<P
     // BFP13 fits 6 blocks with u prefetched one row ahead, not two
     constexpr int minb = sizeof(typename P::V) == 8 ? 4 : 6;
     constexpr int uvd = std::is_same<P, PopBfp13>::value ? 1 : 2;
-    // rows per chunk: short, since each launch waits for the one before and a
-    // warp's march is a chain of loads
-    constexpr int rows = 8;
-    const int nx = g.nx, ny = g.ny, all = (nx + kStripCols - 1) / kStripCols;
-    const int jb = 1 + fw, je = ny - 1 - fw, r0 = (nx - 1 - fw) / kStripCols;
-    Bands bands = {{Win{1, nx - 1, 1, 1 + fw}, Win{1, nx - 1, ny - 1 - fw, ny - 1}, Win{1, 1 + fw, jb, je},
-                    Win{nx - 1 - fw, nx - 1, jb, je}},
-                   {0, 0, 0, r0},
-                   {all, all, fw / kStripCols + 1, (nx - 2) / kStripCols - r0 + 1},
-                   {}, {}};
-    int blocks = 0;
-    for (int q = 0; q < 4; ++q) {
-        bands.first[q] = blocks;
-        bands.blocks_x[q] = (bands.strips[q] + kWarpsPerBlock - 1) / kWarpsPerBlock;
-        blocks += bands.blocks_x[q] * ((bands.w[q].y1 - bands.w[q].y0 + rows - 1) / rows);
-    }
-    frame_kernel<P, minb, uvd><<<blocks, 32 * kWarpsPerBlock, 0, st>>>(g, c, k, A, B, flag, rows, bands);
+    const int strips = (g.nx + kStripCols - 1) / kStripCols;
+    const int bands = 2 * ((strips + kWarpsPerBlock - 1) / kWarpsPerBlock);
+    auto run = [&](auto kern, int W) {
+        const int task = 32 / W * kSideRows, sides = 2 * ((g.ny - 2 - 2 * fw + task - 1) / task);
+        kern<<<bands + (sides + kWarpsPerBlock - 1) / kWarpsPerBlock, 32 * kWarpsPerBlock, 0, st>>>(g, c, k, A, B, flag,
+                                                                                                   fw, bands);
+    };
+    if (fw + 2 <= 8)
+        run(frame_kernel<P, minb, uvd>, 8);
+    else
+        run(frame_wide_kernel<P, minb, uvd>, 16);
     return cudaGetLastError();
 }
 

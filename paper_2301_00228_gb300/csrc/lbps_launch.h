@@ -137,10 +137,13 @@ struct BndTask {   // one thread: boundary point b of lattice dom
 // output columns [xs, xs + 28) of rows [j0, j1) of lattice dom advanced two
 // steps; kFrameStrip, the interior kernel on strip xs, rows [j0, j1), writing
 // only inside the window [x0, x1) x [y0, y1); kNewmarkTask, the Newmark pass
-// of boundary tasks [xs, xs + j1).
+// of boundary tasks [xs, xs + j1); kSideStrip, the interior kernel on columns
+// [x0, x1), rows [j0, j1), kSideTaskRows at most, its lanes from column xs on.
 constexpr int kPairStrip = 0;
 constexpr int kFrameStrip = 1;
 constexpr int kNewmarkTask = 2;
+constexpr int kSideStrip = 3;
+constexpr int kSideTaskRows = 32;
 struct PairTask {
     int dom, kind, xs, j0, j1;
     int x0, x1, y0, y1;
@@ -161,6 +164,17 @@ cudaError_t launch_boundary_batch(const DomDesc<P>* dd, const BndTask* tasks, in
 template <typename P>
 cudaError_t launch_pair_batch(const DomDesc<P>* dd, const PairTask* tasks, int ntasks, const BndTask* btasks,
                               int parity, int stage, unsigned* next, cudaStream_t st);
+// Stage 1 with the two-step strips fed by TMA (FP32 and 16-bit storages; their
+// strips start at columns that are multiples of 28).  maps: per lattice the
+// tensor maps of the populations and u of its two copies, in device memory.
+struct alignas(64) SweepMaps {
+    unsigned char map[4][128];
+};
+template <typename P>
+cudaError_t make_sweep_maps(const Geo& g, View<P> v0, View<P> v1, SweepMaps* out);
+template <typename P>
+cudaError_t launch_sweep_batch(const DomDesc<P>* dd, const SweepMaps* maps, const PairTask* tasks, int ntasks,
+                               const BndTask* btasks, int parity, unsigned* next, cudaStream_t st);
 // Interior of every lattice and the Newmark pass of their boundary points: a
 // persistent grid whose warps take tasks (strips, or 32 boundary points of
 // btasks) through the counter *next (device memory; the launcher zeroes it on

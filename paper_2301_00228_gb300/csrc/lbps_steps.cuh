@@ -21,6 +21,39 @@ namespace {
 // moments stay in the populations' type (FP32 - FP32 rounded through FP64 is
 // the FP32 difference).
 
+// Where boundary point b lies, its difference stencils (BNode::kinds) and the
+// interior neighbours it streams into (BNode::smask).  A rectangle's follow
+// from its place in the perimeter list: computed, so that the loads of u do
+// not wait for the table's (an interior neighbour's stencils are central).
+struct BPoint {
+    int i, j, kinds, smask;
+};
+__device__ __forceinline__ BPoint point_of(const Geo& g, const BNode* __restrict__ bn, int b) {
+    BPoint p;
+    if (g.general) {
+        p.i = LBPS_LD(&bn[b].i);
+        p.j = LBPS_LD(&bn[b].j);
+        p.kinds = LBPS_LD(&bn[b].kinds);
+        p.smask = LBPS_LD(&bn[b].smask);
+        return p;
+    }
+    const int rows = g.periodic_y ? 0 : 2 * g.nx;   // the inverse of perim_index
+    if (b < rows) {
+        p.i = b < g.nx ? b : b - g.nx;
+        p.j = b < g.nx ? 0 : g.ny - 1;
+    } else {
+        const int jlo = g.periodic_y ? 0 : 1, len = g.ny - 2 * jlo, q = b - rows;
+        p.i = q < len ? 0 : g.nx - 1;
+        p.j = jlo + (q < len ? q : q - len);
+    }
+    const bool l = !g.periodic_x && p.i == 0, r = !g.periodic_x && p.i == g.nx - 1;
+    const bool d = !g.periodic_y && p.j == 0, u = !g.periodic_y && p.j == g.ny - 1;
+    p.kinds = (l ? DIFF_FORWARD : r ? DIFF_BACKWARD : DIFF_CENTRAL) |
+              (d ? DIFF_FORWARD : u ? DIFF_BACKWARD : DIFF_CENTRAL) << 2;
+    p.smask = (l || r) && (d || u) ? 0 : l ? 1 : r ? 4 : d ? 2 : 8;   // none at corners
+    return p;
+}
+
 // Unscaled difference of p along an axis: stencil `kind` at index i of n
 // points `stride` elements apart.
 __device__ __forceinline__ double diff3(const double* p, int kind, int i, int n, ptrdiff_t stride) {
@@ -148,14 +181,15 @@ __device__ __forceinline__ void store_point_stress(const Geo& g, double* __restr
 // boundary points: the interior neighbour of a rectangle's edge point (slot
 // nb + b), the body neighbours of a general boundary point (slot 5b + 1 + d).
 __device__ __forceinline__ void neighbour_stresses(const Geo& g, const Consts& c, const double* ux, const double* uy,
-                                          const BNode* __restrict__ bn, int nb, double* __restrict__ sig, int b) {
-    const int i = LBPS_LD(&bn[b].i), j = LBPS_LD(&bn[b].j), kinds = LBPS_LD(&bn[b].kinds);
-    const int mask = g.general ? LBPS_LD(&bn[b].nbmask) : LBPS_LD(&bn[b].smask);
+                                                   const BNode* __restrict__ bn, int nb, double* __restrict__ sig,
+                                                   int b) {
+    const BPoint pt = point_of(g, bn, b);
+    const int mask = g.general ? LBPS_LD(&bn[b].nbmask) : pt.smask;
     for (int d = 0; d < 4; ++d) {   // E, N, W, S
         if (!((mask >> d) & 1)) continue;
-        const int ni = wrap(i + (d == 0) - (d == 2), g.nx), nj = wrap(j + (d == 1) - (d == 3), g.ny);
+        const int ni = wrap(pt.i + (d == 0) - (d == 2), g.nx), nj = wrap(pt.j + (d == 1) - (d == 3), g.ny);
         double s[3];
-        stress_of(c, grad_at(g, c, ux, uy, ni, nj, (kinds >> (4 + 4 * d)) & 3, (kinds >> (6 + 4 * d)) & 3), s);
+        stress_of(c, grad_at(g, c, ux, uy, ni, nj, (pt.kinds >> (4 + 4 * d)) & 3, (pt.kinds >> (6 + 4 * d)) & 3), s);
         const size_t o = g.general ? (size_t)b * 15 + 3 * (1 + d) : ((size_t)nb + b) * 3;
 #pragma unroll
         for (int q = 0; q < 3; ++q) LBPS_ST(&sig[o + q], s[q]);
@@ -164,9 +198,9 @@ __device__ __forceinline__ void neighbour_stresses(const Geo& g, const Consts& c
 
 __device__ __forceinline__ void boundary_stress(const Geo& g, const Consts& c, const double* ux, const double* uy,
                                        const BNode* __restrict__ bn, int nb, double* __restrict__ sig, int b) {
-    const int kinds = LBPS_LD(&bn[b].kinds);
+    const BPoint pt = point_of(g, bn, b);
     double s[3];
-    stress_of(c, grad_at(g, c, ux, uy, LBPS_LD(&bn[b].i), LBPS_LD(&bn[b].j), kinds & 3, (kinds >> 2) & 3), s);
+    stress_of(c, grad_at(g, c, ux, uy, pt.i, pt.j, pt.kinds & 3, (pt.kinds >> 2) & 3), s);
     store_point_stress(g, sig, b, s);
     neighbour_stresses(g, c, ux, uy, bn, nb, sig, b);
 }
@@ -177,7 +211,8 @@ template <int Q, typename P>
 __device__ __forceinline__ void boundary_newmark_q(const Geo& g, const Consts& c, const View<P>& A, const View<P>& B,
                                                    const BNode* __restrict__ bn, int nb,
                                                    const double* __restrict__ sig, double n, int b) {
-    const int i = LBPS_LD(&bn[b].i), j = LBPS_LD(&bn[b].j);
+    const BPoint pt = point_of(g, bn, b);
+    const int i = pt.i, j = pt.j;
     const bool fixed = LBPS_LD(&bn[b].type) == DIRICHLET;
     const size_t p = (size_t)j * g.px + i;
     const double u = LBPS_LD(&A.u[Q * g.plane + p]), v = LBPS_LD(&A.u[(2 + Q) * g.plane + p]);
@@ -270,23 +305,35 @@ __device__ __forceinline__ void stream_out(const Geo& g, const Consts& c, const 
     }
 }
 
-// The reset of point b itself (the stresses at its neighbours are
-// neighbour_stresses').
-template <typename P>
+// The reset of point b itself; with NEIGHBOURS also the stresses at its
+// neighbours (otherwise a part of its own, neighbour_stresses).
+template <typename P, bool NEIGHBOURS = false>
 __device__ __forceinline__ bool boundary_reset(const Geo& g, const Consts& c, const KCof<P>& k, const View<P>& A,
-                                      const View<P>& B, const BNode* __restrict__ bn, int b) {
+                                               const View<P>& B, const BNode* __restrict__ bn, int nb, int b) {
     using V = typename P::V;
-    const int i = LBPS_LD(&bn[b].i), j = LBPS_LD(&bn[b].j);
+    const BPoint pt = point_of(g, bn, b);
+    const int i = pt.i, j = pt.j, smask = pt.smask;
     const size_t p = (size_t)j * g.px + i;
     // The populations at t (copy A's boundary mirror, entry b, coalesced
-    // along the boundary list) and the streaming mask, loaded first: nothing
-    // below writes them, and issued here their latency overlaps the
-    // differences and the stress stores instead of following them.
-    const int smask = LBPS_LD(&bn[b].smask), kinds = LBPS_LD(&bn[b].kinds);
+    // along the boundary list) and every difference are loaded before the
+    // first store: no load may pass a store, and together their latencies
+    // overlap.
     typename P::Raw ra, rb;
     P::template load_raw<false>(A.m, g.mplane, (size_t)b, true, ra);
     // Eq. psi_phi_at_bound: differences of u(t + dt) at (i, j).
-    const Grad d = grad_at(g, c, B.u, B.u + g.plane, i, j, kinds & 3, (kinds >> 2) & 3);
+    const Grad d = grad_at(g, c, B.u, B.u + g.plane, i, j, pt.kinds & 3, (pt.kinds >> 2) & 3);
+    if (NEIGHBOURS) {
+        if (g.general) {
+            neighbour_stresses(g, c, B.u, B.u + g.plane, bn, nb, B.s, b);
+        } else if (smask) {   // the one interior neighbour of an edge point
+            const Grad e = grad_at(g, c, B.u, B.u + g.plane, i + (smask == 1) - (smask == 4),
+                                   j + (smask == 2) - (smask == 8), DIFF_CENTRAL, DIFF_CENTRAL);
+            double s[3];
+            stress_of(c, e, s);
+#pragma unroll
+            for (int q = 0; q < 3; ++q) LBPS_ST(&B.s[((size_t)nb + b) * 3 + q], s[q]);
+        }
+    }
     const double phi = add_rn(d.xx, d.yy);
     const double psi = sub_rn(d.yx, d.xy);
     // Eq. correction-f with J(x_k, t) of the stored populations, then the value
@@ -330,9 +377,9 @@ template <typename P>
 __device__ __forceinline__ void boundary_stream_y(const Geo& g, const Consts& c, const KCof<P>& k, const View<P>& A,
                                          const View<P>& B, const BNode* __restrict__ bn, int b) {
     using V = typename P::V;
-    const int smask = LBPS_LD(&bn[b].smask) & 10;
+    const BPoint pt = point_of(g, bn, b);
+    const int smask = pt.smask & 10, i = pt.i, j = pt.j;
     if (!smask) return;
-    const int i = LBPS_LD(&bn[b].i), j = LBPS_LD(&bn[b].j);
     typename P::Raw ra, rb;
     P::template load_raw<false>(A.m, g.mplane, (size_t)b, true, ra);
     P::template load_raw<false>(B.m, g.mplane, (size_t)b, true, rb);
@@ -408,8 +455,9 @@ __device__ __forceinline__ int streamed_in(const Geo& g, int i, int j, size_t p)
 // frame passes of sweeps of several steps).
 // NC = false: copy A may have been written earlier in the same launch (the
 // many-step kernel, which is bound by FP64 instructions and has registers to
-// spare: it widens the accelerations with integer operations).
-template <typename P, int UVD, bool WIN = false, bool NC = true>
+// spare: it widens the accelerations with integer operations).  GEN, with NC =
+// false: a general geometry.
+template <typename P, int UVD, bool WIN = false, bool NC = true, bool GEN = false>
 __device__ __forceinline__ bool bulk_strip(const Geo& g, const Consts& c, const KCof<P>& k, const View<P>& A,
                                            const View<P>& B, int xs, int j0, int j1, Win w = Win{0, 0, 0, 0}) {
     using V = typename P::V;
@@ -455,9 +503,14 @@ __device__ __forceinline__ bool bulk_strip(const Geo& g, const Consts& c, const 
         Cm[s] = add_rn(add_rn(Cf[s][1], Cf[s][2]), add_rn(Cf[s][3], Cf[s][4]));
         Cs[s] = add_rn(Cf[s][0], Cm[s]);
     }
+    // GEN: the node types, one row ahead too (loaded where they are used, their
+    // latency is in every row's chain: 1024^2 with a hole 41.8 us a step, now 40)
+    unsigned Ct = 0, Nt = 0;
+    if (GEN) Ct = LBPS_LDG(&g.type[at(j0)]);
     bool bad = false;
     for (int j = j0; j < j1; ++j) {
         // prefetch: populations two rows ahead, u and du/dt one row ahead
+        if (GEN) Nt = LBPS_LDG(&g.type[at(j + 1)]);
         P::template load_raw<NC>(A.f, PL, at(j + 2), col_ok && row_ok(j + 2) && j + 2 <= j1, Qr);
         if (UVD == 2)
             load_uv<NC>(A.u, PL, at(j + 2), out_lane && j + 2 < j1, Qu);
@@ -491,7 +544,7 @@ __device__ __forceinline__ bool bulk_strip(const Geo& g, const Consts& c, const 
             const size_t p = at(j);
             // general geometry: only interior points (boundary and void points
             // are the boundary passes' or stay zero)
-            if (out_lane && (WIN || !g.general || LBPS_LDG(&g.type[p]) == 0)) {
+            if (out_lane && (GEN ? Ct == 0 : WIN || !g.general || LBPS_LDG(&g.type[p]) == 0)) {
                 double ax, ay;
                 accel_interior<V, !NC>(sW[0], sE[0], Ps[0], Ns[0], sW[1], sE[1], Ps[1], Ns[1], k, ax, ay);
                 double u1[4];
@@ -517,6 +570,7 @@ __device__ __forceinline__ bool bulk_strip(const Geo& g, const Consts& c, const 
             for (int q = 0; q < 5; ++q) Cf[s][q] = Nf[s][q];
         }
         decode_row<P>(Qr, k, Nf);
+        if (GEN) Ct = Nt;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             Cu[q] = Nu[q];
@@ -525,6 +579,99 @@ __device__ __forceinline__ bool bulk_strip(const Geo& g, const Consts& c, const 
     }
     return bad;
 }
+
+// The interior kernel on a few columns [x0, x1) next to a left or right edge of
+// a rectangle: the warp is 32 / W groups of W lanes, each marching down its own
+// `rows` rows of [j0, je) (group q from j0 + q rows) over the W columns from xb
+// on, which hold [x0 - 1, x1].  A strip of 32 columns there would have a handful
+// of its lanes in the window and pay each row's FP64 instructions (64 cycles
+// each) and loads for them; here one instruction serves 32 / W rows.  The
+// arithmetic of bulk_strip.
+template <typename P, int W>
+__device__ __forceinline__ bool side_strip(const Geo& g, const Consts& c, const KCof<P>& k, const View<P>& A,
+                                           const View<P>& B, int xb, int x0, int x1, int j0, int je, int rows) {
+    using V = typename P::V;
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int col = xb + lane % W;                       // inside the lattice (sides >= W)
+    const int jb = min(j0 + lane / W * rows, je), jend = min(jb + rows, je);
+    const bool out_col = col >= x0 && col < x1;
+    const size_t PL = g.plane;
+    // rows up to jend (at most ny - 1) are read, further ones clamped and masked
+    auto at = [&](int j) { return (size_t)min(j, jend) * (size_t)g.px + (size_t)col; };
+
+    V Ps[2], Pf4[2];
+    V Cf[2][5], Nf[2][5];
+    typename P::Raw Qr;
+    double Cu[4], Nu[4];
+    {
+        V t[2][5];
+        P::load_raw(A.f, PL, at(jb - 1), true, Qr);
+        decode_row<P>(Qr, k, t);
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            Ps[s] = sum5(t[s][0], t[s][1], t[s][2], t[s][3], t[s][4]);
+            Pf4[s] = t[s][4];
+        }
+    }
+    P::load_raw(A.f, PL, at(jb), true, Qr);
+    decode_row<P>(Qr, k, Cf);
+    P::load_raw(A.f, PL, at(jb + 1), true, Qr);
+    decode_row<P>(Qr, k, Nf);
+    load_uv(A.u, PL, at(jb), out_col && jb < jend, Cu);
+    bool bad = false;
+    for (int r = 0; r < rows; ++r) {
+        const int j = jb + r;
+        P::load_raw(A.f, PL, at(j + 2), j + 2 <= jend, Qr);
+        load_uv(A.u, PL, at(j + 1), out_col && j + 1 < jend, Nu);
+        V sW[2], sE[2], Cs[2], Ns[2], out[2][5];
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const V Cm = add_rn(add_rn(Cf[s][1], Cf[s][2]), add_rn(Cf[s][3], Cf[s][4]));
+            Cs[s] = add_rn(Cf[s][0], Cm);
+            Ns[s] = sum5(Nf[s][0], Nf[s][1], Nf[s][2], Nf[s][3], Nf[s][4]);
+            sW[s] = __shfl_up_sync(FULL, Cs[s], 1, W);
+            sE[s] = __shfl_down_sync(FULL, Cs[s], 1, W);
+            const V f3W = __shfl_up_sync(FULL, Cf[s][3], 1, W);
+            const V f1E = __shfl_down_sync(FULL, Cf[s][1], 1, W);
+            out[s][0] = add_rn(Cf[s][0], fma_rn(k.two_a0[s], Cm, -mul_rn(k.eight_a[s], Cf[s][0])));
+            out[s][1] = fma_rn(k.two_a[s], sW[s], -f3W);
+            out[s][3] = fma_rn(k.two_a[s], sE[s], -f1E);
+            out[s][2] = fma_rn(k.two_a[s], Ps[s], -Pf4[s]);
+            out[s][4] = fma_rn(k.two_a[s], Ns[s], -Nf[s][2]);
+        }
+        if (out_col && j < jend) {
+            const size_t p = at(j);
+            double ax, ay, u1[4];
+            accel_interior<V, true>(sW[0], sE[0], Ps[0], Ns[0], sW[1], sE[1], Ps[1], Ns[1], k, ax, ay);
+            newmark(Cu[0], Cu[2], ax, c, u1[0], u1[2]);
+            newmark(Cu[1], Cu[3], ay, c, u1[1], u1[3]);
+            if constexpr (P::kSplitStream)
+                P::store_point_pins(B.f, PL, p, out, k, streamed_in<true>(g, col, j, p));
+            else
+                P::store_point(B.f, PL, p, out, k);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) LBPS_ST(&B.u[(size_t)q * PL + p], u1[q]);
+            bad |= !isfinite(out[0][0] + out[1][0]);
+        }
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            Ps[s] = Cs[s];
+            Pf4[s] = Cf[s][4];
+#pragma unroll
+            for (int q = 0; q < 5; ++q) Cf[s][q] = Nf[s][q];
+        }
+        decode_row<P>(Qr, k, Nf);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) Cu[q] = Nu[q];
+    }
+    return bad;
+}
+
+// Rows per group of a side strip, and the rows of a side task of the batch
+// (groups of 8 lanes).
+constexpr int kSideRows = 8;
+static_assert(kSideTaskRows == 4 * kSideRows, "a side task is one warp");
 
 // ------------------------------------------------- two steps per sweep
 

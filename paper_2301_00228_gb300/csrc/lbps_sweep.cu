@@ -109,7 +109,8 @@ struct Acc {
 template <typename P, int K>
 __device__ __forceinline__ bool sweep_strip(const Geo& g, const Consts& c, const KCof<P>& k,
                                             const CUtensorMap* mf, const CUtensorMap* mu, const View<P>& B, char* ring,
-                                            unsigned long long* bars, int xs, int j0, int j1, bool& timeout) {
+                                            unsigned long long* bars, unsigned& base, int xs, int j0, int j1,
+                                            bool& timeout) {
     using V = typename P::V;
     using S = Sweep<P, K>;
     const unsigned FULL = 0xffffffffu;
@@ -120,21 +121,21 @@ __device__ __forceinline__ bool sweep_strip(const Geo& g, const Consts& c, const
     const int nq = j1 - j0 + 2 * K, ngroups = (nq + 1) / 2;   // rows read, and pairs of them
     const int nit = nq - 2;
 
+    // pair q of this strip is pair base + q of the warp's ring
+    auto slot_of = [&](int q) { return (int)((base + (unsigned)q) % (unsigned)S::DEPTH); };
+    auto arrived = [&](int q) {
+        return mbar_wait(bars + slot_of(q), ((base + (unsigned)q) / (unsigned)S::DEPTH) & 1u);
+    };
     auto issue = [&](int q) {   // lane 0
-        char* slot = ring + (q % S::DEPTH) * S::SLOT;
-        unsigned long long* bar = bars + q % S::DEPTH;
+        char* slot = ring + slot_of(q) * S::SLOT;
+        unsigned long long* bar = bars + slot_of(q);
         // rows j0 - K + 2q, + 1 of the populations; the rows that leave while they enter
         mbar_expect(bar, S::F_BYTES + (q >= K ? S::U_BYTES : 0));
         tma_load(slot, mf, xs - K - S::SKIP, j0 - K + 2 * q, bar);
         if (q >= K) tma_load(slot + S::U_OFF, mu, xs, j0 + 2 * (q - K), bar);
     };
-    if (lane == 0) {
-        for (int q = 0; q < S::DEPTH; ++q) mbar_init(bars + q);
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    if (lane == 0)
         for (int q = 0; q < S::DEPTH && q < ngroups; ++q) issue(q);
-    }
-    __syncwarp();
 
     auto read_row = [&](const char* slot, int half, V (&f)[2][5]) {
         const unsigned* w = reinterpret_cast<const unsigned*>(slot) + half * S::BOX + S::SKIP + lane;
@@ -229,30 +230,29 @@ __device__ __forceinline__ bool sweep_strip(const Geo& g, const Consts& c, const
     };
 
     // rows 0 and 1: the window of the first stage
-    if (!mbar_wait(bars, 0)) {
+    if (!arrived(0)) {
         timeout = true;
         return false;
     }
     {
+        const char* slot = ring + slot_of(0) * S::SLOT;
         V t[2][5];
-        read_row(ring, 0, t);
+        read_row(slot, 0, t);
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             Ps[0][q] = sum5(t[q][0], t[q][1], t[q][2], t[q][3], t[q][4]);
             P4[0][q] = t[q][4];
         }
-        read_row(ring, 1, Cf[0]);
+        read_row(slot, 1, Cf[0]);
 #pragma unroll
         for (int q = 0; q < 2; ++q)
             Cm[0][q] = add_rn(add_rn(Cf[0][q][1], Cf[0][q][2]), add_rn(Cf[0][q][3], Cf[0][q][4]));
     }
     release_slot();
     if (lane == 0 && S::DEPTH < ngroups) issue(S::DEPTH);
-    int slot_i = 1;
-    unsigned parity = 0;
     for (int q = 1; q < ngroups; ++q) {
-        char* slot = ring + slot_i * S::SLOT;
-        if (!mbar_wait(bars + slot_i, parity)) {
+        char* slot = ring + slot_of(q) * S::SLOT;
+        if (!arrived(q)) {
             timeout = true;
             return bad;
         }
@@ -260,12 +260,20 @@ __device__ __forceinline__ bool sweep_strip(const Geo& g, const Consts& c, const
         if (2 * q - 1 < nit) iterate(slot, 1, 2 * q - 1);
         release_slot();
         if (lane == 0 && q + S::DEPTH < ngroups) issue(q + S::DEPTH);
-        if (++slot_i == S::DEPTH) {
-            slot_i = 0;
-            parity ^= 1;
-        }
     }
+    base += (unsigned)ngroups;
     return bad;
+}
+
+// The barriers of a warp's ring, before its first strip.
+template <typename S>
+__device__ __forceinline__ void init_ring(unsigned long long* bars) {
+    if ((threadIdx.x & 31) == 0) {
+        for (int q = 0; q < S::DEPTH; ++q) mbar_init(bars + q);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
 }
 
 // What bounds it: K = 4 in FP32, the FP64 pipe (12 instructions of 64 cycles a
@@ -290,11 +298,78 @@ __global__ void __launch_bounds__(128, MINB) sweep_kernel(Geo g, Consts c, KCof<
     const int xs = (blockIdx.x * kWarpsPerBlock + wid) * S::OUT;
     const int j0 = S::DEEP + blockIdx.y * rows, j1 = min(j0 + rows, g.ny - S::DEEP);
     if (xs >= g.nx - S::DEEP || j0 >= j1) return;   // whole warp
+    init_ring<S>(bars + wid * S::DEPTH);
     bool timeout = false;
+    unsigned base = 0;
     const bool bad = sweep_strip<P, K>(g, c, k, &mf, &mu, B, smem + wid * (S::DEPTH * S::SLOT),
-                                       bars + wid * S::DEPTH, xs, j0, j1, timeout);
+                                       bars + wid * S::DEPTH, base, xs, j0, j1, timeout);
     if (timeout) atomicOr(flag, kFlagTimeout);
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, kFlagNonfinite);
+}
+
+// Stage 1 of a pair of steps of every lattice of a batch (launch_pair_batch):
+// the two-step strips as sweeps of K = 2 fed by TMA, the frame strips and
+// Newmark tasks as in pair_batch_kernel.  The tensor maps of each lattice's
+// two copies lie in device memory.
+template <typename P>
+__global__ void __launch_bounds__(128, 4) sweep_batch_kernel(const DomDesc<P>* __restrict__ dd,
+                                                             const SweepMaps* __restrict__ maps,
+                                                             const PairTask* __restrict__ tasks, int ntasks,
+                                                             const BndTask* __restrict__ btasks, int parity,
+                                                             unsigned* next) {
+    using S = Sweep<P, 2>;
+    extern __shared__ __align__(128) char smem[];
+    __shared__ unsigned long long bars[kWarpsPerBlock * S::DEPTH];
+    __shared__ DomDesc<P> sd[kWarpsPerBlock];
+    const unsigned FULL = 0xffffffffu;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    init_ring<S>(bars + wid * S::DEPTH);
+    unsigned base = 0;
+    int cached = -1;
+    for (;;) {
+        unsigned t = 0;
+        if (lane == 0) t = atomicAdd(next, 1u);
+        t = __shfl_sync(FULL, t, 0);
+        if (t >= (unsigned)ntasks) break;  // whole warp
+        const PairTask tk = tasks[t];
+        if (tk.kind == kNewmarkTask) {
+            if (lane < tk.j1) {
+                const BndTask bt = btasks[tk.xs + lane];
+                const DomDesc<P>& d = dd[bt.dom];
+                const int a = d.cur ^ parity;
+                const double n = (double)LBPS_LD(d.tstep);
+                boundary_newmark(d.g, d.c, d.v[a], d.x, d.bn, d.nb, d.v[a].s, n, bt.b, 0);
+                boundary_newmark(d.g, d.c, d.v[a], d.x, d.bn, d.nb, d.v[a].s, n, bt.b, 1);
+            }
+            continue;
+        }
+        if (tk.dom != cached) {
+            __syncwarp();  // every lane is done with the previous descriptor
+            const unsigned* src = reinterpret_cast<const unsigned*>(dd + tk.dom);
+            unsigned* dst = reinterpret_cast<unsigned*>(sd + wid);
+            for (int q = lane; q < (int)(sizeof(DomDesc<P>) / 4); q += 32) dst[q] = src[q];
+            __syncwarp();
+            cached = tk.dom;
+        }
+        const DomDesc<P>& d = sd[wid];
+        const int a = d.cur ^ parity;
+        bool bad, timeout = false;
+        if (tk.kind == kPairStrip) {
+            const CUtensorMap* m = reinterpret_cast<const CUtensorMap*>(maps + tk.dom) + 2 * a;
+            bad = sweep_strip<P, 2>(d.g, d.c, d.k, m, m + 1, d.v[a ^ 1], smem + wid * (S::DEPTH * S::SLOT),
+                                    bars + wid * S::DEPTH, base, tk.xs, tk.j0, tk.j1, timeout);
+        } else if (tk.kind == kSideStrip) {
+            bad = side_strip<P, 8>(d.g, d.c, d.k, d.v[a], d.x, tk.xs, tk.x0, tk.x1, tk.j0, tk.j1, kSideRows);
+        } else {
+            bad = bulk_strip<P, 1, true>(d.g, d.c, d.k, d.v[a], d.x, tk.xs, tk.j0, tk.j1,
+                                         Win{tk.x0, tk.x1, tk.y0, tk.y1});
+        }
+        if (timeout) {
+            atomicOr(d.flag, kFlagTimeout);
+            break;
+        }
+        if (__any_sync(FULL, bad) && lane == 0) atomicOr(d.flag, kFlagNonfinite);
+    }
 }
 
 using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
@@ -344,9 +419,46 @@ cudaError_t launch_sweep(const Geo& g, const Consts& c, const KCof<P>& k, View<P
     return cudaGetLastError();
 }
 
+static_assert(sizeof(SweepMaps) == 4 * sizeof(CUtensorMap), "four tensor maps");
+
+template <typename P>
+cudaError_t make_sweep_maps(const Geo& g, View<P> v0, View<P> v1, SweepMaps* out) {
+    using S = Sweep<P, 2>;
+    CUtensorMap m[4];
+    const View<P> v[2] = {v0, v1};
+    cudaError_t e = cudaSuccess;
+    for (int q = 0; q < 2 && e == cudaSuccess; ++q) {
+        e = encode(&m[2 * q], CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, v[q].f, g, S::PLANES, S::BOX);
+        if (e == cudaSuccess) e = encode(&m[2 * q + 1], CU_TENSOR_MAP_DATA_TYPE_UINT64, 8, v[q].u, g, 4, S::OUT);
+    }
+    if (e == cudaSuccess) memcpy(out, m, sizeof(m));
+    return e;
+}
+
+template <typename P>
+cudaError_t launch_sweep_batch(const DomDesc<P>* dd, const SweepMaps* maps, const PairTask* tasks, int ntasks,
+                               const BndTask* btasks, int parity, unsigned* next, cudaStream_t st) {
+    using S = Sweep<P, 2>;
+    if (ntasks <= 0) return cudaSuccess;
+    auto kern = sweep_batch_kernel<P>;
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * kWarpsPerBlock, S::kSmem);
+    if (e != cudaSuccess) return e;
+    const int blocks = min(sms * max(per_sm, 1), (ntasks + kWarpsPerBlock - 1) / kWarpsPerBlock);
+    kern<<<blocks, 32 * kWarpsPerBlock, S::kSmem, st>>>(dd, maps, tasks, ntasks, btasks, parity, next);
+    return cudaGetLastError();
+}
+
 #define LBPS_INSTANTIATE(P)                                                                                       \
     template cudaError_t launch_sweep<P, 2>(const Geo&, const Consts&, const KCof<P>&, View<P>, View<P>, unsigned*, \
-                                            cudaStream_t);
+                                            cudaStream_t);                                                        \
+    template cudaError_t make_sweep_maps<P>(const Geo&, View<P>, View<P>, SweepMaps*);                            \
+    template cudaError_t launch_sweep_batch<P>(const DomDesc<P>*, const SweepMaps*, const PairTask*, int,         \
+                                               const BndTask*, int, unsigned*, cudaStream_t);
 
 LBPS_INSTANTIATE(PopDirect<float>)
 LBPS_INSTANTIATE(PopNeq16<__nv_bfloat16>)
