@@ -233,7 +233,14 @@ int lbps_init_device(lbps_lattice* lat, const double* d_ux0, const double* d_uy0
  * (Eq. psi_phi_at_bound, correction-f), LBE with the averaged boundary state
  * (Eq. LBE, LBE_mod), and every sync_every-th step the synchronisation of
  * Sec. 3.2.  Enqueues the work, then waits for the stream and returns
- * LBPS_ERR_NONFINITE if any update produced a non-finite value. */
+ * LBPS_ERR_NONFINITE if any update produced a non-finite value.
+ * Rectangles without periodic axes of 500000 to 3000000 points (64 a side or
+ * more, not FP64 storage) take their steps two per sweep with the bits of
+ * single steps; the first call of two steps or more allocates a scratch copy
+ * for that (cudaMalloc, the size of one state copy; freed at lbps_destroy, or
+ * by lbps_set_step_pairs(lat, 0), after which the lattice keeps to launches
+ * without scratch; without the memory it does so by itself).  Fully periodic
+ * lattices from 500000 points on do the same without scratch. */
 int lbps_step(lbps_lattice* lat, int64_t n);
 
 /* As lbps_step without the final wait and check (use lbps_check later). */

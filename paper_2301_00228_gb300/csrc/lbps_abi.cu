@@ -442,12 +442,73 @@ int run_step(lbps_lattice* lat) {
     return LBPS_OK;
 }
 
-// Two steps per sweep apply to rectangles without periodic axes, at least
-// 16 points a side, with the scratch copy allocated and per-kernel timing off.
-bool pair_ok(const lbps_lattice* lat) {
+// Sweeps of several steps apply to rectangles without periodic axes, at least
+// 16 points a side.
+bool sweeps_apply(const lbps_lattice* lat) {
     const lbps::Geo& g = lat->L.g;
-    return lat->xmem && lat->side && !g.general && !g.periodic_x && !g.periodic_y && g.nx >= 16 && g.ny >= 16 &&
-           lat->L.nb > 0;
+    return lat->side && !g.general && !g.periodic_x && !g.periodic_y && g.nx >= 16 && g.ny >= 16 && lat->L.nb > 0;
+}
+
+// Two steps per sweep, with the scratch copy allocated: turned on by the
+// caller, or exact ones (below) unless the caller asked for single steps'
+// timing or launch shape.
+bool pair_ok(const lbps_lattice* lat) {
+    return lat->xmem && sweeps_apply(lat) && (lat->pairs || (lat->exact && !lat->prof && !lat->tuned));
+}
+
+// Single steps as sweeps of two whose u, du/dt take the steps one by one: the
+// bits of single steps, half their traffic.  Up to the size from which the
+// binding turns on the caller's sweeps; below, the boundary chain (about 29 us
+// per pair) is longer than many steps in one launch.  Measured, us a step
+// against single steps: 700 x 500 14.6 / 13.4, 800^2 15.4 / 19.7 (BF16 18.7 /
+// 22.2), 1024^2 21.0 / 27.4 (BF16 24.7 / 33.9, BFP13 23.9 / 38.0), 1600^2 46 / 74;
+// periodic 512^2 10.3 / 8.9, 768^2 12.0 / 14.7, 1024^2 17.7 / 27.4, 2048^2 59 /
+// 103.
+constexpr int64_t kExactMinPoints = 500000;
+constexpr int64_t kExactMaxPoints = 3000000;
+constexpr int32_t kExactMinSide = 64;
+
+bool exact_wanted(const lbps_lattice* lat) {
+    const int64_t points = (int64_t)lat->L.g.nx * lat->L.g.ny;
+    return sweeps_apply(lat) && !lat->pairs && !lat->exact && !lat->no_scratch && !lat->prof && !lat->tuned &&
+           lat->p.storage != LBPS_STORAGE_F64 && points >= kExactMinPoints && points < kExactMaxPoints &&
+           std::min(lat->L.g.nx, lat->L.g.ny) >= kExactMinSide;
+}
+
+// The scratch copy of a lattice's sweeps, zeroed once: parts of it the frame
+// passes read but do not use then hold finite values.
+int make_scratch(lbps_lattice* lat, char** out) {
+    void* x = nullptr;
+    if (cudaMalloc(&x, lat->L.copy_bytes) != cudaSuccess) {
+        cudaGetLastError();
+        return LBPS_ERR_OOM;
+    }
+    if (cudaMemset(x, 0, lat->L.copy_bytes) != cudaSuccess ||
+        lbps::set_check_range(x, lat->L.copy_bytes, lat->st) != cudaSuccess) {
+        cudaFree(x);
+        cudaGetLastError();
+        return LBPS_ERR_CUDA;
+    }
+    *out = static_cast<char*>(x);
+    return LBPS_OK;
+}
+
+void drop_scratch(lbps_lattice* lat) {
+    for (char** x : {&lat->ymem, &lat->xmem}) {
+        if (!*x) continue;
+        lbps::set_check_range(*x, 0, lat->st);
+        cudaFree(*x);
+        *x = nullptr;
+    }
+}
+
+// Lattices periodic in both axes take exact sweeps of every point, without
+// scratch and without a boundary chain.
+bool periodic_pairs(const lbps_lattice* lat) {
+    const lbps::Geo& g = lat->L.g;
+    return !g.general && g.periodic_x && g.periodic_y && !lat->prof && !lat->tuned &&
+           lat->p.storage != LBPS_STORAGE_F64 && (int64_t)g.nx * g.ny >= kExactMinPoints &&
+           std::min(g.nx, g.ny) >= kExactMinSide;
 }
 
 // Steps n and n + 1 in one sweep of the interior.  Copy A (current) holds
@@ -476,9 +537,11 @@ int run_pair(lbps_lattice* lat) {
             if (r == cudaSuccess) {
                 if constexpr (sizeof(typename P::V) == 8)
                     r = lbps::launch_pair<P>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st, 32);
+                else if (lat->pairs)
+                    r = lbps::launch_sweep<P, 2, false>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st);
                 else
-                    r = lbps::launch_sweep<P, 2>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st);
-                if (r == cudaErrorNotSupported)   // a driver without tensor maps
+                    r = lbps::launch_sweep<P, 2, true>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st);
+                if (r == cudaErrorNotSupported && lat->pairs)   // a driver without tensor maps
                     r = lbps::launch_pair<P>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st, 32);
             }
             if (r == cudaSuccess) r = prof_mark(lat);
@@ -512,7 +575,7 @@ int run_pair(lbps_lattice* lat) {
 constexpr int64_t kQuadMinPoints = 3000000;
 constexpr int32_t kQuadMinSide = 64;
 
-bool quad_ok(const lbps_lattice* lat) { return lat->ymem && pair_ok(lat); }
+bool quad_ok(const lbps_lattice* lat) { return lat->ymem && lat->pairs && pair_ok(lat); }
 
 // Four steps, n .. n + 3, in one sweep of the interior, as run_pair: copy A
 // (current) holds step n, copy B receives step n + 4, and the scratch copies X
@@ -533,7 +596,7 @@ int run_quad(lbps_lattice* lat) {
             cudaError_t r = prof_mark(lat);
             if constexpr (std::is_same<P, lbps::PolF32>::value) {
                 if (r == cudaSuccess)
-                    r = lbps::launch_sweep<P, 4>(g, lat->c, lat->kc<P>(), copy[0], copy[3], lat->flag(), lat->st);
+                    r = lbps::launch_sweep<P, 4, false>(g, lat->c, lat->kc<P>(), copy[0], copy[3], lat->flag(), lat->st);
             } else {
                 r = cudaErrorNotSupported;   // other storages have no second scratch copy
             }
@@ -564,6 +627,26 @@ int run_quad(lbps_lattice* lat) {
     return LBPS_OK;
 }
 
+// Two steps of a lattice periodic in both axes (periodic_pairs).
+int run_periodic_pair(lbps_lattice* lat) {
+    const int a = lat->cur, b = lat->cur ^ 1;
+    const cudaError_t e = lbps::with_policy(lat->p.storage, [&](auto pol) {
+        using P = decltype(pol);
+        if constexpr (sizeof(typename P::V) == 8)
+            return cudaErrorNotSupported;
+        else
+            return lbps::launch_sweep_periodic<P>(lat->L.g, lat->c, lat->kc<P>(), lat->view<P>(a), lat->view<P>(b),
+                                                  lat->flag(), lat->st);
+    });
+    if (e != cudaSuccess) {
+        lat->last_cuda = (int)e;
+        return LBPS_ERR_CUDA;
+    }
+    lat->cur = b;
+    lat->steps += 2;
+    return LBPS_OK;
+}
+
 // k steps: four or two in one sweep where they apply, else single steps
 int run_steps(lbps_lattice* lat, int k) {
     int rc = LBPS_OK;
@@ -571,6 +654,9 @@ int run_steps(lbps_lattice* lat, int k) {
         if (k - s >= 4 && quad_ok(lat)) {
             rc = run_quad(lat);
             s += 4;
+        } else if (k - s >= 2 && periodic_pairs(lat)) {
+            rc = run_periodic_pair(lat);
+            s += 2;
         } else if (k - s >= 2 && pair_ok(lat)) {
             rc = run_pair(lat);
             s += 2;
@@ -647,14 +733,14 @@ int step_graph(lbps_lattice* lat, int k, cudaGraphExec_t* out, int* end_cur) {
 // replayed graph cost no more than the barriers.  Measured, us a step, one
 // launch against graphs of 32 steps: 64^2 FP64 10.9 / 15.7, 128 x 96 7.2 / 9.1,
 // 300^2 8.7 / 10.2 (BF16 11.5 / 13.3, BFP13 13.9 / 16.2), 389 x 1171 15.7 /
-// 18.1, 800^2 19.6 / 21.8, 1024^2 27.4 / 29.2 (BF16 33.7 / 33.6, with a hole
-// 41.8 / 45.7), 1536^2 71 / 59.
+// 18.1, 1024^2 with a hole 39.5 / 45.7, 1536^2 71 / 59.  (Rectangles and fully
+// periodic lattices from 500000 points on take exact sweeps instead.)
 constexpr int64_t kFusedMaxPoints = 1200000;
 // Steps per launch at most (tens of milliseconds at the largest size).
 constexpr int64_t kFusedMaxSteps = 1024;
 
 bool fused_ok(const lbps_lattice* lat) {
-    return !lat->fused_off && !lat->prof && !lat->tuned && !pair_ok(lat) &&
+    return !lat->fused_off && !lat->prof && !lat->tuned && !pair_ok(lat) && !periodic_pairs(lat) &&
            (int64_t)lat->L.g.nx * lat->L.g.ny <= kFusedMaxPoints;
 }
 
@@ -1114,15 +1200,19 @@ int lbps_step_async(lbps_lattice* lat, int64_t n) {
     if (!lat || n < 0) return LBPS_ERR_INVALID;
     if (!lat->initialised) return LBPS_ERR_STATE;
     const int l = lat->p.sync_every;
-    bool fused = fused_ok(lat);
-    if (fused) {
-        // a capturing stream gets the plain launches of single steps
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(lat->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
-            cudaGetLastError();
-            fused = false;
-        }
+    // a capturing stream gets the plain launches of single steps
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool capturing = cudaStreamIsCapturing(lat->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    if (capturing) cudaGetLastError();
+    if (n >= 2 && l != 1 && !capturing && exact_wanted(lat)) {
+        // once per lattice; without the memory it keeps to single steps
+        if (make_scratch(lat, &lat->xmem) == LBPS_OK)
+            lat->exact = true;
+        else
+            lat->no_scratch = true;
+        lat->gen += 1;
     }
+    bool fused = !capturing && fused_ok(lat);
     for (int64_t s = 0; s < n;) {
         if (fused) {
             int64_t m = std::min(n - s, kFusedMaxSteps);
@@ -1162,6 +1252,10 @@ int lbps_step_async(lbps_lattice* lat, int64_t n) {
             int rc = run_quad(lat);
             if (rc != LBPS_OK) return rc;
             s += 4;
+        } else if (n - s >= 2 && periodic_pairs(lat) && !(l > 0 && (lat->steps + 1) % l == 0)) {
+            int rc = run_periodic_pair(lat);
+            if (rc != LBPS_OK) return rc;
+            s += 2;
         } else if (n - s >= 2 && pair_ok(lat) && !(l > 0 && (lat->steps + 1) % l == 0)) {
             int rc = run_pair(lat);
             if (rc != LBPS_OK) return rc;
@@ -1422,50 +1516,32 @@ int lbps_set_tuning(lbps_lattice* lat, int32_t variant, int32_t rows_per_warp) {
 
 int lbps_set_step_pairs(lbps_lattice* lat, int32_t on) {
     if (!lat || on < 0 || on > 1) return LBPS_ERR_INVALID;
-    if ((on != 0) == (lat->xmem != nullptr)) return LBPS_OK;
+    if (on == 0) lat->no_scratch = true;   // no exact sweeps either: their scratch copy would come back
+    if ((on != 0) == lat->pairs && !(on == 0 && lat->xmem)) return LBPS_OK;
     if (cudaStreamSynchronize(lat->st) != cudaSuccess) return LBPS_ERR_CUDA;
     if (on) {
-        void* x = nullptr;
-        if (cudaMalloc(&x, lat->L.copy_bytes) != cudaSuccess) {
-            cudaGetLastError();
-            return LBPS_ERR_OOM;
+        if (!lat->xmem) {
+            const int rc = make_scratch(lat, &lat->xmem);
+            if (rc != LBPS_OK) return rc;
         }
-        // zeroed once: parts of it the frame passes read but do not use then hold finite values
-        if (cudaMemset(x, 0, lat->L.copy_bytes) != cudaSuccess ||
-            lbps::set_check_range(x, lat->L.copy_bytes, lat->st) != cudaSuccess) {
-            cudaFree(x);
-            cudaGetLastError();
-            return LBPS_ERR_CUDA;
-        }
-        lat->xmem = static_cast<char*>(x);
         // the second scratch copy of four steps per sweep; without it the
         // lattice takes two
         if (lat->p.storage == LBPS_STORAGE_F32 && (int64_t)lat->p.nx * lat->p.ny >= kQuadMinPoints &&
-            std::min(lat->p.nx, lat->p.ny) >= kQuadMinSide && cudaMalloc(&x, lat->L.copy_bytes) == cudaSuccess) {
-            if (cudaMemset(x, 0, lat->L.copy_bytes) == cudaSuccess &&
-                lbps::set_check_range(x, lat->L.copy_bytes, lat->st) == cudaSuccess)
-                lat->ymem = static_cast<char*>(x);
-            else
-                cudaFree(x);
-        }
-        cudaGetLastError();
+            std::min(lat->p.nx, lat->p.ny) >= kQuadMinSide)
+            make_scratch(lat, &lat->ymem);
+        lat->pairs = true;
     } else {
-        if (lat->ymem) {
-            lbps::set_check_range(lat->ymem, 0, lat->st);
-            cudaFree(lat->ymem);
-            lat->ymem = nullptr;
-        }
-        lbps::set_check_range(lat->xmem, 0, lat->st);
-        cudaFree(lat->xmem);
-        lat->xmem = nullptr;
+        drop_scratch(lat);
+        lat->pairs = false;
     }
+    lat->exact = false;
     lat->gen += 1;  // captured step graphs hold the other kind of step
     return LBPS_OK;
 }
 
 int lbps_step_pairs(const lbps_lattice* lat) {
     if (!lat) return LBPS_ERR_INVALID;
-    return pair_ok(lat) ? 1 : 0;
+    return lat->pairs && pair_ok(lat) ? 1 : 0;
 }
 
 int lbps_set_graph_steps(lbps_lattice* lat, int32_t k) {
@@ -1609,16 +1685,8 @@ void lbps_destroy(lbps_lattice* lat) {
     if (lat->fork) cudaEventDestroy(lat->fork);
     if (lat->join) cudaEventDestroy(lat->join);
     if (lat->mem) lbps::set_check_range(lat->mem, 0, lat->st);  // checked builds: the block is no longer live
-    if (lat->ymem) {
-        lbps::set_check_range(lat->ymem, 0, lat->st);
-        cudaStreamSynchronize(lat->st);
-        cudaFree(lat->ymem);
-    }
-    if (lat->xmem) {
-        lbps::set_check_range(lat->xmem, 0, lat->st);
-        cudaStreamSynchronize(lat->st);
-        cudaFree(lat->xmem);
-    }
+    if (lat->xmem) cudaStreamSynchronize(lat->st);
+    drop_scratch(lat);
     if (lat->owns && lat->mem) {
         cudaStreamSynchronize(lat->st);
         cudaFree(lat->mem);

@@ -67,9 +67,15 @@ cudaError_t launch_frame(const Geo& g, const Consts& c, const KCof<P>& k, View<P
                          cudaStream_t st, int fw);
 
 // K steps (2 or 4) of the points at least K + 1 from every edge, A -> B.
-template <typename P, int K>
+// EXACT (K = 2): u, du/dt take the steps one by one, the bits of single steps.
+template <typename P, int K, bool EXACT>
 cudaError_t launch_sweep(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, View<P> B, unsigned* flag,
                          cudaStream_t st);
+// Two exact steps of every point of a lattice periodic in both axes (sides of
+// at least 64), A -> B.
+template <typename P>
+cudaError_t launch_sweep_periodic(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, View<P> B, unsigned* flag,
+                                  cudaStream_t st);
 
 template <typename P>
 cudaError_t launch_sync(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, cudaStream_t st);

@@ -86,10 +86,13 @@ struct lbps_lattice {
     char* mem;
     bool owns;
     int cur;            // copy holding time t
-    // two steps per sweep (lbps_set_step_pairs): the scratch state copy that
-    // holds step n + 1 on the boundary and the points up to 3 from it
-    // (cudaMalloc'd, copy_bytes), null when off
+    // sweeps of two steps: the scratch state copy that holds step n + 1 on the
+    // boundary and the points up to 3 from it (cudaMalloc'd, copy_bytes).
+    // pairs: turned on by the caller (lbps_set_step_pairs); exact: by
+    // lbps_step on a mid-size lattice, for the bits of single steps;
+    // no_scratch: the caller turned sweeps off, or there was no memory.
     char* xmem = nullptr;
+    bool pairs = false, exact = false, no_scratch = false;
     // four steps per sweep (large lattices): a second scratch copy
     char* ymem = nullptr;
     lbps::Tuning tuning;  // bulk-kernel launch shape

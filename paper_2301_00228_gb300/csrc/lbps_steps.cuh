@@ -689,18 +689,20 @@ constexpr int kDeep = 3;       // the two-step kernel writes points at least thi
 // at step n + 2 only on interior points at step n + 1 that are at least 2
 // from the edges, which the boundary reset of step n does not touch, so
 // nothing here needs the boundary passes.
-template <typename P>
+// WRAP: a lattice periodic in both axes; every point, and u, du/dt take the
+// steps one by one.
+template <typename P, bool WRAP = false>
 __device__ __forceinline__ bool pair_strip(const Geo& g, const Consts& c, const KCof<P>& k, const View<P>& A,
                                            const View<P>& B, int xs, int j0, int j1) {
     using V = typename P::V;
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int xl = xs - 2 + lane;
-    const bool col_ok = xl < g.nx;             // xl >= 1 always (xs >= kDeep)
-    const int col = col_ok ? xl : g.nx - 1;
-    const bool out_lane = lane >= 2 && lane < 2 + kPairCols && xl < g.nx - kDeep;
+    const bool col_ok = WRAP || xl < g.nx;             // without WRAP xl >= 1 always (xs >= kDeep)
+    const int col = WRAP ? wrap(xl, g.nx) : col_ok ? xl : g.nx - 1;
+    const bool out_lane = lane >= 2 && lane < 2 + kPairCols && xl < (WRAP ? g.nx : g.nx - kDeep);
     const size_t PL = g.plane;
-    auto at = [&](int j) { return (size_t)j * (size_t)g.px + (size_t)col; };
+    auto at = [&](int j) { return (size_t)(WRAP ? wrap(j, g.ny) : j) * (size_t)g.px + (size_t)col; };
 
     // step n (state n, read): rows r - 1, r, r + 1 and r + 2 in flight
     V P0s[2], P0f4[2];
@@ -797,8 +799,16 @@ __device__ __forceinline__ bool pair_strip(const Geo& g, const Consts& c, const 
                 V ax, ay;
                 accel_interior_v<V>(sW[0], sE[0], P1s[0], N1s[0], sW[1], sE[1], P1s[1], N1s[1], k, ax, ay);
                 double u2[4];
-                newmark2(C1u[0], C1u[2], C1a[0], ax, c, u2[0], u2[2]);
-                newmark2(C1u[1], C1u[3], C1a[1], ay, c, u2[1], u2[3]);
+                if constexpr (WRAP) {
+                    double u1[4];
+                    newmark(C1u[0], C1u[2], widen(C1a[0]), c, u1[0], u1[2]);
+                    newmark(C1u[1], C1u[3], widen(C1a[1]), c, u1[1], u1[3]);
+                    newmark(u1[0], u1[2], widen(ax), c, u2[0], u2[2]);
+                    newmark(u1[1], u1[3], widen(ay), c, u2[1], u2[3]);
+                } else {
+                    newmark2(C1u[0], C1u[2], C1a[0], ax, c, u2[0], u2[2]);
+                    newmark2(C1u[1], C1u[3], C1a[1], ay, c, u2[1], u2[3]);
+                }
                 P::store_point(B.f, PL, p, out, k);
 #pragma unroll
                 for (int q = 0; q < 4; ++q) LBPS_ST(&B.u[(size_t)q * PL + p], u2[q]);

@@ -15,6 +15,7 @@
 // stored form, so the populations are the bits of single steps.  u, du/dt wait
 // in shared memory until their row leaves and then take two steps at a time
 // (newmark2).
+#include <algorithm>
 #include <cstring>
 
 #include <cuda.h>
@@ -106,17 +107,19 @@ struct Acc {
     V sa[2], sb[2];  // 3 a0 + a1 and a0 + a1 of the pair before
 };
 
-template <typename P, int K>
+// EXACT: u, du/dt take the steps one by one (the bits of single steps), not two
+// at a time.  margin: the distance from the edges of the points it writes.
+template <typename P, int K, bool EXACT = false>
 __device__ __forceinline__ bool sweep_strip(const Geo& g, const Consts& c, const KCof<P>& k,
                                             const CUtensorMap* mf, const CUtensorMap* mu, const View<P>& B, char* ring,
                                             unsigned long long* bars, unsigned& base, int xs, int j0, int j1,
-                                            bool& timeout) {
+                                            bool& timeout, int margin = K + 1) {
     using V = typename P::V;
     using S = Sweep<P, K>;
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int col = xs - K + lane;
-    const bool out_lane = lane >= K && lane < 32 - K && col >= S::DEEP && col < g.nx - S::DEEP;
+    const bool out_lane = lane >= K && lane < 32 - K && col >= margin && col < g.nx - margin;
     const size_t PL = g.plane;
     const int nq = j1 - j0 + 2 * K, ngroups = (nq + 1) / 2;   // rows read, and pairs of them
     const int nit = nq - 2;
@@ -220,8 +223,16 @@ __device__ __forceinline__ bool sweep_strip(const Geo& g, const Consts& c, const
                     u[2 + q] = fma_rn(c.dt, sb, u[2 + q]);
                 }
             }
-            newmark2(u[0], u[2], from.a[0], ax, c, u[0], u[2]);
-            newmark2(u[1], u[3], from.a[1], ay, c, u[1], u[3]);
+            if constexpr (EXACT) {
+                static_assert(K == 2, "one acceleration is kept");
+                newmark(u[0], u[2], widen(from.a[0]), c, u[0], u[2]);
+                newmark(u[1], u[3], widen(from.a[1]), c, u[1], u[3]);
+                newmark(u[0], u[2], widen(ax), c, u[0], u[2]);
+                newmark(u[1], u[3], widen(ay), c, u[1], u[3]);
+            } else {
+                newmark2(u[0], u[2], from.a[0], ax, c, u[0], u[2]);
+                newmark2(u[1], u[3], from.a[1], ay, c, u[1], u[3]);
+            }
             P::store_point(B.f, PL, p, out, k);
 #pragma unroll
             for (int q = 0; q < 4; ++q) LBPS_ST(&B.u[(size_t)q * PL + p], u[q]);
@@ -286,7 +297,7 @@ __device__ __forceinline__ void init_ring(unsigned long long* bars) {
 // now FP32 two steps 1626, four steps 2304; FP16 1443).  Blocks per SM: what
 // the registers allow without spilling in earnest (K = 4 at 128 registers
 // spills 314 bytes and takes 3340 us).
-template <typename P, int K, int MINB>
+template <typename P, int K, int MINB, bool EXACT>
 __global__ void __launch_bounds__(128, MINB) sweep_kernel(Geo g, Consts c, KCof<P> k,
                                                           const __grid_constant__ CUtensorMap mf,
                                                           const __grid_constant__ CUtensorMap mu, View<P> B,
@@ -301,8 +312,36 @@ __global__ void __launch_bounds__(128, MINB) sweep_kernel(Geo g, Consts c, KCof<
     init_ring<S>(bars + wid * S::DEPTH);
     bool timeout = false;
     unsigned base = 0;
-    const bool bad = sweep_strip<P, K>(g, c, k, &mf, &mu, B, smem + wid * (S::DEPTH * S::SLOT),
+    const bool bad = sweep_strip<P, K, EXACT>(g, c, k, &mf, &mu, B, smem + wid * (S::DEPTH * S::SLOT),
                                        bars + wid * S::DEPTH, base, xs, j0, j1, timeout);
+    if (timeout) atomicOr(flag, kFlagTimeout);
+    if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, kFlagNonfinite);
+}
+
+// Two exact steps of a lattice periodic in both axes, every point: the strips
+// and chunks whose reads stay inside the planes by TMA, those across a seam
+// (a box does not wrap) with loads through registers.
+template <typename P, int MINB>
+__global__ void __launch_bounds__(128, MINB) sweep_periodic_kernel(Geo g, Consts c, KCof<P> k,
+                                                                   const __grid_constant__ CUtensorMap mf,
+                                                                   const __grid_constant__ CUtensorMap mu, View<P> A,
+                                                                   View<P> B, unsigned* flag, int rows) {
+    using S = Sweep<P, 2>;
+    extern __shared__ __align__(128) char smem[];
+    __shared__ unsigned long long bars[kWarpsPerBlock * S::DEPTH];
+    const int wid = threadIdx.x >> 5;
+    const int xs = (blockIdx.x * kWarpsPerBlock + wid) * S::OUT;
+    const int j0 = blockIdx.y * rows, j1 = min(j0 + rows, g.ny);
+    if (xs >= g.nx || j0 >= j1) return;   // whole warp
+    bool bad, timeout = false;
+    if (xs >= 2 && xs + 30 <= g.nx && j0 >= 2 && j1 + 3 <= g.ny) {
+        init_ring<S>(bars + wid * S::DEPTH);
+        unsigned base = 0;
+        bad = sweep_strip<P, 2, true>(g, c, k, &mf, &mu, B, smem + wid * (S::DEPTH * S::SLOT), bars + wid * S::DEPTH,
+                                      base, xs, j0, j1, timeout, 0);
+    } else {
+        bad = pair_strip<P, true>(g, c, k, A, B, xs, j0, j1);
+    }
     if (timeout) atomicOr(flag, kFlagTimeout);
     if (__any_sync(0xffffffffu, bad) && (threadIdx.x & 31) == 0) atomicOr(flag, kFlagNonfinite);
 }
@@ -392,9 +431,40 @@ cudaError_t encode(CUtensorMap* m, CUtensorMapDataType type, int elem, void* bas
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// Rows per chunk.  Tall chunks recompute fewer rows around them; short ones
+// end more often, so that the boundary launches beside the sweep find room
+// on the SMs, and fill the last wave.  Measured, us a step: K = 4 FP32 2047
+// x 1533 41.8 / 43.0 / 35.6 / 46.1 with 32 / 64 / 96 / 128 rows, 8192^2
+// 601 / 578 / 576 / 578; K = 2 FP16 2047 x 1533 48.1 / 49.2 / 71.1 with 16 /
+// 32 / 64 rows, 4096^2 204 / 201 / -, BFP13 4096^2 206 / 201 / 211.
+// Below 6 M points a K = 2 launch is a few waves of blocks: the height of 16 .. 32
+// rows whose waves cost least, a chunk costing its rows and 8 around them
+// (1024^2 BF16: 16 rows are 640 blocks on 608 places). free: places left to the
+// boundary launches beside the sweep, in tenths.
+int sweep2_rows(const Geo& g, int blocks_x, int height, int per_sm, int free) {
+    if ((long long)g.nx * g.ny >= (6ll << 20)) return 32;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return 16;
+    }
+    const long long places = std::max(1, sms * per_sm * (10 - free) / 10);
+    int rows = 16;
+    long long best = 0;
+    for (int r = 16; r <= 32; r += 2) {
+        const long long blocks = (long long)blocks_x * ((height + r - 1) / r);
+        const long long cost = (blocks + places - 1) / places * (r + 8);
+        if (best == 0 || cost < best) {
+            best = cost;
+            rows = r;
+        }
+    }
+    return rows;
+}
+
 }  // namespace
 
-template <typename P, int K>
+template <typename P, int K, bool EXACT>
 cudaError_t launch_sweep(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, View<P> B, unsigned* flag,
                          cudaStream_t st) {
     using S = Sweep<P, K>;
@@ -402,20 +472,32 @@ cudaError_t launch_sweep(const Geo& g, const Consts& c, const KCof<P>& k, View<P
     cudaError_t e = encode(&mf, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, A.f, g, S::PLANES, S::BOX);
     if (e == cudaSuccess) e = encode(&mu, CU_TENSOR_MAP_DATA_TYPE_UINT64, 8, A.u, g, 4, S::OUT);
     if (e != cudaSuccess) return e;
-    auto kern = sweep_kernel<P, K, S::MINB>;
+    auto kern = sweep_kernel<P, K, S::MINB, EXACT>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
     if (e != cudaSuccess) return e;
     const int strips = (g.nx - S::DEEP + S::OUT - 1) / S::OUT;
     const int height = g.ny - 2 * S::DEEP, blocks_x = (strips + kWarpsPerBlock - 1) / kWarpsPerBlock;
-    // Rows per chunk.  Tall chunks recompute fewer rows around them; short ones
-    // end more often, so that the boundary launches beside the sweep find room
-    // on the SMs, and fill the last wave.  Measured, us a step: K = 4 FP32 2047
-    // x 1533 41.8 / 43.0 / 35.6 / 46.1 with 32 / 64 / 96 / 128 rows, 8192^2
-    // 601 / 578 / 576 / 578; K = 2 FP16 2047 x 1533 48.1 / 49.2 / 71.1 with 16 /
-    // 32 / 64 rows, 4096^2 204 / 201 / -, BFP13 4096^2 206 / 201 / 211.
-    const int rows = K == 4 ? 96 : (long long)g.nx * g.ny < (6ll << 20) ? 16 : 32;
+    const int rows = K == 4 ? 96 : sweep2_rows(g, blocks_x, height, S::MINB, 1);
     const dim3 grid(blocks_x, (height + rows - 1) / rows);
     kern<<<grid, 32 * kWarpsPerBlock, S::kSmem, st>>>(g, c, k, mf, mu, B, flag, rows);
+    return cudaGetLastError();
+}
+
+template <typename P>
+cudaError_t launch_sweep_periodic(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, View<P> B, unsigned* flag,
+                                  cudaStream_t st) {
+    using S = Sweep<P, 2>;
+    CUtensorMap mf, mu;
+    cudaError_t e = encode(&mf, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, A.f, g, S::PLANES, S::BOX);
+    if (e == cudaSuccess) e = encode(&mu, CU_TENSOR_MAP_DATA_TYPE_UINT64, 8, A.u, g, 4, S::OUT);
+    if (e != cudaSuccess) return e;
+    auto kern = sweep_periodic_kernel<P, 4>;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
+    if (e != cudaSuccess) return e;
+    const int strips = (g.nx + S::OUT - 1) / S::OUT, blocks_x = (strips + kWarpsPerBlock - 1) / kWarpsPerBlock;
+    const int rows = sweep2_rows(g, blocks_x, g.ny, 4, 0);
+    const dim3 grid(blocks_x, (g.ny + rows - 1) / rows);
+    kern<<<grid, 32 * kWarpsPerBlock, S::kSmem, st>>>(g, c, k, mf, mu, A, B, flag, rows);
     return cudaGetLastError();
 }
 
@@ -454,8 +536,12 @@ cudaError_t launch_sweep_batch(const DomDesc<P>* dd, const SweepMaps* maps, cons
 }
 
 #define LBPS_INSTANTIATE(P)                                                                                       \
-    template cudaError_t launch_sweep<P, 2>(const Geo&, const Consts&, const KCof<P>&, View<P>, View<P>, unsigned*, \
-                                            cudaStream_t);                                                        \
+    template cudaError_t launch_sweep<P, 2, false>(const Geo&, const Consts&, const KCof<P>&, View<P>, View<P>,   \
+                                                   unsigned*, cudaStream_t);                                      \
+    template cudaError_t launch_sweep<P, 2, true>(const Geo&, const Consts&, const KCof<P>&, View<P>, View<P>,    \
+                                                  unsigned*, cudaStream_t);                                       \
+    template cudaError_t launch_sweep_periodic<P>(const Geo&, const Consts&, const KCof<P>&, View<P>, View<P>,    \
+                                                  unsigned*, cudaStream_t);                                       \
     template cudaError_t make_sweep_maps<P>(const Geo&, View<P>, View<P>, SweepMaps*);                            \
     template cudaError_t launch_sweep_batch<P>(const DomDesc<P>*, const SweepMaps*, const PairTask*, int,         \
                                                const BndTask*, int, unsigned*, cudaStream_t);
@@ -464,8 +550,8 @@ LBPS_INSTANTIATE(PopDirect<float>)
 LBPS_INSTANTIATE(PopNeq16<__nv_bfloat16>)
 LBPS_INSTANTIATE(PopNeq16<__half>)
 LBPS_INSTANTIATE(PopBfp13)
-template cudaError_t launch_sweep<PopDirect<float>, 4>(const Geo&, const Consts&, const KC<float>&,
-                                                       View<PopDirect<float>>, View<PopDirect<float>>, unsigned*,
-                                                       cudaStream_t);
+template cudaError_t launch_sweep<PopDirect<float>, 4, false>(const Geo&, const Consts&, const KC<float>&,
+                                                              View<PopDirect<float>>, View<PopDirect<float>>,
+                                                              unsigned*, cudaStream_t);
 
 }  // namespace lbps

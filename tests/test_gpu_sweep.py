@@ -1,4 +1,6 @@
-"""Four time steps per sweep (FP32 lattices of 3 M points and more) against
+"""Sweeps of several steps.  Exact sweeps of two (mid-size lattices) against
+single launches (a lattice whose launch shape was set takes those): the same
+bits.  Four time steps per sweep (FP32 lattices of 3 M points and more) against
 single steps: the populations and step counts are the same bits, u and du/dt
 agree up to the rounding of the composed Newmark update (one FP32 rounding of
 the acceleration sums per pair of steps: 1e-7 of the field's largest magnitude
@@ -53,3 +55,46 @@ def test_four_steps_per_sweep_equal_single_steps(L, size, chunks, sync):
         else:
             err = float((got[k] - want[k]).abs().max()) / float(want[k].abs().max())
             assert err <= 1e-7, (size, k, err)
+
+
+@pytest.mark.parametrize("storage", ["f32", "f16", "bf16", "bfp13"])
+@pytest.mark.parametrize("size", [(64, 7900), (7843, 65), (740, 701), (1003, 997)])
+@pytest.mark.parametrize("kw", [dict(), dict(periodic_x=True, periodic_y=True), dict(sync_every=5),
+                                dict(sync_every=5, periodic_x=True, periodic_y=True)])
+def test_exact_sweeps_equal_single_launches(L, storage, size, kw):
+    """500000 points and more, strips of 28 columns and chunks of 16 .. 32 rows
+    with every kind of remainder, seams of periodic axes, odd step counts,
+    synchronisation points inside pairs."""
+    lats = []
+    for separate in (False, True):
+        lat = L.Lattice.rectangle(*size, 1.5, 1.0, (2, 1, 1, 2), np.linspace(-2e-4, 2e-4, 8), a0_phi=0.99,
+                                  storage=storage, **kw)
+        if separate:
+            L.lbps_set_tuning(lat._h, 2, 8)
+        y, x = (torch.arange(n, dtype=torch.float64, device="cuda") for n in (size[1], size[0]))
+        u = [1e-3 * torch.sin(a * x)[None, :] * torch.cos(b * y)[:, None] for a, b in ((0.05, 0.03), (0.02, 0.07))]
+        lat.init(*u, *(1e-2 * q.flip(0).contiguous() for q in u))
+        lats.append(lat.step(1).step(9).step(34))
+    assert lats[0].check() == 0 and lats[0].steps == lats[1].steps == 44
+    for k in FIELDS:
+        assert torch.equal(lats[0].read_device(k), lats[1].read_device(k)), k
+    for lat in lats:
+        lat.close()
+
+
+def test_exact_sweeps_and_the_switch(L):
+    """Turning sweeps off frees the scratch copy and keeps the bits; turning
+    them on takes over from exact ones."""
+    out = []
+    for switch in ((), (0,), (1, 0)):
+        lat = L.Lattice.rectangle(800, 700, 1.5, 1.0, (2, 1, 1, 2), np.zeros(8), a0_phi=0.99)
+        u = W.pulse_displacement(800, 700, 300.0, 400.0, 40.0, 1e-3, "rotation")
+        lat.init(*u).step(6)
+        for on in switch:
+            L.lbps_set_step_pairs(lat._h, on)
+            assert L.lbps_step_pairs(lat._h) == on
+        lat.step(7)
+        out.append([lat.read(k) for k in FIELDS])
+        lat.close()
+    for other in out[1:]:
+        assert all(np.array_equal(a, b) for a, b in zip(out[0], other))
