@@ -1365,14 +1365,17 @@ int lbps_energy(lbps_lattice* lat, double out[3]) {
     lbps::NvtxRange nvtx("lbps_energy");
     if (!lat || !out) return LBPS_ERR_INVALID;
     if (!lat->initialised) return LBPS_ERR_STATE;
-    double n[2][4];
-    for (int q = 0; q < 2; ++q) {
-        int rc = lbps_norms(lat, q == 0 ? LBPS_KINETIC_ENERGY : LBPS_STRAIN_ENERGY, nullptr, n[q]);
-        if (rc != LBPS_OK) return rc;
-    }
+    double n[2];
+    cudaError_t e = lbps::with_policy(lat->p.storage, [&](auto pol) {
+        using P = decltype(pol);
+        return lbps::launch_energy<P>(lat->L.g, lat->c, lat->view<P>(lat->cur), lat->partials(), lat->out4(), lat->st);
+    });
+    if (e == cudaSuccess) e = cudaMemcpyAsync(n, lat->out4(), sizeof(n), cudaMemcpyDeviceToHost, lat->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(lat->st);
+    if (e != cudaSuccess) return LBPS_ERR_CUDA;
     const double area = lat->p.dh * lat->p.dh;
-    out[0] = n[0][2] * area;
-    out[1] = n[1][2] * area;
+    out[0] = n[0] * area;
+    out[1] = n[1] * area;
     out[2] = out[0] + out[1];
     return LBPS_OK;
 }

@@ -206,15 +206,6 @@ __device__ __forceinline__ double add_rn(double a, double b) { return __dadd_rn(
 __device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
 
-// One-dimensional second-order difference stencil at index i of n points:
-// central where both neighbours exist (or wrap), one-sided three-point at a
-// non-periodic end.  Offsets and weights (to be scaled by 1/(2 dh)).
-struct Sten {
-    int n;
-    int d[3];
-    double w[3];
-};
-
 // Is (i, j) (wrapped along periodic axes) a point of the body?
 __device__ __forceinline__ bool body_at(const Geo& g, int i, int j) {
     if (i < 0 || i >= g.nx) {
@@ -228,68 +219,42 @@ __device__ __forceinline__ bool body_at(const Geo& g, int i, int j) {
     return !g.general || LBPS_LDG(&g.type[(size_t)j * g.px + i]) != VOID;
 }
 
-__device__ __forceinline__ Sten stencil(int i, int n, int periodic) {
-    Sten s;
-    if (periodic || (i > 0 && i < n - 1)) {
-        s.n = 2; s.d[0] = -1; s.w[0] = -1.0; s.d[1] = 1; s.w[1] = 1.0; s.d[2] = 0; s.w[2] = 0.0;
-    } else if (i == 0) {
-        s.n = 3; s.d[0] = 0; s.w[0] = -3.0; s.d[1] = 1; s.w[1] = 4.0; s.d[2] = 2; s.w[2] = -1.0;
-    } else {
-        s.n = 3; s.d[0] = 0; s.w[0] = 3.0; s.d[1] = -1; s.w[1] = -4.0; s.d[2] = -2; s.w[2] = 1.0;
+// Difference stencil (DIFF_*, reading R4) at (i, j) along (dx, dy): central
+// where both neighbours are in the body (for a rectangle: inside it, or wrapped),
+// else one-sided three-point towards it (for a general geometry its existence
+// is checked at creation).
+__device__ __forceinline__ int diff_kind(const Geo& g, int i, int j, int dx, int dy) {
+    if (!g.general) {
+        const int q = dx ? i : j, n = dx ? g.nx : g.ny;
+        if (dx ? g.periodic_x : g.periodic_y) return DIFF_CENTRAL;
+        return q == 0 ? DIFF_FORWARD : q == n - 1 ? DIFF_BACKWARD : DIFF_CENTRAL;
     }
-    return s;
-}
-
-// The same choice from the node types (general geometry, reading R14):
-// central where both neighbours along (dx, dy) are in the body, else
-// one-sided towards the body (its existence is checked at creation).
-__device__ __forceinline__ Sten stencil_g(const Geo& g, int i, int j, int dx, int dy) {
-    Sten s;
     const bool hp = body_at(g, i + dx, j + dy), hm = body_at(g, i - dx, j - dy);
-    if (hp && hm) {
-        s.n = 2; s.d[0] = -1; s.w[0] = -1.0; s.d[1] = 1; s.w[1] = 1.0; s.d[2] = 0; s.w[2] = 0.0;
-    } else if (hp) {
-        s.n = 3; s.d[0] = 0; s.w[0] = -3.0; s.d[1] = 1; s.w[1] = 4.0; s.d[2] = 2; s.w[2] = -1.0;
-    } else {
-        s.n = 3; s.d[0] = 0; s.w[0] = 3.0; s.d[1] = -1; s.w[1] = -4.0; s.d[2] = -2; s.w[2] = 1.0;
-    }
-    return s;
+    return hp && hm ? DIFF_CENTRAL : hp ? DIFF_FORWARD : DIFF_BACKWARD;
 }
 
-__device__ __forceinline__ Sten stencil_x(const Geo& G, int i, int j) {
-    return G.general ? stencil_g(G, i, j, 1, 0) : stencil(i, G.nx, G.periodic_x);
-}
-__device__ __forceinline__ Sten stencil_y(const Geo& G, int i, int j) {
-    return G.general ? stencil_g(G, i, j, 0, 1) : stencil(j, G.ny, G.periodic_y);
+// Unscaled difference of p along an axis: stencil `kind` at index i of n
+// points `stride` elements apart.
+__device__ __forceinline__ double diff3(const double* p, int kind, int i, int n, ptrdiff_t stride) {
+    if (kind == DIFF_CENTRAL)
+        return sub_rn(LBPS_LD(p + (wrap(i + 1, n) - i) * stride), LBPS_LD(p + (wrap(i - 1, n) - i) * stride));
+    const int s = kind == DIFF_FORWARD ? 1 : -1;
+    const double u0 = LBPS_LD(p), u1 = LBPS_LD(p + (wrap(i + s, n) - i) * stride),
+                 u2 = LBPS_LD(p + (wrap(i + 2 * s, n) - i) * stride);
+    return s > 0 ? fma_rn(-1.0, u2, fma_rn(4.0, u1, mul_rn(-3.0, u0)))
+                 : fma_rn(1.0, u2, fma_rn(-4.0, u1, mul_rn(3.0, u0)));
 }
 
 // d/dx and d/dy of a FP64 array with row stride `stride` (reading of the
 // paper's "second order accurate finite differences", Sec. 3.1.2).
-// (A central difference, weights -1 and 1, is one subtraction: the same
-// bits as the weighted sum, fewer FP64 operations.)
-__device__ inline double ddx(const double* __restrict__ g, size_t stride, int i, int j, const Geo& G,
-                             double inv2h) {
-    Sten s = stencil_x(G, i, j);
-    const double* r = g + (size_t)j * stride;
-    double acc = 0.0;
-    if (s.n == 2)
-        acc = sub_rn(LBPS_LD(&r[wrap(i + 1, G.nx)]), LBPS_LD(&r[wrap(i - 1, G.nx)]));
-    else
-        for (int q = 0; q < s.n; ++q) acc = fma_rn(s.w[q], LBPS_LD(&r[wrap(i + s.d[q], G.nx)]), acc);
-    return mul_rn(acc, inv2h);
+__device__ __forceinline__ double ddx(const double* __restrict__ g, size_t stride, int i, int j, const Geo& G,
+                                      double inv2h) {
+    return mul_rn(diff3(g + (size_t)j * stride + i, diff_kind(G, i, j, 1, 0), i, G.nx, 1), inv2h);
 }
 
-__device__ inline double ddy(const double* __restrict__ g, size_t stride, int i, int j, const Geo& G,
-                             double inv2h) {
-    Sten s = stencil_y(G, i, j);
-    double acc = 0.0;
-    if (s.n == 2)
-        acc = sub_rn(LBPS_LD(&g[(size_t)wrap(j + 1, G.ny) * stride + i]),
-                     LBPS_LD(&g[(size_t)wrap(j - 1, G.ny) * stride + i]));
-    else
-        for (int q = 0; q < s.n; ++q)
-            acc = fma_rn(s.w[q], LBPS_LD(&g[(size_t)wrap(j + s.d[q], G.ny) * stride + i]), acc);
-    return mul_rn(acc, inv2h);
+__device__ __forceinline__ double ddy(const double* __restrict__ g, size_t stride, int i, int j, const Geo& G,
+                                      double inv2h) {
+    return mul_rn(diff3(g + (size_t)j * stride + i, diff_kind(G, i, j, 0, 1), j, G.ny, (ptrdiff_t)stride), inv2h);
 }
 
 // FP32 -> FP64 exactly by integer operations only (the conversion
@@ -471,9 +436,10 @@ struct PopDirect {
         }
     }
     // The same equilibria stored at p.
+    template <typename J>
     __device__ __forceinline__ static void store_eq_point(T* __restrict__ f, size_t plane, size_t p, const Consts& c,
-                                                          const double (&sv)[2], const double (&jx)[2],
-                                                          const double (&jy)[2], const KC<T>& k) {
+                                                          const double (&sv)[2], const J (&jx)[2], const J (&jy)[2],
+                                                          const KC<T>& k) {
         Raw r;
         eq_raw(p, c, sv, jx, jy, k, r);
         store_raw(f, plane, p, r);
@@ -731,10 +697,10 @@ struct PopNeq16 {
         r.w[1] = w;
     }
     // The same equilibria stored at p, each packed word written once.
+    template <typename J>
     __device__ __forceinline__ static void store_eq_point(float* __restrict__ f, size_t plane, size_t p,
-                                                          const Consts& c, const double (&sv)[2],
-                                                          const double (&jx)[2], const double (&jy)[2],
-                                                          const KC<float>& k) {
+                                                          const Consts& c, const double (&sv)[2], const J (&jx)[2],
+                                                          const J (&jy)[2], const KC<float>& k) {
         Raw r;
         eq_raw(p, c, sv, jx, jy, k, r);
         store_raw(f, plane, p, r);
@@ -960,10 +926,10 @@ struct PopBfp13 {
             r.w[s] = bfp13_encode(dev, dev);
         }
     }
+    template <typename J>
     __device__ __forceinline__ static void store_eq_point(float* __restrict__ f, size_t plane, size_t p,
-                                                          const Consts& c, const double (&sv)[2],
-                                                          const double (&jx)[2], const double (&jy)[2],
-                                                          const KC<float>& k) {
+                                                          const Consts& c, const double (&sv)[2], const J (&jx)[2],
+                                                          const J (&jy)[2], const KC<float>& k) {
         Raw r;
         eq_raw(p, c, sv, jx, jy, k, r);
         store_raw(f, plane, p, r);

@@ -60,8 +60,16 @@ __global__ void init_kernel(Geo g, Consts c, KCof<P> k, View<P> A) {
     double vx = LBPS_LD(&A.u[2 * g.plane + p]), vy = LBPS_LD(&A.u[3 * g.plane + p]);
     // First moments from du/dt (J_phi = -v, J_psi = (-v_y, v_x)), in lattice
     // units Jbar = J dt / dh (c cancels: c^alpha . J / (2 c^2) = e_alpha . Jbar / 2).
+    // At rest (both +0) the products are known; skipping them and their
+    // conversions leaves 12 of 22 FP64 instructions (the kernel is bound by them).
+    const double sv[2] = {phi, psi};
+    if ((__double_as_longlong(vx) | __double_as_longlong(vy)) == 0) {
+        const typename P::V jx[2] = {-(typename P::V)0, -(typename P::V)0}, jy[2] = {-(typename P::V)0, (typename P::V)0};
+        P::store_eq_point(A.f, g.plane, p, c, sv, jx, jy, k);
+        return;
+    }
     double q = c.dt / c.dh;
-    const double sv[2] = {phi, psi}, jx[2] = {-vx * q, -vy * q}, jy[2] = {-vy * q, vx * q};
+    const double jx[2] = {-vx * q, -vy * q}, jy[2] = {-vy * q, vx * q};
     P::store_eq_point(A.f, g.plane, p, c, sv, jx, jy, k);
 }
 
@@ -86,8 +94,8 @@ __global__ void finite_check_kernel(Geo g, const double* __restrict__ u, int pla
 // smaller by c_s / c_d).  Maximum over the lattice into *out (FP32 bits of a
 // non-negative value, which order like unsigned integers).
 __global__ void scale_probe_kernel(Geo g, Consts c, const double* __restrict__ u, double sq, unsigned* out) {
-    __shared__ float sh[256];
-    int t = threadIdx.y * blockDim.x + threadIdx.x;
+    __shared__ unsigned sh[8];
+    const int lane = threadIdx.x;   // a block is 8 warps
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     int j = blockIdx.y * blockDim.y + threadIdx.y;
     float est = 0.0f;
@@ -97,17 +105,21 @@ __global__ void scale_probe_kernel(Geo g, Consts c, const double* __restrict__ u
         size_t p = (size_t)j * g.px + i;
         double phi = ddx(ux, g.px, i, j, g, c.inv2h) + ddy(uy, g.px, i, j, g, c.inv2h);
         double psi = ddx(uy, g.px, i, j, g, c.inv2h) - ddy(ux, g.px, i, j, g, c.inv2h);
-        double v = fabs(LBPS_LD(&u[2 * g.plane + p])) + fabs(LBPS_LD(&u[3 * g.plane + p]));
-        double e = sq * fmax(fabs(phi), fabs(psi)) + v * c.dt / c.dh;
+        const double vx = LBPS_LD(&u[2 * g.plane + p]), vy = LBPS_LD(&u[3 * g.plane + p]);
+        double e = sq * fmax(fabs(phi), fabs(psi));
+        // at rest there is nothing to add (and no FP64 division)
+        if (((__double_as_longlong(vx) | __double_as_longlong(vy)) << 1) != 0)
+            e += (fabs(vx) + fabs(vy)) * c.dt / c.dh;
         est = isfinite(e) ? (float)e : 3.0e38f;
     }
-    sh[t] = est;
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(est));
+    if (lane == 0) sh[threadIdx.y] = m;
     __syncthreads();
-    for (int w = 128; w > 0; w >>= 1) {
-        if (t < w) sh[t] = fmaxf(sh[t], sh[t + w]);
-        __syncthreads();
+    if (lane == 0 && threadIdx.y == 0) {
+        unsigned best = 0;
+        for (int q = 0; q < 8; ++q) best = max(best, sh[q]);
+        atomicMax(out, best);
     }
-    if (t == 0) atomicMax(out, __float_as_uint(sh[0]));
 }
 
 // ------------------------------------------------------------- boundary
@@ -431,13 +443,12 @@ __global__ void sync_kernel(Geo g, Consts c, KCof<P> k, View<P> A) {
     double s[2];
     s[0] = ddx(ux, g.px, i, j, g, c.inv2h) + ddy(uy, g.px, i, j, g, c.inv2h);
     s[1] = ddx(uy, g.px, i, j, g, c.inv2h) - ddy(ux, g.px, i, j, g, c.inv2h);
-    double jx[2], jy[2];
+    V jx[2], jy[2];   // first moments in the arithmetic type of the storage
     for (int set = 0; set < 2; ++set) {
         V f[5];
         P::load5(A.f, g.plane, p, set, k, f);
-        // first moments in the arithmetic type of the storage
-        jx[set] = (double)sub_rn(f[1], f[3]);
-        jy[set] = (double)sub_rn(f[2], f[4]);
+        jx[set] = sub_rn(f[1], f[3]);
+        jy[set] = sub_rn(f[2], f[4]);
     }
     P::store_eq_point(A.f, g.plane, p, c, s, jx, jy, k);
 }
@@ -575,6 +586,63 @@ __global__ void __launch_bounds__(kNormThreads) norms_final_kernel(const double*
     }
     if (threadIdx.x == 0)
         for (int q = 0; q < 4; ++q) out[q] = sh[q][0];
+}
+
+// Both energies in one pass: per block the sums over body points of |du/dt|^2,
+// tr(d)^2, d_xx^2 + d_yy^2 and (d_xy + d_yx)^2 with the unscaled differences d
+// of u; the constants come in at the end (13 FP64 instructions a point instead
+// of 32 for the two densities; bound by them).
+template <typename P>
+__global__ void __launch_bounds__(kNormThreads) energy_partial_kernel(Geo g, View<P> A, double* partials) {
+    __shared__ double sh[4][kNormThreads];
+    const double* ux = A.u;
+    const double* uy = A.u + g.plane;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int j = blockIdx.x; j < g.ny; j += gridDim.x)
+        for (int i = threadIdx.x; i < g.nx; i += kNormThreads) {
+            if (!body_at(g, i, j)) continue;
+            const size_t p = (size_t)j * g.px + i;
+            const double vx = LBPS_LD(&A.u[2 * g.plane + p]), vy = LBPS_LD(&A.u[3 * g.plane + p]);
+            const int kx = diff_kind(g, i, j, 1, 0), ky = diff_kind(g, i, j, 0, 1);
+            const double exx = diff3(ux + p, kx, i, g.nx, 1), eyx = diff3(uy + p, kx, i, g.nx, 1);
+            const double exy = diff3(ux + p, ky, j, g.ny, g.px), eyy = diff3(uy + p, ky, j, g.ny, g.px);
+            const double tr = add_rn(exx, eyy), sh2 = add_rn(exy, eyx);
+            s[0] = fma_rn(vx, vx, fma_rn(vy, vy, s[0]));
+            s[1] = fma_rn(tr, tr, s[1]);
+            s[2] = fma_rn(exx, exx, fma_rn(eyy, eyy, s[2]));
+            s[3] = fma_rn(sh2, sh2, s[3]);
+        }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sh[q][threadIdx.x] = s[q];
+    __syncthreads();
+    for (int w = kNormThreads / 2; w > 0; w >>= 1) {
+        if (threadIdx.x < w)
+            for (int q = 0; q < 4; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x < 4) partials[(size_t)blockIdx.x * 4 + threadIdx.x] = sh[threadIdx.x][0];
+}
+
+// out = kinetic and strain energy per dh^2 (sums of the densities).
+__global__ void __launch_bounds__(kNormThreads) energy_final_kernel(Consts c, const double* partials, int nblk,
+                                                                    double* out) {
+    __shared__ double sh[4][kNormThreads];
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int b = threadIdx.x; b < nblk; b += kNormThreads)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s[q] += partials[(size_t)b * 4 + q];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sh[q][threadIdx.x] = s[q];
+    __syncthreads();
+    for (int w = kNormThreads / 2; w > 0; w >>= 1) {
+        if (threadIdx.x < w)
+            for (int q = 0; q < 4; ++q) sh[q][threadIdx.x] += sh[q][threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        out[0] = 0.5 * c.rho * sh[0][0];
+        out[1] = (0.5 * c.lam * sh[1][0] + c.mu * (sh[2][0] + 0.5 * sh[3][0])) * (c.inv2h * c.inv2h);
+    }
 }
 
 // Rows of a state copy to or from a caller buffer, 16 bytes per thread and
@@ -856,7 +924,16 @@ cudaError_t launch_norms(const Geo& g, const Consts& c, const KCof<P>& k, View<P
     return cudaGetLastError();
 }
 
+template <typename P>
+cudaError_t launch_energy(const Geo& g, const Consts& c, View<P> A, double* partials, double* out2, cudaStream_t st) {
+    const int nblk = std::min(g.ny, kNormBlocks);
+    energy_partial_kernel<P><<<nblk, kNormThreads, 0, st>>>(g, A, partials);
+    energy_final_kernel<<<1, kNormThreads, 0, st>>>(c, partials, nblk, out2);
+    return cudaGetLastError();
+}
+
 #define LBPS_INSTANTIATE(P)                                                                                   \
+    template cudaError_t launch_energy<P>(const Geo&, const Consts&, View<P>, double*, double*, cudaStream_t);   \
     template cudaError_t launch_init<P>(const Geo&, const Consts&, const KCof<P>&, View<P>, cudaStream_t);  \
     template cudaError_t launch_frame<P>(const Geo&, const Consts&, const KCof<P>&, View<P>, View<P>, unsigned*,  \
                                          cudaStream_t, int);                                                  \

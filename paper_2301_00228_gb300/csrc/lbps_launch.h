@@ -93,6 +93,11 @@ template <typename P>
 cudaError_t launch_norms(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, int field, const double* ref,
                          double* partials, double* out4, cudaStream_t st);
 
+// out2 = sums of the kinetic and the strain energy density over the body points
+// (scratch as launch_norms).
+template <typename P>
+cudaError_t launch_energy(const Geo& g, const Consts& c, View<P> A, double* partials, double* out2, cudaStream_t st);
+
 // ---- many steps in one launch (lbps_fused.cu)
 
 // Advances copy A (current) by `steps` time steps in one cooperative launch:

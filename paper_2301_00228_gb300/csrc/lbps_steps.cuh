@@ -54,18 +54,6 @@ __device__ __forceinline__ BPoint point_of(const Geo& g, const BNode* __restrict
     return p;
 }
 
-// Unscaled difference of p along an axis: stencil `kind` at index i of n
-// points `stride` elements apart.
-__device__ __forceinline__ double diff3(const double* p, int kind, int i, int n, ptrdiff_t stride) {
-    if (kind == DIFF_CENTRAL)
-        return sub_rn(LBPS_LD(p + (wrap(i + 1, n) - i) * stride), LBPS_LD(p + (wrap(i - 1, n) - i) * stride));
-    const int s = kind == DIFF_FORWARD ? 1 : -1;
-    const double u0 = LBPS_LD(p), u1 = LBPS_LD(p + (wrap(i + s, n) - i) * stride),
-                 u2 = LBPS_LD(p + (wrap(i + 2 * s, n) - i) * stride);
-    return s > 0 ? fma_rn(-1.0, u2, fma_rn(4.0, u1, mul_rn(-3.0, u0)))
-                 : fma_rn(1.0, u2, fma_rn(-4.0, u1, mul_rn(3.0, u0)));
-}
-
 // Differences of u at (i, j): xx = du_x/dx, yx = du_y/dx, xy = du_x/dy, yy = du_y/dy.
 struct Grad {
     double xx, yx, xy, yy;
