@@ -423,6 +423,7 @@ int lbps_batch_step(lbps_batch* b, int64_t n) {
     for (auto* l : b->lats) {
         l->steps += n;
         l->cur ^= flips;
+        l->flag_other = true;   // the batch's kernels set the device flag only
     }
     return LBPS_OK;
 }
@@ -515,6 +516,7 @@ int lbps_batch_tune(lbps_batch* b, int32_t repeats, int32_t* variant, int32_t* r
     if (!b || repeats < 1) return LBPS_ERR_INVALID;
     int rc = refresh(b);
     if (rc != LBPS_OK) return rc;
+    for (auto* l : b->lats) l->flag_other = true;   // the timed steps may set the device flag
     const int rows_c[] = {8, 16, 32, 64, 128};
     const int var_c[] = {0, 1, 2, 4, 5, 6};
     cudaEvent_t e0, e1;

@@ -42,7 +42,8 @@ __device__ __forceinline__ void add_release(unsigned* p, unsigned x) {
 // the last block arrives and the low bits are as before.  phase: the top bit
 // before the barrier, flipped here.  Returns false in every thread of a block
 // whose wait ran out.
-__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned& phase, unsigned* flag, int* alive) {
+__device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned& phase, unsigned* flag, unsigned* host,
+                                             int* alive) {
     __syncthreads();
     if (threadIdx.x == 0) {
         add_release(bar, blockIdx.x == 0 ? 0x80000000u - (gridDim.x - 1u) : 1u);
@@ -50,6 +51,7 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned& phase, uns
         while (((poll_acquire(bar) ^ phase) & 0x80000000u) == 0u && ++polls < kMaxPolls) {}
         if (polls >= kMaxPolls) {
             atomicOr(flag, kFlagTimeout);
+            if (host) *(volatile unsigned*)(host + 1) = 1u;
             *alive = 0;
         }
     }
@@ -63,8 +65,8 @@ __device__ __forceinline__ bool grid_barrier(unsigned* bar, unsigned& phase, uns
 template <typename P, int THREADS, int UVD, bool GEN>
 __global__ void __launch_bounds__(THREADS, 1) fused_kernel(Geo g, Consts c, KCof<P> k, View<P> A0, View<P> B0,
                                                            const BNode* __restrict__ bn, int nb, unsigned* flag,
-                                                           unsigned long long* tstep, unsigned* bar, int steps,
-                                                           int rows) {
+                                                           unsigned long long* tstep, unsigned* bar,
+                                                           unsigned* host, int steps, int rows) {
     __shared__ int alive;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, warps = blockDim.x >> 5;
     const int G = gridDim.x, cta = blockIdx.x;
@@ -109,7 +111,7 @@ __global__ void __launch_bounds__(THREADS, 1) fused_kernel(Geo g, Consts c, KCof
             }
         }
         if (nb > 0) {
-            if (!grid_barrier(bar, phase, flag, &alive)) return;
+            if (!grid_barrier(bar, phase, flag, host, &alive)) return;
             for (int t = wid; t < nbp; t += warps) {
                 const int b = 32 * (b0 + (t >> 1)) + lane;
                 if (b >= nb) continue;
@@ -119,16 +121,19 @@ __global__ void __launch_bounds__(THREADS, 1) fused_kernel(Geo g, Consts c, KCof
                     bad |= boundary_reset<P>(g, c, k, A, B, table, nb, b);
             }
             if (P::kSplitStream) {
-                if (!grid_barrier(bar, phase, flag, &alive)) return;
+                if (!grid_barrier(bar, phase, flag, host, &alive)) return;
                 for (int t = b0 + wid; t < b1; t += warps) {
                     const int b = 32 * t + lane;
                     if (b < nb) boundary_stream_y(g, c, k, A, B, table, b);
                 }
             }
         }
-        if (s + 1 < steps && !grid_barrier(bar, phase, flag, &alive)) return;
+        if (s + 1 < steps && !grid_barrier(bar, phase, flag, host, &alive)) return;
     }
-    if (bad) atomicOr(flag, kFlagNonfinite);
+    if (bad) {
+        atomicOr(flag, kFlagNonfinite);
+        if (host) *(volatile unsigned*)host = 1u;
+    }
     // every block has read the counter before its first barrier
     if (nb > 0 && cta == 0 && threadIdx.x == 0) LBPS_ST(tstep, n0 + (unsigned)steps);
 }
@@ -137,7 +142,7 @@ __global__ void __launch_bounds__(THREADS, 1) fused_kernel(Geo g, Consts c, KCof
 
 template <typename P>
 cudaError_t launch_fused(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, View<P> B, const BNode* bn,
-                         int nb, unsigned* flag, unsigned long long* tstep, unsigned* bar, int steps,
+                         int nb, unsigned* flag, unsigned long long* tstep, unsigned* bar, unsigned* host, int steps,
                          cudaStream_t st) {
     // FP64 storage needs 128 registers a thread.  The others: 16 warps per SM
     // up to 2^19 points, where the phases are short (389 x 1171: 15.7 us a step
@@ -172,7 +177,7 @@ cudaError_t launch_fused(const Geo& g, const Consts& c, const KCof<P>& k, View<P
     Geo ga = g;
     Consts ca = c;
     KCof<P> ka = k;
-    void* args[] = {&ga, &ca, &ka, &A, &B, &bn, &nb, &flag, &tstep, &bar, &steps, &rows};
+    void* args[] = {&ga, &ca, &ka, &A, &B, &bn, &nb, &flag, &tstep, &bar, &host, &steps, &rows};
     return cudaLaunchCooperativeKernel(kern, dim3(blocks), dim3(32 * warps), args, 0, st);
 }
 
@@ -185,7 +190,7 @@ int fused_check_report(unsigned long long out[2]) { return read_check_report(out
 
 #define LBPS_INSTANTIATE(P)                                                                                      \
     template cudaError_t launch_fused<P>(const Geo&, const Consts&, const KCof<P>&, View<P>, View<P>, const BNode*, \
-                                         int, unsigned*, unsigned long long*, unsigned*, int, cudaStream_t);
+                                         int, unsigned*, unsigned long long*, unsigned*, unsigned*, int, cudaStream_t);
 
 LBPS_INSTANTIATE(PopDirect<float>)
 LBPS_INSTANTIATE(PopDirect<double>)

@@ -104,13 +104,15 @@ cudaError_t launch_energy(const Geo& g, const Consts& c, View<P> A, double* part
 // the odd steps write B, the even ones A.  Every step is the interior strips
 // and the boundary Newmark pass, a barrier over the grid, the boundary reset
 // and another barrier.  bar: the barrier's word (zero at creation).  A wait
-// that runs out sets kFlagTimeout in *flag.  Returns
+// that runs out sets kFlagTimeout in *flag.  host (null or mapped host memory):
+// word 0 is set to 1 with kFlagNonfinite, word 1 with kFlagTimeout, so that a
+// caller who has waited for the stream need not copy *flag.  Returns
 // cudaErrorCooperativeLaunchTooLarge (nothing launched) where the grid cannot
 // be resident at once.
 constexpr unsigned kFlagNonfinite = 1u, kFlagTimeout = 2u;
 template <typename P>
 cudaError_t launch_fused(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, View<P> B, const BNode* bn,
-                         int nb, unsigned* flag, unsigned long long* tstep, unsigned* bar, int steps,
+                         int nb, unsigned* flag, unsigned long long* tstep, unsigned* bar, unsigned* host, int steps,
                          cudaStream_t st);
 #ifdef LBPS_CHECKED
 cudaError_t fused_check_table(const char* const* los, const char* const* his, int n);

@@ -98,6 +98,11 @@ struct lbps_lattice {
     lbps::Tuning tuning;  // bulk-kernel launch shape
     bool tuned = false;   // set by the caller (lbps_set_tuning): the steps then run in that shape
     bool fused_off = false;  // the device refused a cooperative launch
+    // mapped host words that launch_fused sets beside the flag (null: none), and
+    // whether anything else may have set the flag since the initialisation
+    unsigned* host_flag = nullptr;
+    bool flag_other = true;
+    bool captured = false;   // steps were captured by the caller: replays may set the flag any time
     int last_cuda = 0;    // cudaError_t of the last failing CUDA call
     int64_t steps;
     bool initialised;

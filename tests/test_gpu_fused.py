@@ -89,3 +89,38 @@ def test_fused_on_two_streams(L):
     got = run([torch.cuda.Stream(), torch.cuda.Stream()])
     for a, b in zip(got, want):
         assert all(np.array_equal(x, y) for x, y in zip(a, b))
+
+
+def test_nonfinite_is_seen_on_every_path(L):
+    """The check after many-step launches alone reads host words instead of the
+    device flag; it must see what a launch sets, keep it, forget it at the next
+    initialisation, and see the flag of other paths (a batch, launches of a set
+    shape, a loaded state's steps)."""
+    u = W.pulse_displacement(64, 48, 20.0, 20.0, 4.0, 1e-3)
+    bad = [a * 1e300 for a in u]
+
+    def raises(lat, n=4):
+        with pytest.raises(L.LbpsError) as e:
+            lat.step(n)
+        assert e.value.code == L.LBPS_ERR_NONFINITE
+        assert lat.check() == L.LBPS_ERR_NONFINITE
+
+    lat = lattice(L, 64, 48)
+    lat.step(3)
+    saved = lat.save_state()
+    lat.init(*bad)
+    raises(lat)
+    lat.init(*u).step(5)                       # forgotten
+    assert lat.check() == 0
+    lat.init(*bad)
+    b = L.Batch([lat])
+    b.step(4)                                  # set by the batch, read by the lattice
+    assert b.check() == L.LBPS_ERR_NONFINITE and lat.check() == L.LBPS_ERR_NONFINITE
+    b.close()
+    lat.init(*u).step(2)
+    lat.load_state(saved).step(3)
+    assert lat.check() == 0
+    L.lbps_set_tuning(lat._h, 2, 8)
+    lat.init(*bad)
+    raises(lat)
+    lat.close()
