@@ -180,12 +180,12 @@ def measured_peaks():
 
 def kernel_source_hash():
     """sha256 (first 16 hex digits) of the code the normal build compiles
-    from the kernel sources: the three files without // comments, blank lines
+    from the kernel sources: the four files without // comments, blank lines
     and the branches only the range-checked build compiles (#ifdef
     LBPS_CHECKED), so editing a comment or the checked build keeps the
     recorded ncu traffic valid and editing the normal build's code does not."""
     code = []
-    for name in ("lbps_kernels.cu", "lbps_steps.cuh", "lbps_device.cuh"):
+    for name in ("lbps_kernels.cu", "lbps_sweep.cu", "lbps_steps.cuh", "lbps_device.cuh"):
         text = (ROOT / "paper_2301_00228_gb300" / "csrc" / name).read_text()
         stack = []  # per open #if: True while its lines belong to the checked build only
         for line in text.splitlines():

@@ -351,7 +351,8 @@ int lbps_batch_graph_steps(const lbps_batch* b);
  * each lattice's scratch copy, the first step's reset, a persistent kernel
  * for the second step on the points 1..2 from the edges and its Newmark pass,
  * and the second step's reset.  Every lattice gets the same bits as when it
- * takes two steps per sweep on its own.  Turning it on calls
+ * takes two steps per sweep on its own (FP32 lattices that take four differ from
+ * that by the rounding of u, du/dt at the points 3 and 4 from the edges).  Turning it on calls
  * lbps_set_step_pairs(lat, 1) for every lattice (a scratch state copy each;
  * its error code if that fails) and returns LBPS_ERR_INVALID, changing
  * nothing, if a lattice is not a rectangle without periodic axes and at least
@@ -497,7 +498,7 @@ int lbps_set_graph_steps(lbps_lattice* lat, int32_t k);
  * The sweep runs beside a chain
  * of boundary and frame launches on a second stream of greatest priority.
  * It pays from about 800^2 points (FP32, us a step against single steps:
- * 8192^2 576 / 1563; 4096^2 159 / 400; 2047 x 1533 36 / 85). */
+ * 8192^2 567 / 1562; 4096^2 162 / 400; 2047 x 1533 36 / 85). */
 int lbps_set_step_pairs(lbps_lattice* lat, int32_t on);
 
 /* 1 if lbps_step takes two steps per sweep on this lattice (turned on and

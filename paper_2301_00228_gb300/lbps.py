@@ -358,10 +358,11 @@ def lbps_set_origin(h, row0):
 
 # ---- convenience wrapper --------------------------------------------------
 
-# From about this many points two time steps per sweep are faster than one
-# (FP32, lbps_step with CUDA graphs: 8192^2 72.1 against 43.2 GLUPS, 4096^2
-# 63.1 against 41.9, 2048^2 46.6 against 37.1, 1536^2 32.5 against 33.6;
-# FP64 storage is bound by its FP64 population arithmetic, so not there).
+# From this many points the binding turns sweeps of several steps on (FP32: four
+# steps per sweep; us a step against single ones, 8192^2 567 / 1562, 4096^2 162 /
+# 400); smaller lattices take exact sweeps or many steps in one launch by
+# themselves.  FP64 storage is bound by its FP64 population arithmetic, so not
+# there.
 PAIRS_AUTO_POINTS = 3_000_000
 
 
@@ -371,7 +372,7 @@ class Lattice:
     def __init__(self, nx, ny, lam, mu, rho=1.0, dh=1.0, a0_phi=0.9999, periodic_x=False, periodic_y=False,
                  node_type=None, bc_value=None, bc_feq_mode=0, sync_every=0, storage="f32", pop_scale_exp=0,
                  stream=None, cell=None, bc_j_mode=0, step_pairs="auto"):
-        """step_pairs: two time steps per sweep (lbps_set_step_pairs); "auto"
+        """step_pairs: two or four time steps per sweep (lbps_set_step_pairs); "auto"
         turns them on for lattices of at least PAIRS_AUTO_POINTS points where
         they apply (rectangles without periodic axes) and the storage is not
         FP64, where they are faster (the scratch state copy they need is
