@@ -476,14 +476,17 @@ bool exact_wanted(const lbps_lattice* lat) {
 }
 
 // The scratch copy of a lattice's sweeps, zeroed once: parts of it the frame
-// passes read but do not use then hold finite values.
+// passes read but do not use then hold finite values.  Cleared on the lattice's
+// own stream: the legacy default stream does not order a clear before the
+// first sweep on a non-blocking one.
 int make_scratch(lbps_lattice* lat, char** out) {
     void* x = nullptr;
     if (cudaMalloc(&x, lat->L.copy_bytes) != cudaSuccess) {
         cudaGetLastError();
         return LBPS_ERR_OOM;
     }
-    if (cudaMemset(x, 0, lat->L.copy_bytes) != cudaSuccess ||
+    if (cudaMemsetAsync(x, 0, lat->L.copy_bytes, lat->st) != cudaSuccess ||
+        cudaStreamSynchronize(lat->st) != cudaSuccess ||
         lbps::set_check_range(x, lat->L.copy_bytes, lat->st) != cudaSuccess) {
         cudaFree(x);
         cudaGetLastError();

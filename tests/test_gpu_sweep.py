@@ -98,3 +98,26 @@ def test_exact_sweeps_and_the_switch(L):
         lat.close()
     for other in out[1:]:
         assert all(np.array_equal(a, b) for a, b in zip(out[0], other))
+
+
+@pytest.mark.parametrize("pairs", [False, True])
+def test_scratch_is_cleared_before_the_first_sweep(L, pairs):
+    """The first sweeps of a lattice on its own stream, the default stream busy
+    for longer than they take: clearing the scratch copy does not wait for it."""
+    out = []
+    a = torch.ones(8192, 8192, device="cuda")
+    for busy in (False, True):
+        lat = L.Lattice.rectangle(1200, 1100, 1.5, 1.0, (2, 1, 1, 2), np.zeros(8), a0_phi=0.99,
+                                  stream=torch.cuda.Stream())
+        lat.init(*W.pulse_displacement(1200, 1100, 300.0, 400.0, 40.0, 1e-3, "rotation"))
+        torch.cuda.synchronize()
+        if busy:
+            for _ in range(400):
+                a.mul_(1.0)
+        if pairs:
+            L.lbps_set_step_pairs(lat._h, 1)
+        lat.step(200)
+        torch.cuda.synchronize()
+        out.append([lat.read(k) for k in FIELDS])
+        lat.close()
+    assert all(np.array_equal(a, b) for a, b in zip(*out))
