@@ -62,6 +62,13 @@ __device__ __forceinline__ void tma_load(void* dst, const CUtensorMap* map, int 
         : "memory");
 }
 
+// Before the first use of a tensor map that lies in global memory (written by
+// the host): what was copied there is seen by the copies issued from here on,
+// not a map that an earlier launch used at the same address.
+__device__ __forceinline__ void acquire_map(const CUtensorMap* map) {
+    asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
+}
+
 template <typename P>
 constexpr bool kHashed = false;
 template <typename H>
@@ -364,7 +371,7 @@ __global__ void __launch_bounds__(128, 4) sweep_batch_kernel(const DomDesc<P>* _
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     init_ring<S>(bars + wid * S::DEPTH);
     unsigned base = 0;
-    int cached = -1;
+    int cached = -1, mapped = -1;   // the lattice of the descriptor, of the maps acquired last
     for (;;) {
         unsigned t = 0;
         if (lane == 0) t = atomicAdd(next, 1u);
@@ -395,6 +402,13 @@ __global__ void __launch_bounds__(128, 4) sweep_batch_kernel(const DomDesc<P>* _
         bool bad, timeout = false;
         if (tk.kind == kPairStrip) {
             const CUtensorMap* m = reinterpret_cast<const CUtensorMap*>(maps + tk.dom) + 2 * a;
+            if (tk.dom != mapped) {
+                if (lane == 0) {   // the lane that issues the copies
+                    acquire_map(m);
+                    acquire_map(m + 1);
+                }
+                mapped = tk.dom;
+            }
             bad = sweep_strip<P, 2>(d.g, d.c, d.k, m, m + 1, d.v[a ^ 1], smem + wid * (S::DEPTH * S::SLOT),
                                     bars + wid * S::DEPTH, base, tk.xs, tk.j0, tk.j1, timeout);
         } else if (tk.kind == kSideStrip) {
