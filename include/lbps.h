@@ -41,7 +41,8 @@ extern "C" {
 #define LBPS_ERR_NONFINITE (-4) /* the state became non-finite (instability)  */
 #define LBPS_ERR_TIMEOUT (-5)   /* a barrier inside a launch of many steps ran
                                    out (the blocks were not all running); the
-                                   state is undefined until the next init    */
+                                   lattice has no state (LBPS_ERR_STATE) until
+                                   the next init or lbps_state_load          */
 #define LBPS_ERR_STATE (-6)     /* call out of order (e.g. step before init)  */
 
 /* Node types of the boundary mask (Sec. 2, Fig. 1). */

@@ -850,14 +850,19 @@ int stage_u(lbps_lattice* lat, const double* ux0, const double* uy0, const doubl
     return LBPS_OK;
 }
 
+// Zeroes the flag and, beside it, the step counter and the barrier word of
+// launch_fused, and the flag's host words: before a new state.
+cudaError_t clear_flags(lbps_lattice* lat) {
+    cudaError_t e = cudaMemsetAsync(lat->flag(), 0, kAlign, lat->st);
+    if (e == cudaSuccess && lat->host_flag) e = cudaMemsetAsync(lat->host_flag, 0, 2 * sizeof(unsigned), lat->st);
+    return e;
+}
+
 // Make the staged copy current and initialise it: the initialisation kernel
 // (and the 16-bit scale choice before it).
 int init_staged(lbps_lattice* lat) {
     lat->cur ^= 1;
-    // the non-finite flag and, beside it, the step counter and the barrier word
-    if (cudaMemsetAsync(lat->flag(), 0, kAlign, lat->st) != cudaSuccess) return LBPS_ERR_CUDA;
-    if (lat->host_flag && cudaMemsetAsync(lat->host_flag, 0, 2 * sizeof(unsigned), lat->st) != cudaSuccess)
-        return LBPS_ERR_CUDA;
+    if (clear_flags(lat) != cudaSuccess) return LBPS_ERR_CUDA;
     lat->flag_other = lat->host_flag == nullptr || lat->captured;
     if (lat->neq16()) {
         int rc = choose_scale(lat);
@@ -1305,7 +1310,10 @@ int lbps_check(lbps_lattice* lat) {
         const volatile unsigned* h = lat->host_flag;
         flag = (h[0] ? lbps::kFlagNonfinite : 0u) | (h[1] ? lbps::kFlagTimeout : 0u);
     }
-    if (flag & lbps::kFlagTimeout) return LBPS_ERR_TIMEOUT;
+    if (flag & lbps::kFlagTimeout) {
+        lat->initialised = false;   // no state, and arrivals left in the barrier word: the next init or load clears it
+        return LBPS_ERR_TIMEOUT;
+    }
     return flag ? LBPS_ERR_NONFINITE : LBPS_OK;
 }
 
@@ -1486,9 +1494,10 @@ int lbps_state_load(lbps_lattice* lat, const void* src, size_t bytes) {
     cudaError_t e = cudaMemcpyAsync(lat->mem + lat->L.off_copy[0], static_cast<const char*>(src) + sizeof(h),
                                     lat->L.copy_bytes, cudaMemcpyDefault, lat->st);
     unsigned long long n = (unsigned long long)h.steps;
-    // the non-finite flag cleared, the device step counter set
+    // the flags and the barrier word cleared (a launch that timed out leaves
+    // arrivals in it), the device step counter set
     lat->flag_other = true;
-    if (e == cudaSuccess) e = cudaMemsetAsync(lat->flag(), 0, sizeof(unsigned), lat->st);
+    if (e == cudaSuccess) e = clear_flags(lat);
     if (e == cudaSuccess) e = cudaMemcpyAsync(lat->tstep(), &n, sizeof(n), cudaMemcpyHostToDevice, lat->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(lat->st);
     if (e != cudaSuccess) {

@@ -436,8 +436,13 @@ int lbps_batch_check(lbps_batch* b) {
         e = cudaMemcpyAsync(&flags[d], b->lats[d]->flag(), sizeof(unsigned), cudaMemcpyDeviceToHost, b->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
     if (e != cudaSuccess) return fail(b, e);
-    for (unsigned f : flags)
-        if (f & lbps::kFlagTimeout) return LBPS_ERR_TIMEOUT;
+    bool timeout = false;
+    for (size_t d = 0; d < flags.size(); ++d)
+        if (flags[d] & lbps::kFlagTimeout) {
+            b->lats[d]->initialised = false;   // as lbps_check
+            timeout = true;
+        }
+    if (timeout) return LBPS_ERR_TIMEOUT;
     for (unsigned f : flags)
         if (f) return LBPS_ERR_NONFINITE;
     return LBPS_OK;

@@ -91,10 +91,13 @@ __global__ void __launch_bounds__(THREADS, 1) fused_kernel(Geo g, Consts c, KCof
         table = sbn - 32 * b0;
     }
 #endif
-    if (threadIdx.x == 0) alive = 1;
+    // after a launch that timed out the barrier word holds arrivals of blocks
+    // that are gone: nothing runs until the next state clears it
+    if (threadIdx.x == 0) alive = (LBPS_LD(flag) & kFlagTimeout) == 0u;
     const unsigned long long n0 = LBPS_LD(tstep);
     unsigned phase = poll_acquire(bar);   // before this block's first arrival, so the top bit is the old one
     __syncthreads();
+    if (!alive) return;
     bool bad = false;
     for (int s = 0; s < steps; ++s) {
         const View<P> A = (s & 1) ? B0 : A0, B = (s & 1) ? A0 : B0;

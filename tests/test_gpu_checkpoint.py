@@ -103,3 +103,28 @@ def test_load_rejects_other_setup(L):
         assert e.value.code == L.LBPS_ERR_INVALID, q
     same_again = make(L, "f32", init=False).load_state(buf)
     assert same_again.steps == 3
+
+
+def test_load_clears_the_barrier_word(L):
+    """A launch that timed out leaves arrivals in the grid barrier's word (here
+    written there by hand, nothing in flight) and its flag set.  Launches before
+    the next state do nothing; a loaded state clears both and goes on with the
+    bits of an undisturbed lattice."""
+    a = make(L, "f32").step(20)
+    b = make(L, "f32").step(9)
+    saved = b.save_state()
+    staging = -(-min(5 * 45 * 38 * 8, 8 << 20) // 256) * 256
+    words = b._mem[b.nbytes - staging - 256:b.nbytes - staging].view(torch.int32)
+    w = words.cpu()
+    assert w[0] == 0 and w[2] == 9 and w[32] & 0x7fffffff == 0   # flag, step counter, barrier word
+    words[32] += 5
+    words[0] = 2
+    torch.cuda.synchronize()
+    before = b._mem.clone()
+    b.step_async(3)
+    torch.cuda.synchronize()
+    assert torch.equal(b._mem, before)
+    b.load_state(saved)
+    assert words[32] == 0 and words[0] == 0
+    b.step(11)
+    same(a, b, "after a timeout")
