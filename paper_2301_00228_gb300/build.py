@@ -32,6 +32,14 @@ def sources():
     return sorted(CSRC.glob("*.cu"))
 
 
+def flags() -> list[str]:
+    # -fmad=false: no compiler-chosen multiply-add contraction, so every kernel
+    # that evaluates a shared formula gets the same bits (the hot loops use
+    # explicit fused intrinsics where they want them).
+    return ARCH + ["-O3", "-lineinfo", "-std=c++17", "-fmad=false", "-Xcompiler", "-fPIC", "-I", str(INCLUDE),
+                   "-I", str(CSRC)]
+
+
 def _stale(outp: Path, deps) -> bool:
     if not outp.exists():
         return True
@@ -44,15 +52,11 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False, 
     kernel memory access range- and alignment-checked (LBPS_CHECKED)."""
     BUILD.mkdir(exist_ok=True)
     headers = list(CSRC.glob("*.cuh")) + list(CSRC.glob("*.h")) + list(INCLUDE.glob("*.h"))
-    # -fmad=false: no compiler-chosen multiply-add contraction, so every kernel
-    # that evaluates a shared formula gets the same bits (the hot loops use
-    # explicit fused intrinsics where they want them).
-    flags = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-fmad=false", "-Xcompiler", "-fPIC", "-I", str(INCLUDE),
-                    "-I", str(CSRC)]
+    opts = flags()
     if ptxas_info:
-        flags += ["-Xptxas", "-v"]
+        opts += ["-Xptxas", "-v"]
     if checked:
-        flags += ["-DLBPS_CHECKED"]
+        opts += ["-DLBPS_CHECKED"]
     lib = PKG / ("liblbps_checked.so" if checked else "liblbps.so")
     procs = []
     objs = []
@@ -60,7 +64,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False, 
         obj = BUILD / (src.stem + ("_checked" if checked else "") + ".o")
         objs.append(obj)
         if force or ptxas_info or _stale(obj, [src] + headers):
-            cmd = [nvcc()] + flags + ["-c", str(src), "-o", str(obj)]
+            cmd = [nvcc()] + opts + ["-c", str(src), "-o", str(obj)]
             if verbose:
                 print(" ".join(cmd), flush=True)
             procs.append((src, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))

@@ -27,7 +27,11 @@ namespace lbps {
 namespace {
 
 // Polls of an mbarrier before a warp gives up (a second or more).
-constexpr int kMaxWaits = 1 << 22;
+#ifndef LBPS_SWEEP_POLLS
+#define LBPS_SWEEP_POLLS (1 << 22)
+#endif
+constexpr int kMaxWaits = LBPS_SWEEP_POLLS;
+constexpr int kDrainWaits = 1 << 22;   // for each copy still under way then
 
 __device__ __forceinline__ unsigned smem_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -39,8 +43,10 @@ __device__ __forceinline__ void mbar_expect(unsigned long long* bar, unsigned by
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
 }
 
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity) {
-    for (int n = 0; n < kMaxWaits; ++n) {
+// The same answer in every lane of the warp.
+__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity, int polls) {
+#pragma unroll 1
+    for (int n = 0; n < polls; ++n) {
         unsigned ok;
         asm volatile(
             "{\n.reg .pred p;\n"
@@ -49,7 +55,7 @@ __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned pari
             : "=r"(ok)
             : "r"(smem_addr(bar)), "r"(parity)
             : "memory");
-        if (ok) return true;
+        if (__all_sync(0xffffffffu, ok)) return true;
     }
     return false;
 }
@@ -133,8 +139,17 @@ __device__ __forceinline__ bool sweep_strip(const Geo& g, const Consts& c, const
 
     // pair q of this strip is pair base + q of the warp's ring
     auto slot_of = [&](int q) { return (int)((base + (unsigned)q) % (unsigned)S::DEPTH); };
+    // a warp gives up as a whole (its lanes shuffle), and only when the copies
+    // it issued have landed or run out too (after the return the block's shared
+    // memory may be another block's)
+    auto landed = [&](int q, int polls) {
+        return mbar_wait(bars + slot_of(q), ((base + (unsigned)q) / (unsigned)S::DEPTH) & 1u, polls);
+    };
     auto arrived = [&](int q) {
-        return mbar_wait(bars + slot_of(q), ((base + (unsigned)q) / (unsigned)S::DEPTH) & 1u);
+        if (landed(q, kMaxWaits)) return true;
+#pragma unroll 1
+        for (int p = q; p < q + S::DEPTH && p < ngroups; ++p) landed(p, kDrainWaits);
+        return false;
     };
     auto issue = [&](int q) {   // lane 0
         char* slot = ring + slot_of(q) * S::SLOT;
