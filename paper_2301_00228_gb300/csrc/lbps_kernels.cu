@@ -755,10 +755,21 @@ cudaError_t launch_copy_segments(const CopySegs& s, cudaStream_t st) {
     return cudaGetLastError();
 }
 
+#ifdef LBPS_CHECKED
+namespace {
+// the table of live blocks, mirrored on the host and uploaded whole
+std::vector<std::pair<const char*, const char*>> ranges;
+}  // namespace
+
+bool check_live(const void* p, size_t bytes) {
+    const char* lo = static_cast<const char*>(p);
+    return std::any_of(ranges.begin(), ranges.end(),
+                       [&](const auto& r) { return lo >= r.first && lo + bytes <= r.second; });
+}
+#endif
+
 cudaError_t set_check_range(const void* base, size_t bytes, cudaStream_t st) {
 #ifdef LBPS_CHECKED
-    // the table of live blocks, mirrored on the host and uploaded whole
-    static std::vector<std::pair<const char*, const char*>> ranges;
     const char* lo = static_cast<const char*>(base);
     ranges.erase(std::remove_if(ranges.begin(), ranges.end(), [&](const auto& r) { return r.first == lo; }),
                  ranges.end());
@@ -775,6 +786,7 @@ cudaError_t set_check_range(const void* base, size_t bytes, cudaStream_t st) {
     cudaError_t e = cudaStreamSynchronize(st);  // no kernel in flight sees a half-written table
     if (e == cudaSuccess) e = upload_check_table(los.data(), his.data(), n);
     if (e == cudaSuccess) e = fused_check_table(los.data(), his.data(), n);
+    if (e == cudaSuccess) e = sweep_check_table(los.data(), his.data(), n);
     return e;
 #else
     (void)base;
@@ -789,6 +801,7 @@ int check_report(unsigned long long out[2]) {
     if (cudaDeviceSynchronize() != cudaSuccess) return -1;
     int rc = read_check_report(out);
     if (rc > 0 && out[0] == 0) rc = fused_check_report(out);
+    if (rc > 0 && out[0] == 0) rc = sweep_check_report(out);
     return rc;
 #else
     out[0] = out[1] = 0;

@@ -115,8 +115,13 @@ cudaError_t launch_fused(const Geo& g, const Consts& c, const KCof<P>& k, View<P
                          int nb, unsigned* flag, unsigned long long* tstep, unsigned* bar, unsigned* host, int steps,
                          cudaStream_t st);
 #ifdef LBPS_CHECKED
+// The other units' copies of the table of live blocks and of the record
+// (set_check_range, check_report), and whether [p, p + bytes) lies in one block.
 cudaError_t fused_check_table(const char* const* los, const char* const* his, int n);
 int fused_check_report(unsigned long long out[2]);
+cudaError_t sweep_check_table(const char* const* los, const char* const* his, int n);
+int sweep_check_report(unsigned long long out[2]);
+bool check_live(const void* p, size_t bytes);
 #endif
 
 // ---- batches: many lattices advanced by one launch of each kernel per step

@@ -450,6 +450,10 @@ cudaError_t encode(CUtensorMap* m, CUtensorMapDataType type, int elem, void* bas
     cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
     if (e != cudaSuccess) return e;
     if (found != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
+#ifdef LBPS_CHECKED
+    // the copies read only inside the map (and zeros beyond it), the map only inside a live block
+    if (!check_live(base, (size_t)planes * g.plane * elem)) return cudaErrorInvalidValue;
+#endif
     const cuuint64_t dims[3] = {(cuuint64_t)g.px, (cuuint64_t)g.ny, (cuuint64_t)planes};
     const cuuint64_t strides[2] = {(cuuint64_t)g.px * elem, (cuuint64_t)g.plane * elem};
     const cuuint32_t box[3] = {(cuuint32_t)box_x, 2, (cuuint32_t)planes}, one[3] = {1, 1, 1};
@@ -563,6 +567,13 @@ cudaError_t launch_sweep_batch(const DomDesc<P>* dd, const SweepMaps* maps, cons
     kern<<<blocks, 32 * kWarpsPerBlock, S::kSmem, st>>>(dd, maps, tasks, ntasks, btasks, parity, next);
     return cudaGetLastError();
 }
+
+#ifdef LBPS_CHECKED
+cudaError_t sweep_check_table(const char* const* los, const char* const* his, int n) {
+    return upload_check_table(los, his, n);
+}
+int sweep_check_report(unsigned long long out[2]) { return read_check_report(out); }
+#endif
 
 #define LBPS_INSTANTIATE(P)                                                                                       \
     template cudaError_t launch_sweep<P, 2, false>(const Geo&, const Consts&, const KCof<P>&, View<P>, View<P>,   \
