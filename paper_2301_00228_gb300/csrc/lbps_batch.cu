@@ -369,6 +369,9 @@ int lbps_batch_step(lbps_batch* b, int64_t n) {
     lbps::NvtxRange nvtx("lbps_batch_step");
     if (!b || n < 0) return LBPS_ERR_INVALID;
     if (n == 0) return LBPS_OK;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    const bool capturing = cudaStreamIsCapturing(b->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    if (capturing) cudaGetLastError();
     // start after the work already queued on the lattices' own streams
     for (auto* l : b->lats) {
         if (l->st == b->st) continue;
@@ -424,6 +427,7 @@ int lbps_batch_step(lbps_batch* b, int64_t n) {
         l->steps += n;
         l->cur ^= flips;
         l->flag_other = true;   // the batch's kernels set the device flag only
+        l->captured |= capturing;   // as a replay of these steps does at any time
     }
     return LBPS_OK;
 }
