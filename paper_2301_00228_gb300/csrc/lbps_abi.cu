@@ -1217,7 +1217,8 @@ int lbps_step_async(lbps_lattice* lat, int64_t n) {
     if (!lat || n < 0) return LBPS_ERR_INVALID;
     if (!lat->initialised) return LBPS_ERR_STATE;
     const int l = lat->p.sync_every;
-    // a capturing stream gets the plain launches of single steps
+    // a capturing stream gets the plain launches of single steps: a graph cannot
+    // be launched into a capture, nor memory for scratch allocated
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool capturing = cudaStreamIsCapturing(lat->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
     if (capturing) {
@@ -1252,9 +1253,9 @@ int lbps_step_async(lbps_lattice* lat, int64_t n) {
         // graph_k steps at once from a graph, else 2, unless per-kernel timing
         // is on or a synchronisation falls after one of the first k - 1 of them
         int k = 0;
-        const bool quad = n - s >= 4 && quad_ok(lat) && !(l > 0 && l - lat->steps % l < 4);
+        const bool quad = n - s >= 4 && !capturing && quad_ok(lat) && !(l > 0 && l - lat->steps % l < 4);
         for (int c : {lat->graph_k, quad ? 0 : 2}) {
-            if (k == 0 && c > 0 && n - s >= c && !lat->prof && !(l > 0 && l - lat->steps % l < c)) k = c;
+            if (k == 0 && c > 0 && n - s >= c && !capturing && !lat->prof && !(l > 0 && l - lat->steps % l < c)) k = c;
         }
         if (k > 0) {
             cudaGraphExec_t g = nullptr;
@@ -1273,11 +1274,11 @@ int lbps_step_async(lbps_lattice* lat, int64_t n) {
             int rc = run_quad(lat);
             if (rc != LBPS_OK) return rc;
             s += 4;
-        } else if (n - s >= 2 && periodic_pairs(lat) && !(l > 0 && (lat->steps + 1) % l == 0)) {
+        } else if (n - s >= 2 && !capturing && periodic_pairs(lat) && !(l > 0 && (lat->steps + 1) % l == 0)) {
             int rc = run_periodic_pair(lat);
             if (rc != LBPS_OK) return rc;
             s += 2;
-        } else if (n - s >= 2 && pair_ok(lat) && !(l > 0 && (lat->steps + 1) % l == 0)) {
+        } else if (n - s >= 2 && !capturing && pair_ok(lat) && !(l > 0 && (lat->steps + 1) % l == 0)) {
             int rc = run_pair(lat);
             if (rc != LBPS_OK) return rc;
             s += 2;

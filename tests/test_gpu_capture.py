@@ -50,3 +50,37 @@ def test_replayed_batch_steps_reach_the_lattice_check(L):
     b.close()
     for lat in lats:
         lat.close()
+
+
+@pytest.mark.parametrize("size,kw", [((300, 200), {}), ((1030, 520), {}), ((300, 200), dict(step_pairs=True)),
+                                     ((1030, 520), dict(periodic_x=True, periodic_y=True))])
+@pytest.mark.parametrize("warm", [0, 4])
+def test_captured_steps_are_single_steps(L, size, kw, warm):
+    """lbps_step_async into a capture, on lattices that otherwise take many
+    steps a launch or sweeps: one step replayed once and four steps replayed
+    three times give the bits of uncaptured single launches."""
+    s = torch.cuda.Stream()
+
+    def start(single):
+        lat, u = lattice(L, *size, s, **({} if single else kw), **({k: v for k, v in kw.items() if single and
+                                                                     k != "step_pairs"}))
+        if single:
+            L.lbps_set_tuning(lat._h, 2, 8)
+        lat.set_load(L.LBPS_NEUMANN, 20 * lat.dt, 45 * lat.dt)
+        return lat.init(*u).step(warm)
+
+    for n, replays in ((1, 1), (4, 3)):
+        lat, want = start(False), start(True)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=s):
+            lat.step_async(n)
+        for _ in range(replays):
+            g.replay()
+        torch.cuda.synchronize()
+        want.step(n * replays)
+        assert lat.check() == 0
+        for k in ("f_phi", "f_psi") + (() if "step_pairs" in kw and warm else ("ux", "uy", "vx", "vy")):
+            assert np.array_equal(lat.read(k), want.read(k)), (n, k)
+        lat.close()
+        want.close()
