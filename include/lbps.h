@@ -235,13 +235,10 @@ int lbps_init_device(lbps_lattice* lat, const double* d_ux0, const double* d_uy0
  * (Eq. LBE, LBE_mod), and every sync_every-th step the synchronisation of
  * Sec. 3.2.  Enqueues the work, then waits for the stream and returns
  * LBPS_ERR_NONFINITE if any update produced a non-finite value.
- * Rectangles without periodic axes of 500000 to 3000000 points (64 a side or
- * more, not FP64 storage) take their steps two per sweep with the bits of
- * single steps; the first call of two steps or more allocates a scratch copy
- * for that (cudaMalloc, the size of one state copy; freed at lbps_destroy, or
- * by lbps_set_step_pairs(lat, 0), after which the lattice keeps to launches
- * without scratch; without the memory it does so by itself).  Fully periodic
- * lattices from 500000 points on do the same without scratch. */
+ * Allocates no device memory: what sweeps of several steps need beside the
+ * lattice's block is allocated by lbps_set_sweeps.  Fully periodic lattices
+ * from 500000 points on (64 a side or more, not FP64 storage) take their steps
+ * two per sweep, with the bits of single steps and without scratch. */
 int lbps_step(lbps_lattice* lat, int64_t n);
 
 /* As lbps_step without the final wait and check (use lbps_check later). */
@@ -354,8 +351,10 @@ int lbps_batch_graph_steps(const lbps_batch* b);
  * and the second step's reset.  Every lattice gets the same bits as when it
  * takes two steps per sweep on its own (FP32 lattices that take four differ from
  * that by the rounding of u, du/dt at the points 3 and 4 from the edges).  Turning it on calls
- * lbps_set_step_pairs(lat, 1) for every lattice (a scratch state copy each;
- * its error code if that fails) and returns LBPS_ERR_INVALID, changing
+ * lbps_set_sweeps(lat, LBPS_SWEEPS_TWO) for every lattice that has no composed
+ * sweeps (a scratch state copy each; its error code if that fails; a lattice
+ * whose copy is given up afterwards makes lbps_batch_step return
+ * LBPS_ERR_STATE) and returns LBPS_ERR_INVALID, changing
  * nothing, if a lattice is not a rectangle without periodic axes and at least
  * 16 points a side.  lbps_batch_step then runs n / 2 pairs and an odd last
  * step as a single step; no CUDA graph (the launches are few per pair).
@@ -501,6 +500,34 @@ int lbps_set_graph_steps(lbps_lattice* lat, int32_t k);
  * It pays from about 800^2 points (FP32, us a step against single steps:
  * 8192^2 567 / 1562; 4096^2 162 / 400; 2047 x 1533 36 / 85). */
 int lbps_set_step_pairs(lbps_lattice* lat, int32_t on);
+
+/* The sweeps lbps_step takes on a lattice, and the scratch state copies (beside
+ * the lattice's block, cudaMalloc'd here, freed by another kind or at
+ * lbps_destroy; at most lbps_state_bytes / 2 each) they need:
+ *   NONE   (the default) no sweeps, no scratch.
+ *   EXACT  two steps per sweep, u and du/dt integrated step by step: the bits
+ *          of single steps, between synchronisations.  One copy.  Not FP64
+ *          storage.  Lattices whose launch shape was set or that record
+ *          per-kernel timing keep to single steps.
+ *   TWO    as lbps_set_step_pairs, two steps per sweep.  One copy.
+ *   FOUR   as lbps_set_step_pairs, four steps per sweep.  Two copies.  FP32
+ *          storage, 64 points a side or more.
+ *   AUTO   the fastest by size (lbps_default_sweeps), with less scratch or none
+ *          where the memory cannot be had.
+ * LBPS_ERR_INVALID where the kind does not apply (sweeps apply to rectangles
+ * without periodic axes, 16 points a side or more; AUTO is then NONE),
+ * LBPS_ERR_OOM, with the sweeps as before, without the memory.
+ * lbps_sweeps: the kind in use.  lbps_default_sweeps: the kind AUTO takes for
+ * a rectangle of these parameters (or an error code): EXACT from 500000 points,
+ * FOUR or TWO from 3000000. */
+#define LBPS_SWEEPS_AUTO (-1)
+#define LBPS_SWEEPS_NONE 0
+#define LBPS_SWEEPS_EXACT 1
+#define LBPS_SWEEPS_TWO 2
+#define LBPS_SWEEPS_FOUR 3
+int lbps_set_sweeps(lbps_lattice* lat, int32_t kind);
+int lbps_sweeps(const lbps_lattice* lat);
+int lbps_default_sweeps(const lbps_params* params);
 
 /* 1 if lbps_step takes two steps per sweep on this lattice (turned on and
  * applicable), else 0. */

@@ -443,39 +443,49 @@ int run_step(lbps_lattice* lat) {
 }
 
 // Sweeps of several steps apply to rectangles without periodic axes, at least
-// 16 points a side.
+// 16 points a side, and run beside a boundary chain on the side stream.
 bool sweeps_apply(const lbps_lattice* lat) {
     const lbps::Geo& g = lat->L.g;
-    return lat->side && !g.general && !g.periodic_x && !g.periodic_y && g.nx >= 16 && g.ny >= 16 && lat->L.nb > 0;
+    return !g.general && !g.periodic_x && !g.periodic_y && g.nx >= 16 && g.ny >= 16 && lat->L.nb > 0;
 }
 
-// Two steps per sweep, with the scratch copy allocated: turned on by the
-// caller, or exact ones (below) unless the caller asked for single steps'
-// timing or launch shape.
+// Two steps per sweep, with the scratch copy allocated: composed ones, or exact
+// ones (below) unless the caller asked for single steps' timing or launch
+// shape.
 bool pair_ok(const lbps_lattice* lat) {
-    return lat->xmem && sweeps_apply(lat) && (lat->pairs || (lat->exact && !lat->prof && !lat->tuned));
+    return lat->xmem && lat->side && sweeps_apply(lat) &&
+           (lat->pairs || (lat->exact && !lat->prof && !lat->tuned));
 }
 
 // Single steps as sweeps of two whose u, du/dt take the steps one by one: the
-// bits of single steps, half their traffic.  Up to the size from which the
-// binding turns on the caller's sweeps; below, the boundary chain (about 29 us
+// bits of single steps, half their traffic.  By default up to the size from
+// which the composed ones are; below, the boundary chain (about 29 us
 // per pair) is longer than many steps in one launch.  Measured, us a step
 // against single steps: 700 x 500 14.6 / 13.4, 800^2 15.4 / 19.7 (BF16 18.7 /
 // 22.2), 1024^2 21.0 / 27.4 (BF16 24.7 / 33.9, BFP13 23.9 / 38.0), 1600^2 46 / 74;
 // periodic 512^2 10.3 / 8.9, 768^2 12.0 / 14.7, 1024^2 17.7 / 27.4, 2048^2 59 /
 // 103.
 constexpr int64_t kExactMinPoints = 500000;
-constexpr int64_t kExactMaxPoints = 3000000;
 constexpr int32_t kExactMinSide = 64;
+// Composed sweeps by default from here; four steps per sweep in FP32 storage
+// (the others' codecs bind four steps: BFP13 4096^2 263 us a step against 201
+// with two; FP32 2047 x 1533: 35.6 us a step against 54 with two).
+constexpr int64_t kPairsMinPoints = 3000000;
+constexpr int32_t kQuadMinSide = 64;
 
-bool exact_wanted(const lbps_lattice* lat) {
-    const int64_t points = (int64_t)lat->L.g.nx * lat->L.g.ny;
-    return sweeps_apply(lat) && !lat->pairs && !lat->exact && !lat->no_scratch && !lat->prof && !lat->tuned &&
-           lat->p.storage != LBPS_STORAGE_F64 && points >= kExactMinPoints && points < kExactMaxPoints &&
-           std::min(lat->L.g.nx, lat->L.g.ny) >= kExactMinSide;
+// The sweeps that are fastest on a rectangle of these parameters
+// (LBPS_SWEEPS_*).
+int default_sweeps(const lbps_params& p) {
+    const int64_t points = (int64_t)p.nx * p.ny;
+    const int32_t side = std::min(p.nx, p.ny);
+    if (p.periodic_x || p.periodic_y || p.storage == LBPS_STORAGE_F64 || side < 16) return LBPS_SWEEPS_NONE;
+    if (points >= kPairsMinPoints)
+        return p.storage == LBPS_STORAGE_F32 && side >= kQuadMinSide ? LBPS_SWEEPS_FOUR : LBPS_SWEEPS_TWO;
+    return points >= kExactMinPoints && side >= kExactMinSide && p.sync_every != 1 ? LBPS_SWEEPS_EXACT
+                                                                                   : LBPS_SWEEPS_NONE;
 }
 
-// The scratch copy of a lattice's sweeps, zeroed once: parts of it the frame
+// A scratch copy of a lattice's sweeps, zeroed once: parts of it the frame
 // passes read but do not use then hold finite values.  Cleared on the lattice's
 // own stream: the legacy default stream does not order a clear before the
 // first sweep on a non-blocking one.
@@ -496,13 +506,34 @@ int make_scratch(lbps_lattice* lat, char** out) {
     return LBPS_OK;
 }
 
-void drop_scratch(lbps_lattice* lat) {
-    for (char** x : {&lat->ymem, &lat->xmem}) {
-        if (!*x) continue;
-        lbps::set_check_range(*x, 0, lat->st);
-        cudaFree(*x);
-        *x = nullptr;
+void drop_scratch(lbps_lattice* lat, int keep = 0) {
+    char** x[2] = {&lat->xmem, &lat->ymem};
+    for (int q = 1; q >= keep; --q) {
+        if (!*x[q]) continue;
+        lbps::set_check_range(*x[q], 0, lat->st);
+        cudaFree(*x[q]);
+        *x[q] = nullptr;
     }
+}
+
+// Holds `copies` scratch copies (0 .. 2) for exact or composed sweeps.  An
+// allocation that fails leaves everything as it was.
+int hold_scratch(lbps_lattice* lat, int copies, bool exact, bool pairs) {
+    const int held = (lat->xmem != nullptr) + (lat->ymem != nullptr);
+    if (held == copies && lat->exact == exact && lat->pairs == pairs) return LBPS_OK;
+    if (cudaStreamSynchronize(lat->st) != cudaSuccess) return LBPS_ERR_CUDA;
+    for (int q = held; q < copies; ++q) {
+        const int rc = make_scratch(lat, q == 0 ? &lat->xmem : &lat->ymem);
+        if (rc != LBPS_OK) {
+            drop_scratch(lat, held);
+            return rc;
+        }
+    }
+    drop_scratch(lat, copies);
+    lat->exact = exact;
+    lat->pairs = pairs;
+    lat->gen += 1;  // captured step graphs hold the other kind of step
+    return LBPS_OK;
 }
 
 // Lattices periodic in both axes take exact sweeps of every point, without
@@ -571,12 +602,6 @@ int run_pair(lbps_lattice* lat) {
     lat->steps += 2;
     return LBPS_OK;
 }
-
-// Four steps per sweep: FP32 storage (the others' codecs bind four steps: BFP13
-// 4096^2 263 us a step against 201 with two) from the size at which the binding
-// turns sweeps on by itself (2047 x 1533: 35.6 us a step against 54 with two).
-constexpr int64_t kQuadMinPoints = 3000000;
-constexpr int32_t kQuadMinSide = 64;
 
 bool quad_ok(const lbps_lattice* lat) { return lat->ymem && lat->pairs && pair_ok(lat); }
 
@@ -1218,20 +1243,12 @@ int lbps_step_async(lbps_lattice* lat, int64_t n) {
     if (!lat->initialised) return LBPS_ERR_STATE;
     const int l = lat->p.sync_every;
     // a capturing stream gets the plain launches of single steps: a graph cannot
-    // be launched into a capture, nor memory for scratch allocated
+    // be launched into a capture
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool capturing = cudaStreamIsCapturing(lat->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
     if (capturing) {
         cudaGetLastError();
         lat->captured = true;
-    }
-    if (n >= 2 && l != 1 && !capturing && exact_wanted(lat)) {
-        // once per lattice; without the memory it keeps to single steps
-        if (make_scratch(lat, &lat->xmem) == LBPS_OK)
-            lat->exact = true;
-        else
-            lat->no_scratch = true;
-        lat->gen += 1;
     }
     bool fused = !capturing && fused_ok(lat);
     for (int64_t s = 0; s < n;) {
@@ -1551,29 +1568,44 @@ int lbps_set_tuning(lbps_lattice* lat, int32_t variant, int32_t rows_per_warp) {
     return LBPS_OK;
 }
 
+int lbps_default_sweeps(const lbps_params* params) {
+    const int rc = validate_params(params);
+    return rc == LBPS_OK ? default_sweeps(*params) : rc;
+}
+
+int lbps_sweeps(const lbps_lattice* lat) {
+    if (!lat) return LBPS_ERR_INVALID;
+    if (!lat->xmem || !sweeps_apply(lat)) return LBPS_SWEEPS_NONE;
+    return lat->exact ? LBPS_SWEEPS_EXACT : lat->ymem ? LBPS_SWEEPS_FOUR : LBPS_SWEEPS_TWO;
+}
+
+int lbps_set_sweeps(lbps_lattice* lat, int32_t kind) {
+    if (!lat || kind < LBPS_SWEEPS_AUTO || kind > LBPS_SWEEPS_FOUR) return LBPS_ERR_INVALID;
+    if (kind == LBPS_SWEEPS_AUTO) {
+        int k = lat->L.g.general ? LBPS_SWEEPS_NONE : default_sweeps(lat->p);
+        int rc = lbps_set_sweeps(lat, k);
+        if (rc == LBPS_ERR_OOM && k == LBPS_SWEEPS_FOUR) rc = lbps_set_sweeps(lat, LBPS_SWEEPS_TWO);
+        return rc == LBPS_ERR_OOM ? lbps_set_sweeps(lat, LBPS_SWEEPS_NONE) : rc;
+    }
+    if (kind != LBPS_SWEEPS_NONE && !sweeps_apply(lat)) return LBPS_ERR_INVALID;
+    if (kind == LBPS_SWEEPS_EXACT && lat->p.storage == LBPS_STORAGE_F64) return LBPS_ERR_INVALID;
+    if (kind == LBPS_SWEEPS_FOUR &&
+        (lat->p.storage != LBPS_STORAGE_F32 || std::min(lat->p.nx, lat->p.ny) < kQuadMinSide))
+        return LBPS_ERR_INVALID;
+    const int copies = kind == LBPS_SWEEPS_FOUR ? 2 : kind == LBPS_SWEEPS_NONE ? 0 : 1;
+    return hold_scratch(lat, copies, kind == LBPS_SWEEPS_EXACT, kind >= LBPS_SWEEPS_TWO);
+}
+
 int lbps_set_step_pairs(lbps_lattice* lat, int32_t on) {
     if (!lat || on < 0 || on > 1) return LBPS_ERR_INVALID;
-    if (on == 0) lat->no_scratch = true;   // no exact sweeps either: their scratch copy would come back
-    if ((on != 0) == lat->pairs && !(on == 0 && lat->xmem)) return LBPS_OK;
-    if (cudaStreamSynchronize(lat->st) != cudaSuccess) return LBPS_ERR_CUDA;
-    if (on) {
-        if (!lat->xmem) {
-            const int rc = make_scratch(lat, &lat->xmem);
-            if (rc != LBPS_OK) return rc;
-        }
-        // the second scratch copy of four steps per sweep; without it the
-        // lattice takes two
-        if (lat->p.storage == LBPS_STORAGE_F32 && (int64_t)lat->p.nx * lat->p.ny >= kQuadMinPoints &&
-            std::min(lat->p.nx, lat->p.ny) >= kQuadMinSide)
-            make_scratch(lat, &lat->ymem);
-        lat->pairs = true;
-    } else {
-        drop_scratch(lat);
-        lat->pairs = false;
-    }
-    lat->exact = false;
-    lat->gen += 1;  // captured step graphs hold the other kind of step
-    return LBPS_OK;
+    if (!on) return hold_scratch(lat, 0, false, false);
+    if (lat->pairs) return LBPS_OK;
+    // without memory for the second copy of four steps per sweep the lattice
+    // takes two
+    const bool four = sweeps_apply(lat) && lat->p.storage == LBPS_STORAGE_F32 &&
+                      (int64_t)lat->p.nx * lat->p.ny >= kPairsMinPoints && std::min(lat->p.nx, lat->p.ny) >= kQuadMinSide;
+    const int rc = hold_scratch(lat, four ? 2 : 1, false, true);
+    return rc == LBPS_ERR_OOM && four ? hold_scratch(lat, 1, false, true) : rc;
 }
 
 int lbps_step_pairs(const lbps_lattice* lat) {

@@ -368,6 +368,9 @@ int lbps_batch_set_tuning(lbps_batch* b, int32_t variant, int32_t rows_per_warp)
 int lbps_batch_step(lbps_batch* b, int64_t n) {
     lbps::NvtxRange nvtx("lbps_batch_step");
     if (!b || n < 0) return LBPS_ERR_INVALID;
+    if (b->pairs)
+        for (const auto* l : b->lats)
+            if (!l->xmem) return LBPS_ERR_STATE;   // its scratch copy was given up since
     if (n == 0) return LBPS_OK;
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     const bool capturing = cudaStreamIsCapturing(b->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
@@ -475,7 +478,8 @@ int lbps_batch_set_step_pairs(lbps_batch* b, int32_t on) {
             return LBPS_ERR_INVALID;
     }
     for (lbps_lattice* l : b->lats) {   // the scratch copy of each lattice
-        const int rc = lbps_set_step_pairs(l, 1);
+        // one scratch copy each (a second one only serves a lattice on its own)
+        const int rc = l->pairs ? LBPS_OK : lbps_set_sweeps(l, LBPS_SWEEPS_TWO);
         if (rc != LBPS_OK) return rc;
     }
     // the tensor maps of every lattice's copies; without them (FP64 storage, a

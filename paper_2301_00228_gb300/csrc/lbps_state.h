@@ -88,11 +88,10 @@ struct lbps_lattice {
     int cur;            // copy holding time t
     // sweeps of two steps: the scratch state copy that holds step n + 1 on the
     // boundary and the points up to 3 from it (cudaMalloc'd, copy_bytes).
-    // pairs: turned on by the caller (lbps_set_step_pairs); exact: by
-    // lbps_step on a mid-size lattice, for the bits of single steps;
-    // no_scratch: the caller turned sweeps off, or there was no memory.
+    // pairs: composed sweeps; exact: those with the bits of single steps
+    // (lbps_set_sweeps).
     char* xmem = nullptr;
-    bool pairs = false, exact = false, no_scratch = false;
+    bool pairs = false, exact = false;
     // four steps per sweep (large lattices): a second scratch copy
     char* ymem = nullptr;
     lbps::Tuning tuning;  // bulk-kernel launch shape

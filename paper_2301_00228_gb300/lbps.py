@@ -35,6 +35,7 @@ LBPS_STORAGE_F32, LBPS_STORAGE_F64, LBPS_STORAGE_BF16, LBPS_STORAGE_F16, LBPS_ST
 FIELDS = {"ux": LBPS_UX, "uy": LBPS_UY, "vx": LBPS_VX, "vy": LBPS_VY, "phi": LBPS_PHI, "psi": LBPS_PSI,
           "f_phi": LBPS_F_PHI, "f_psi": LBPS_F_PSI, "consistency": LBPS_CONSISTENCY,
           "kinetic_energy": LBPS_KINETIC_ENERGY, "strain_energy": LBPS_STRAIN_ENERGY}
+LBPS_SWEEPS_AUTO, LBPS_SWEEPS_NONE, LBPS_SWEEPS_EXACT, LBPS_SWEEPS_TWO, LBPS_SWEEPS_FOUR = range(-1, 4)
 STORAGES = {"f32": LBPS_STORAGE_F32, "f64": LBPS_STORAGE_F64, "bf16": LBPS_STORAGE_BF16,
             "f16": LBPS_STORAGE_F16, "bfp13": LBPS_STORAGE_BFP13}
 
@@ -98,6 +99,9 @@ def _load():
         "lbps_set_graph_steps": (ctypes.c_int, [vp, i32]),
         "lbps_set_step_pairs": (ctypes.c_int, [vp, i32]),
         "lbps_step_pairs": (ctypes.c_int, [vp]),
+        "lbps_set_sweeps": (ctypes.c_int, [vp, i32]),
+        "lbps_sweeps": (ctypes.c_int, [vp]),
+        "lbps_default_sweeps": (ctypes.c_int, [P(lbps_params)]),
         "lbps_profile": (ctypes.c_int, [vp, i32]),
         "lbps_profile_read": (ctypes.c_int, [vp, vp]),
         "lbps_set_stream": (ctypes.c_int, [vp, vp]),
@@ -312,6 +316,19 @@ def lbps_step_pairs(h):
     return int(_lib.lbps_step_pairs(h))
 
 
+def lbps_set_sweeps(h, kind):
+    _check(_lib.lbps_set_sweeps(h, int(kind)), "lbps_set_sweeps")
+
+
+def lbps_sweeps(h):
+    return int(_lib.lbps_sweeps(h))
+
+
+def lbps_default_sweeps(params):
+    kind = int(_lib.lbps_default_sweeps(ctypes.byref(params)))
+    return kind if kind >= 0 else _check(kind, "lbps_default_sweeps")
+
+
 def lbps_set_graph_steps(h, k):
     _check(_lib.lbps_set_graph_steps(h, int(k)), "lbps_set_graph_steps")
 
@@ -358,11 +375,10 @@ def lbps_set_origin(h, row0):
 
 # ---- convenience wrapper --------------------------------------------------
 
-# From this many points the binding turns sweeps of several steps on (FP32: four
+# From this many points a lattice takes composed sweeps by default (FP32: four
 # steps per sweep; us a step against single ones, 8192^2 567 / 1562, 4096^2 162 /
-# 400); smaller lattices take exact sweeps or many steps in one launch by
-# themselves.  FP64 storage is bound by its FP64 population arithmetic, so not
-# there.
+# 400); smaller ones take exact sweeps or many steps in one launch.  FP64 storage
+# is bound by its FP64 population arithmetic, so not there.
 PAIRS_AUTO_POINTS = 3_000_000
 
 
@@ -372,11 +388,11 @@ class Lattice:
     def __init__(self, nx, ny, lam, mu, rho=1.0, dh=1.0, a0_phi=0.9999, periodic_x=False, periodic_y=False,
                  node_type=None, bc_value=None, bc_feq_mode=0, sync_every=0, storage="f32", pop_scale_exp=0,
                  stream=None, cell=None, bc_j_mode=0, step_pairs="auto"):
-        """step_pairs: two or four time steps per sweep (lbps_set_step_pairs); "auto"
-        turns them on for lattices of at least PAIRS_AUTO_POINTS points where
-        they apply (rectangles without periodic axes) and the storage is not
-        FP64, where they are faster (the scratch state copy they need is
-        allocated then)."""
+        """step_pairs: True, two or four time steps per sweep where they apply
+        (lbps_set_step_pairs); "auto", the sweeps that are fastest by size
+        (lbps_set_sweeps): rectangles without periodic axes of 500000 points
+        and more, not FP64 storage, allocate one scratch state copy or two;
+        False, single steps, no memory beside the lattice's own."""
         import torch
 
         self.nx, self.ny = int(nx), int(ny)
@@ -395,9 +411,9 @@ class Lattice:
         self._h = lbps_create_cells(self.params, nt, bv, cl, self._mem.data_ptr(), self.nbytes)
         c, _ = lbps_info(self._h)
         self.cd, self.cs, self.a_phi, self.a_psi, self.a0_psi, self.dt = (float(x) for x in c)
-        if step_pairs == "auto":  # FP64 storage is FP64-bound with single steps already
-            step_pairs = self.nx * self.ny >= PAIRS_AUTO_POINTS and storage != "f64"
-        if step_pairs:
+        if step_pairs == "auto":
+            lbps_set_sweeps(self._h, LBPS_SWEEPS_AUTO)
+        elif step_pairs:
             lbps_set_step_pairs(self._h, 1)
             if not lbps_step_pairs(self._h):  # does not apply here: free the scratch copy
                 lbps_set_step_pairs(self._h, 0)

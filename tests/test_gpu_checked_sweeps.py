@@ -40,6 +40,8 @@ runs = 0
 for storage in ("f32", "f16", "bfp13"):
     for size, kw in (((1003, 517), {}), ((517, 1003), dict(periodic_x=True, periodic_y=True))):   # exact
         a = rect(size, storage, **kw)
+        if not kw:
+            L.lbps_set_sweeps(a._h, L.LBPS_SWEEPS_EXACT)
         same(a.step(5), rect(size, storage, True, **kw).step(5), (storage, size))
         runs += 1
     pairs = [((67, 45), storage), ((16, 16), storage)] + ([((1733, 1741), "f32")] if storage == "f32" else [])
