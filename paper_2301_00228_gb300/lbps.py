@@ -437,6 +437,15 @@ class Lattice:
         except Exception:
             pass
 
+    @property
+    def sweeps(self):
+        return lbps_sweeps(self._h)
+
+    def set_sweeps(self, kind):
+        """The sweeps its steps take (LBPS_SWEEPS_*) and the scratch they need."""
+        lbps_set_sweeps(self._h, kind)
+        return self
+
     def init(self, ux0, uy0, vx0=None, vy0=None):
         torch = self._torch
         if isinstance(ux0, torch.Tensor):

@@ -11,7 +11,8 @@ times and serves them as they arrive:
   of each kernel per time step for all of them, CUDA graphs for step pairs),
   in chunks no longer than the shortest remaining solve, so every solve stops
   exactly at its step count; a solve that is alone on the device is stepped
-  directly (lbps_step, the single-lattice kernels and their launch shape);
+  directly (lbps_step, the single-lattice kernels and their launch shape), in
+  the sweeps of its size where the budget has room for their scratch;
 * completion: finished solves leave the batch at the chunk boundary; they
   are read out (their u fields) and freed while the next chunk runs, and
   requests that arrive meanwhile are created and initialised then too (on
@@ -101,15 +102,33 @@ def pairs_apply(d):
 def footprint(d, storage="f32", pairs=False):
     """Device bytes one solve holds while admitted; with two steps per sweep
     also the scratch state copy, counted as half the lattice's block (which
-    holds two copies and more: an upper bound)."""
+    holds two copies and more: an upper bound).  A solve that is alone may be
+    granted more beside this (lone_sweeps)."""
     b = lbps.lbps_state_bytes(_params(d, storage))
     return b + b // 2 if pairs and pairs_apply(d) else b
+
+
+SCRATCH_COPIES = {lbps.LBPS_SWEEPS_NONE: 0, lbps.LBPS_SWEEPS_EXACT: 1, lbps.LBPS_SWEEPS_TWO: 1,
+                  lbps.LBPS_SWEEPS_FOUR: 2}
+
+
+def lone_sweeps(d, storage, charged, room):
+    """(kind, bytes): the sweeps of a solve that is alone, and what their scratch
+    copies take beyond the `charged` ones, within `room` bytes; the fastest kind
+    for its size, else two steps per sweep instead of four, else none."""
+    kind = lbps.lbps_default_sweeps(_params(d, storage))
+    half = lbps.lbps_state_bytes(_params(d, storage)) // 2
+    for k in (kind, lbps.LBPS_SWEEPS_TWO if kind == lbps.LBPS_SWEEPS_FOUR else lbps.LBPS_SWEEPS_NONE):
+        extra = max(0, SCRATCH_COPIES[k] - charged) * half
+        if extra <= room:
+            return k, extra
+    return lbps.LBPS_SWEEPS_NONE, 0
 
 
 def _lattice(d, storage, u0=None, stream=None):
     lat = lbps.Lattice.rectangle(d.nx, d.ny, d.lam, d.mu, d.edge_type, np.asarray(d.edge_value, float).ravel(),
                                  periodic_x=d.periodic_x, periodic_y=d.periodic_y, a0_phi=d.a0_phi,
-                                 storage=storage, stream=stream)
+                                 storage=storage, stream=stream, step_pairs=False)   # no more than its block
     ux, uy = u0 if u0 is not None else d.displacement()
     return lat.init(ux, uy)
 
@@ -170,6 +189,13 @@ def serve_batched(requests, budget_bytes, storage="f32", max_chunk=500, keep_fie
     state = {"next": 0, "used": 0}
     batch = None
     batch_members = ()
+    lone = []                    # the solve granted sweeps beyond its charge: [lattice, bytes]
+
+    def end_lone():
+        for lat, extra in lone:
+            lat.set_sweeps(lbps.LBPS_SWEEPS_NONE)
+            state["used"] -= extra
+        lone.clear()
 
     def arrivals():
         now = clk.now()
@@ -215,6 +241,9 @@ def serve_batched(requests, budget_bytes, storage="f32", max_chunk=500, keep_fie
     while state["next"] < len(reqs) or waiting or ready or active or finished:
         arrivals()
         now = clk.now()
+        if lone and (any(a[0].cancelled_by(now) for a in active) or
+                     waiting and 0 <= budget_bytes - state["used"] + lone[0][1] - foot(waiting[0].domain) < lone[0][1]):
+            end_lone()           # withdrawn, or a request fits only without its scratch
         for group in (ready, active):
             for a in [a for a in group if a[0].cancelled_by(now)]:
                 group.remove(a)
@@ -235,6 +264,7 @@ def serve_batched(requests, budget_bytes, storage="f32", max_chunk=500, keep_fie
             continue
         members = tuple(id(a[1]) for a in active)
         if members != batch_members:
+            end_lone()
             if batch is not None:
                 batch.close()
                 batch = None
@@ -245,11 +275,14 @@ def serve_batched(requests, budget_bytes, storage="f32", max_chunk=500, keep_fie
                 if pairs and all(pairs_apply(a[0].domain) for a in active):
                     batch.set_step_pairs(True)
                 rep.rebuilds += 1
-            elif pairs:
-                # alone: two steps per sweep only where they pay on one lattice
+            elif hasattr(active[0][1], "set_sweeps"):
+                # alone: the sweeps of its size, as far as the budget goes
                 d = active[0][0].domain
-                lbps.lbps_set_step_pairs(active[0][1]._h,
-                                         int(pairs_apply(d) and d.nx * d.ny >= lbps.PAIRS_AUTO_POINTS))
+                kind, extra = lone_sweeps(d, storage, int(pairs and pairs_apply(d)), budget_bytes - state["used"])
+                active[0][1].set_sweeps(kind)
+                lone.append([active[0][1], extra])
+                state["used"] += extra
+                rep.peak_bytes = max(rep.peak_bytes, state["used"])
             batch_members = members
         k = min(max_chunk, min(a[2] for a in active))
         if batch is not None:
@@ -270,6 +303,7 @@ def serve_batched(requests, budget_bytes, storage="f32", max_chunk=500, keep_fie
             a[2] -= k
         done = [a for a in active if a[2] == 0]
         if done:
+            end_lone()
             finished.extend(done)
             active = [a for a in active if a[2] > 0]
             if not active and not ready and not waiting:
@@ -295,7 +329,7 @@ def serve_one_at_a_time(requests, storage="f32", keep_fields=True, clock=time.pe
             continue
         admitted = clk.now()
         u0 = prepared.get(r.rid) if prepared else None
-        lat = _lattice(r.domain, storage, u0)
+        lat = _lattice(r.domain, storage, u0).set_sweeps(lbps.LBPS_SWEEPS_AUTO)
         lat.step(r.steps)
         res = Result(r.rid, r.arrival, admitted, 0.0)
         if keep_fields:
