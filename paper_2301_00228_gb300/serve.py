@@ -262,7 +262,7 @@ def serve_batched(requests, budget_bytes, storage="f32", max_chunk=500, keep_fie
             if state["next"] < len(reqs) and not waiting:
                 clk.wait_until(reqs[state["next"]].arrival)
             continue
-        members = tuple(id(a[1]) for a in active)
+        members = tuple(a[0].rid for a in active)   # not the lattices: a new one may lie where a closed one lay
         if members != batch_members:
             end_lone()
             if batch is not None:

@@ -38,6 +38,7 @@ class FakeLattice:
 class FakeBatch:
     def __init__(self, lats, stream=None):
         self.lats = lats
+        self.made_of = [lat.d for lat in lats]
 
     def set_step_pairs(self, on):
         for lat in self.lats:
@@ -45,6 +46,7 @@ class FakeBatch:
                 lat.set_sweeps(L.LBPS_SWEEPS_TWO)
 
     def step(self, k):
+        assert all(lat.d is d for lat, d in zip(self.lats, self.made_of)), "a batch of closed lattices"
         for lat in self.lats:
             step(lat, k)
 
@@ -144,3 +146,24 @@ def test_members_of_a_batch_hold_what_they_are_charged(serve):
 def test_a_withdrawn_lone_solve_gives_everything_back(serve):
     rep, made = serve([MID, SMALL], 2 * block(*MID), arrivals=[0.0, 40.0], steps=[4000, 50], cancel=[5.0, None])
     assert rep.cancelled == [0] and [r.rid for r in rep.results] == [1]
+
+
+@pytest.mark.parametrize("arrival", range(1, 14))
+def test_new_members_get_a_batch_of_their_own(serve, monkeypatch, arrival):
+    """Two requests that arrive as a batch of two ends, their lattices made where
+    the closed ones lay (here: the same objects)."""
+    pool = []
+
+    def recycle(d, storage, u0=None, stream=None):
+        free = [x for x in pool if x not in FakeLattice.live]
+        if not free:
+            pool.append(FakeLattice(d, storage))
+            return pool[-1]
+        free[0].__init__(d, storage)
+        return free[0]
+
+    monkeypatch.setattr(S, "_lattice", recycle)
+    BUDGET[0] = 10 * block(*MID)
+    reqs = [S.Request(q, 0.0 if q < 2 else arrival + 0.5, W.Domain(*SMALL, 1.0, 1.0), 100) for q in range(4)]
+    rep = S.serve_batched(reqs, BUDGET[0], max_chunk=100, keep_fields=False, clock=StepClock())
+    assert len(rep.results) == 4
