@@ -515,7 +515,8 @@ int lbps_set_step_pairs(lbps_lattice* lat, int32_t on);
  *   AUTO   the fastest by size (lbps_default_sweeps), with less scratch or none
  *          where the memory cannot be had.
  * LBPS_ERR_INVALID where the kind does not apply (sweeps apply to rectangles
- * without periodic axes, 16 points a side or more; AUTO is then NONE),
+ * without periodic axes, 16 points a side or more; AUTO is then NONE; with a
+ * driver that makes no tensor maps EXACT and FOUR do not apply),
  * LBPS_ERR_OOM, with the sweeps as before, without the memory.
  * lbps_sweeps: the kind in use.  lbps_default_sweeps: the kind AUTO takes for
  * a rectangle of these parameters (or an error code): EXACT from 500000 points,

@@ -451,7 +451,8 @@ bool sweeps_apply(const lbps_lattice* lat) {
 
 // Two steps per sweep, with the scratch copy allocated: composed ones, or exact
 // ones (below) unless the caller asked for single steps' timing or launch
-// shape.
+// shape.  Without tensor maps (lat->maps) two composed steps load their rows
+// through registers (pair_kernel); the other sweeps do not apply.
 bool pair_ok(const lbps_lattice* lat) {
     return lat->xmem && lat->side && sweeps_apply(lat) &&
            (lat->pairs || (lat->exact && !lat->prof && !lat->tuned));
@@ -540,7 +541,7 @@ int hold_scratch(lbps_lattice* lat, int copies, bool exact, bool pairs) {
 // scratch and without a boundary chain.
 bool periodic_pairs(const lbps_lattice* lat) {
     const lbps::Geo& g = lat->L.g;
-    return !g.general && g.periodic_x && g.periodic_y && !lat->prof && !lat->tuned &&
+    return lat->maps && !g.general && g.periodic_x && g.periodic_y && !lat->prof && !lat->tuned &&
            lat->p.storage != LBPS_STORAGE_F64 && (int64_t)g.nx * g.ny >= kExactMinPoints &&
            std::min(g.nx, g.ny) >= kExactMinSide;
 }
@@ -569,14 +570,15 @@ int run_pair(lbps_lattice* lat) {
             // beside it are not timed, as the Newmark pass of a single step)
             cudaError_t r = prof_mark(lat);
             if (r == cudaSuccess) {
-                if constexpr (sizeof(typename P::V) == 8)
-                    r = lbps::launch_pair<P>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st, 32);
-                else if (lat->pairs)
-                    r = lbps::launch_sweep<P, 2, false>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st);
-                else
-                    r = lbps::launch_sweep<P, 2, true>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st);
-                if (r == cudaErrorNotSupported && lat->pairs)   // a driver without tensor maps
-                    r = lbps::launch_pair<P>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st, 32);
+                bool swept = false;
+                if constexpr (sizeof(typename P::V) == 4)
+                    if (lat->maps) {
+                        r = lat->pairs
+                                ? lbps::launch_sweep<P, 2, false>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st)
+                                : lbps::launch_sweep<P, 2, true>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st);
+                        swept = true;
+                    }
+                if (!swept) r = lbps::launch_pair<P>(g, lat->c, lat->kc<P>(), A, B, lat->flag(), lat->st, 32);
             }
             if (r == cudaSuccess) r = prof_mark(lat);
             if (r == cudaSuccess && lat->prof) lat->ev_kind.push_back(0);
@@ -1056,6 +1058,7 @@ int lbps_create_cells(const lbps_params* params, const uint8_t* node_type, const
     lat->p = *params;
     lat->L = L;
     lat->setup_hash = setup_hash(params, bd, node_type);
+    lat->maps = lbps::tensor_maps();
     lat->st = reinterpret_cast<cudaStream_t>(params->cuda_stream);
     if (device_mem) {
         if (device_bytes < L.total || (reinterpret_cast<uintptr_t>(device_mem) % kAlign) != 0) {
@@ -1583,14 +1586,15 @@ int lbps_set_sweeps(lbps_lattice* lat, int32_t kind) {
     if (!lat || kind < LBPS_SWEEPS_AUTO || kind > LBPS_SWEEPS_FOUR) return LBPS_ERR_INVALID;
     if (kind == LBPS_SWEEPS_AUTO) {
         int k = lat->L.g.general ? LBPS_SWEEPS_NONE : default_sweeps(lat->p);
+        if (!lat->maps) k = k >= LBPS_SWEEPS_TWO ? LBPS_SWEEPS_TWO : LBPS_SWEEPS_NONE;
         int rc = lbps_set_sweeps(lat, k);
         if (rc == LBPS_ERR_OOM && k == LBPS_SWEEPS_FOUR) rc = lbps_set_sweeps(lat, LBPS_SWEEPS_TWO);
         return rc == LBPS_ERR_OOM ? lbps_set_sweeps(lat, LBPS_SWEEPS_NONE) : rc;
     }
     if (kind != LBPS_SWEEPS_NONE && !sweeps_apply(lat)) return LBPS_ERR_INVALID;
-    if (kind == LBPS_SWEEPS_EXACT && lat->p.storage == LBPS_STORAGE_F64) return LBPS_ERR_INVALID;
+    if (kind == LBPS_SWEEPS_EXACT && (!lat->maps || lat->p.storage == LBPS_STORAGE_F64)) return LBPS_ERR_INVALID;
     if (kind == LBPS_SWEEPS_FOUR &&
-        (lat->p.storage != LBPS_STORAGE_F32 || std::min(lat->p.nx, lat->p.ny) < kQuadMinSide))
+        (!lat->maps || lat->p.storage != LBPS_STORAGE_F32 || std::min(lat->p.nx, lat->p.ny) < kQuadMinSide))
         return LBPS_ERR_INVALID;
     const int copies = kind == LBPS_SWEEPS_FOUR ? 2 : kind == LBPS_SWEEPS_NONE ? 0 : 1;
     return hold_scratch(lat, copies, kind == LBPS_SWEEPS_EXACT, kind >= LBPS_SWEEPS_TWO);
@@ -1602,7 +1606,7 @@ int lbps_set_step_pairs(lbps_lattice* lat, int32_t on) {
     if (lat->pairs) return LBPS_OK;
     // without memory for the second copy of four steps per sweep the lattice
     // takes two
-    const bool four = sweeps_apply(lat) && lat->p.storage == LBPS_STORAGE_F32 &&
+    const bool four = lat->maps && sweeps_apply(lat) && lat->p.storage == LBPS_STORAGE_F32 &&
                       (int64_t)lat->p.nx * lat->p.ny >= kPairsMinPoints && std::min(lat->p.nx, lat->p.ny) >= kQuadMinSide;
     const int rc = hold_scratch(lat, four ? 2 : 1, false, true);
     return rc == LBPS_ERR_OOM && four ? hold_scratch(lat, 1, false, true) : rc;

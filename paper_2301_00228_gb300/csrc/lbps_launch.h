@@ -66,6 +66,8 @@ template <typename P>
 cudaError_t launch_frame(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, View<P> B, unsigned* flag,
                          cudaStream_t st, int fw);
 
+// Whether the driver makes the tensor maps that the sweeps' rows come by.
+bool tensor_maps();
 // K steps (2 or 4) of the points at least K + 1 from every edge, A -> B.
 // EXACT (K = 2): u, du/dt take the steps one by one, the bits of single steps.
 template <typename P, int K, bool EXACT>

@@ -92,6 +92,7 @@ struct lbps_lattice {
     // (lbps_set_sweeps).
     char* xmem = nullptr;
     bool pairs = false, exact = false;
+    bool maps = false;  // the driver makes tensor maps
     // four steps per sweep (large lattices): a second scratch copy
     char* ymem = nullptr;
     lbps::Tuning tuning;  // bulk-kernel launch shape

@@ -444,12 +444,25 @@ using EncodeFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, voi
                               const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                               CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-cudaError_t encode(CUtensorMap* m, CUtensorMapDataType type, int elem, void* base, const Geo& g, int planes, int box_x) {
+// cuTensorMapEncodeTiled of the driver, null where it has none.
+EncodeFn encode_fn() {
+#ifdef LBPS_NO_TENSOR_MAPS
+    return nullptr;
+#else
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult found;
-    cudaError_t e = cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found);
-    if (e != cudaSuccess) return e;
-    if (found != cudaDriverEntryPointSuccess) return cudaErrorNotSupported;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found) !=
+        cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return found == cudaDriverEntryPointSuccess ? reinterpret_cast<EncodeFn>(fn) : nullptr;
+#endif
+}
+
+cudaError_t encode(CUtensorMap* m, CUtensorMapDataType type, int elem, void* base, const Geo& g, int planes, int box_x) {
+    const EncodeFn fn = encode_fn();
+    if (!fn) return cudaErrorNotSupported;
 #ifdef LBPS_CHECKED
     // the copies read only inside the map (and zeros beyond it), the map only inside a live block
     if (!check_live(base, (size_t)planes * g.plane * elem)) return cudaErrorInvalidValue;
@@ -457,10 +470,9 @@ cudaError_t encode(CUtensorMap* m, CUtensorMapDataType type, int elem, void* bas
     const cuuint64_t dims[3] = {(cuuint64_t)g.px, (cuuint64_t)g.ny, (cuuint64_t)planes};
     const cuuint64_t strides[2] = {(cuuint64_t)g.px * elem, (cuuint64_t)g.plane * elem};
     const cuuint32_t box[3] = {(cuuint32_t)box_x, 2, (cuuint32_t)planes}, one[3] = {1, 1, 1};
-    const CUresult r = reinterpret_cast<EncodeFn>(fn)(m, type, 3, base, dims, strides, box, one,
-                                                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
-                                                      CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                                                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    const CUresult r = fn(m, type, 3, base, dims, strides, box, one, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                          CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
@@ -496,6 +508,8 @@ int sweep2_rows(const Geo& g, int blocks_x, int height, int per_sm, int free) {
 }
 
 }  // namespace
+
+bool tensor_maps() { return encode_fn() != nullptr; }
 
 template <typename P, int K, bool EXACT>
 cudaError_t launch_sweep(const Geo& g, const Consts& c, const KCof<P>& k, View<P> A, View<P> B, unsigned* flag,
