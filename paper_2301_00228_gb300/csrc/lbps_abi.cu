@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -774,6 +775,44 @@ bool fused_ok(const lbps_lattice* lat) {
            (int64_t)lat->L.g.nx * lat->L.g.ny <= kFusedMaxPoints;
 }
 
+// The mapped host words of many-step launches: pairs out of one page that the
+// process keeps, as freeing page-locked memory waits for the whole device (a
+// lattice closed beside 628 ms of other work: 30 us against those 628 ms).
+class HostWords {
+  public:
+    unsigned* take() {
+        const std::lock_guard<std::mutex> lock(m_);
+        if (!page_) {
+            if (cudaHostAlloc(reinterpret_cast<void**>(&page_), kPage, cudaHostAllocMapped | cudaHostAllocPortable) !=
+                cudaSuccess) {
+                cudaGetLastError();
+                page_ = nullptr;
+                return nullptr;
+            }
+            for (size_t q = kPage / kPair; q-- > 0;) free_.push_back(page_ + q * (kPair / sizeof(unsigned)));
+        }
+        if (free_.empty()) return nullptr;
+        unsigned* w = free_.back();
+        free_.pop_back();
+        return w;
+    }
+    void give_back(unsigned* w) {
+        const std::lock_guard<std::mutex> lock(m_);
+        free_.push_back(w);
+    }
+
+  private:
+    static constexpr size_t kPage = 16384, kPair = 2 * sizeof(unsigned);   // 2048 lattices
+    std::mutex m_;
+    unsigned* page_ = nullptr;
+    std::vector<unsigned*> free_;
+};
+
+HostWords& host_words() {
+    static HostWords* w = new HostWords;   // lives as long as any lattice may
+    return *w;
+}
+
 // m steps in one launch (launch_fused); *done = false where the device
 // refuses the cooperative launch (the steps then run as separate launches).
 int run_fused(lbps_lattice* lat, int m, bool* done) {
@@ -784,6 +823,7 @@ int run_fused(lbps_lattice* lat, int m, bool* done) {
                                      lat->L.nb, lat->flag(), lat->tstep(), lat->bar(), lat->host_flag, m, lat->st);
     });
     *done = e == cudaSuccess;
+    lat->unchecked = true;
     if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
         cudaGetLastError();
         lat->fused_off = true;
@@ -1146,12 +1186,8 @@ int lbps_create_cells(const lbps_params* params, const uint8_t* node_type, const
         // at 6 blocks per SM; one row ahead fits in 80 registers
         if (params->storage == LBPS_STORAGE_BFP13) lat->tuning.variant = 4;
     }
-    if ((int64_t)params->nx * params->ny <= kFusedMaxPoints &&
-        cudaHostAlloc(reinterpret_cast<void**>(&lat->host_flag), 2 * sizeof(unsigned),
-                      cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
-        cudaGetLastError();
-        lat->host_flag = nullptr;   // lbps_check then copies the flag
-    }
+    // (without the words lbps_check copies the flag)
+    if ((int64_t)params->nx * params->ny <= kFusedMaxPoints) lat->host_flag = host_words().take();
     // the side stream of the boundary Newmark pass; if it cannot be had, the
     // pass runs on the lattice's stream (same results, no overlap).  It has
     // the greatest priority: its short dependent launches then take SM slots
@@ -1325,6 +1361,7 @@ int lbps_check(lbps_lattice* lat) {
         lat->last_cuda = (int)e;
         return LBPS_ERR_CUDA;
     }
+    lat->unchecked = lat->moved;
     // only many-step launches since the initialisation: their host words say the
     // same without a copy (a launch and its check 9.9 us against 14.7)
     if (!lat->flag_other) {
@@ -1742,6 +1779,7 @@ int lbps_set_origin(lbps_lattice* lat, int64_t row0) {
 
 int lbps_set_stream(lbps_lattice* lat, void* cuda_stream) {
     if (!lat) return LBPS_ERR_INVALID;
+    lat->moved |= lat->unchecked;   // waiting for the new stream says nothing about launches on the old one
     lat->st = reinterpret_cast<cudaStream_t>(cuda_stream);
     lat->p.cuda_stream = cuda_stream;
     return LBPS_OK;
@@ -1761,8 +1799,10 @@ void lbps_destroy(lbps_lattice* lat) {
     if (lat->xmem) cudaStreamSynchronize(lat->st);
     drop_scratch(lat);
     if (lat->host_flag) {
-        cudaStreamSynchronize(lat->st);
-        cudaFreeHost(lat->host_flag);
+        // no launch may write the words once they are another lattice's; where
+        // none is known to be over (the stream may be gone by now), wait for all
+        if (lat->unchecked) cudaDeviceSynchronize();
+        host_words().give_back(lat->host_flag);
     }
     if (lat->owns && lat->mem) {
         cudaStreamSynchronize(lat->st);

@@ -101,6 +101,8 @@ struct lbps_lattice {
     // mapped host words that launch_fused sets beside the flag (null: none), and
     // whether anything else may have set the flag since the initialisation
     unsigned* host_flag = nullptr;
+    bool unchecked = false;  // many-step launches may be under way,
+    bool moved = false;      // some of them on a stream the lattice has left
     bool flag_other = true;
     bool captured = false;   // steps were captured by the caller: replays may set the flag any time
     int last_cuda = 0;    // cudaError_t of the last failing CUDA call
