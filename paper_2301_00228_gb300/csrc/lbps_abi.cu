@@ -2,8 +2,10 @@
 // include/lbps.h).  Host-side work only: validation, the rectangle helper,
 // the device memory layout, and enqueueing the kernels of lbps_kernels.cu.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <new>
 #include <vector>
@@ -770,9 +772,54 @@ constexpr int64_t kFusedMaxPoints = 1200000;
 // Steps per launch at most (tens of milliseconds at the largest size).
 constexpr int64_t kFusedMaxSteps = 1024;
 
-bool fused_ok(const lbps_lattice* lat) {
-    return !lat->fused_off && !lat->prof && !lat->tuned && !pair_ok(lat) && !periodic_pairs(lat) &&
-           (int64_t)lat->L.g.nx * lat->L.g.ny <= kFusedMaxPoints;
+// The streams that live lattices use.  A many-step launch takes every SM for
+// itself, so lattices on several streams run one after the other in it, where
+// their separate launches run side by side.
+class StreamsInUse {
+  public:
+    void add(cudaStream_t st) {
+        const std::lock_guard<std::mutex> lock(m_);
+        ++uses_[st];
+        distinct_.store((int)uses_.size(), std::memory_order_relaxed);
+    }
+    void drop(cudaStream_t st) {
+        const std::lock_guard<std::mutex> lock(m_);
+        const auto it = uses_.find(st);
+        if (it != uses_.end() && --it->second == 0) uses_.erase(it);
+        distinct_.store((int)uses_.size(), std::memory_order_relaxed);
+    }
+    int distinct() const { return distinct_.load(std::memory_order_relaxed); }
+
+  private:
+    std::mutex m_;
+    std::map<cudaStream_t, int> uses_;
+    std::atomic<int> distinct_{0};
+};
+
+StreamsInUse& streams_in_use() {
+    static StreamsInUse* s = new StreamsInUse;   // lives as long as any lattice may
+    return *s;
+}
+
+// Many-step launches beside lattices on other streams: small lattices only, up
+// to this many points where two streams are in use or a single step is asked
+// for, up to kFusedSharedPoints otherwise.  Measured, us for a step of all
+// lattices (FP32, calls of 20 steps; calls of one step), many-step against
+// separate launches: 2 lattices of 160 x 128 8.1 / 12.4 (12.5 / 17.2), of 200 x
+// 150 15.6 / 13.4 (17.7 / 16.7); 8 of 100 x 64 16.7 / 23.8 (22.7 / 60.7), of 128
+// x 96 30.2 / 24.4 (28.9 / 61.2), of 160 x 128 31.0 / 24.7 (37.1 / 62.0), of 300 x
+// 300 70 / 31 (91 / 61); 4 of 700 x 500 56 / 39 (74 / 40).
+constexpr int64_t kFusedSharedPoints1 = 20480;
+constexpr int64_t kFusedSharedPoints = 8192;
+
+// n: the steps asked for.
+bool fused_ok(const lbps_lattice* lat, int64_t n) {
+    const int64_t points = (int64_t)lat->L.g.nx * lat->L.g.ny;
+    const int streams = streams_in_use().distinct();
+    const int64_t most = streams <= 1             ? kFusedMaxPoints
+                         : streams == 2 || n == 1 ? kFusedSharedPoints1
+                                                  : kFusedSharedPoints;
+    return !lat->fused_off && !lat->prof && !lat->tuned && !pair_ok(lat) && !periodic_pairs(lat) && points <= most;
 }
 
 // The mapped host words of many-step launches: pairs out of one page that the
@@ -1186,6 +1233,7 @@ int lbps_create_cells(const lbps_params* params, const uint8_t* node_type, const
         // at 6 blocks per SM; one row ahead fits in 80 registers
         if (params->storage == LBPS_STORAGE_BFP13) lat->tuning.variant = 4;
     }
+    streams_in_use().add(lat->st);
     // (without the words lbps_check copies the flag)
     if ((int64_t)params->nx * params->ny <= kFusedMaxPoints) lat->host_flag = host_words().take();
     // the side stream of the boundary Newmark pass; if it cannot be had, the
@@ -1289,7 +1337,7 @@ int lbps_step_async(lbps_lattice* lat, int64_t n) {
         cudaGetLastError();
         lat->captured = true;
     }
-    bool fused = !capturing && fused_ok(lat);
+    bool fused = !capturing && fused_ok(lat, n);
     for (int64_t s = 0; s < n;) {
         if (fused) {
             int64_t m = std::min(n - s, kFusedMaxSteps);
@@ -1780,7 +1828,9 @@ int lbps_set_origin(lbps_lattice* lat, int64_t row0) {
 int lbps_set_stream(lbps_lattice* lat, void* cuda_stream) {
     if (!lat) return LBPS_ERR_INVALID;
     lat->moved |= lat->unchecked;   // waiting for the new stream says nothing about launches on the old one
+    streams_in_use().drop(lat->st);
     lat->st = reinterpret_cast<cudaStream_t>(cuda_stream);
+    streams_in_use().add(lat->st);
     lat->p.cuda_stream = cuda_stream;
     return LBPS_OK;
 }
@@ -1809,6 +1859,7 @@ void lbps_destroy(lbps_lattice* lat) {
         cudaFree(lat->mem);
     }
     for (cudaEvent_t e : lat->ev_pool) cudaEventDestroy(e);
+    streams_in_use().drop(lat->st);
     delete lat;
 }
 
