@@ -465,7 +465,9 @@ int lbps_check_report(uint64_t out[2]);
  * lattice whose launch shape was set takes its single steps as launches of
  * that shape; otherwise lattices up to 1200000 points take many steps in one
  * cooperative launch (the same bits; not while lbps_profile records or the
- * stream is being captured). */
+ * stream is being captured, not rectangles with more than 8192 or 16384
+ * boundary points, by storage and size, and where the process has lattices on
+ * several streams only those up to 8192 or 20480 points). */
 int lbps_set_tuning(lbps_lattice* lat, int32_t variant, int32_t rows_per_warp);
 
 /* Steps per CUDA graph of lbps_step: k even, 2..64 (LBPS_ERR_INVALID
@@ -519,8 +521,8 @@ int lbps_set_step_pairs(lbps_lattice* lat, int32_t on);
  * driver that makes no tensor maps EXACT and FOUR do not apply),
  * LBPS_ERR_OOM, with the sweeps as before, without the memory.
  * lbps_sweeps: the kind in use.  lbps_default_sweeps: the kind AUTO takes for
- * a rectangle of these parameters (or an error code): EXACT from 500000 points,
- * FOUR or TWO from 3000000. */
+ * a rectangle of these parameters (or an error code): EXACT from 500000 points
+ * and 128 columns, FOUR or TWO from 3000000 points. */
 #define LBPS_SWEEPS_AUTO (-1)
 #define LBPS_SWEEPS_NONE 0
 #define LBPS_SWEEPS_EXACT 1

@@ -468,9 +468,12 @@ bool pair_ok(const lbps_lattice* lat) {
 // against single steps: 700 x 500 14.6 / 13.4, 800^2 15.4 / 19.7 (BF16 18.7 /
 // 22.2), 1024^2 21.0 / 27.4 (BF16 24.7 / 33.9, BFP13 23.9 / 38.0), 1600^2 46 / 74;
 // periodic 512^2 10.3 / 8.9, 768^2 12.0 / 14.7, 1024^2 17.7 / 27.4, 2048^2 59 /
-// 103.
+// 103.  Narrow lattices lose (the columns of the side bands, a sector each, are a
+// large part of the chain), exact over single steps, FP32 / FP16 / BFP13: 64 x
+// 34375 1.06 / 1.04 / 1.05, 90 x 24444 1.05 / 1.09 / 1.08, 128 x 17187 0.84 / 0.85 /
+// 0.88; flat ones gain, 34375 x 64 0.77 / 0.91 / 0.84.
 constexpr int64_t kExactMinPoints = 500000;
-constexpr int32_t kExactMinSide = 64;
+constexpr int32_t kExactMinSide = 64, kExactMinWidth = 128;
 // Composed sweeps by default from here; four steps per sweep in FP32 storage
 // (the others' codecs bind four steps: BFP13 4096^2 263 us a step against 201
 // with two; FP32 2047 x 1533: 35.6 us a step against 54 with two).
@@ -485,8 +488,8 @@ int default_sweeps(const lbps_params& p) {
     if (p.periodic_x || p.periodic_y || p.storage == LBPS_STORAGE_F64 || side < 16) return LBPS_SWEEPS_NONE;
     if (points >= kPairsMinPoints)
         return p.storage == LBPS_STORAGE_F32 && side >= kQuadMinSide ? LBPS_SWEEPS_FOUR : LBPS_SWEEPS_TWO;
-    return points >= kExactMinPoints && side >= kExactMinSide && p.sync_every != 1 ? LBPS_SWEEPS_EXACT
-                                                                                   : LBPS_SWEEPS_NONE;
+    const bool exact = points >= kExactMinPoints && side >= kExactMinSide && p.nx >= kExactMinWidth && p.sync_every != 1;
+    return exact ? LBPS_SWEEPS_EXACT : LBPS_SWEEPS_NONE;
 }
 
 // A scratch copy of a lattice's sweeps, zeroed once: parts of it the frame
@@ -812,6 +815,23 @@ StreamsInUse& streams_in_use() {
 constexpr int64_t kFusedSharedPoints1 = 20480;
 constexpr int64_t kFusedSharedPoints = 8192;
 
+// Rectangles with this many boundary points or more take separate launches:
+// their boundary passes then fill a grid of their own, where the many-step
+// launch has 16 warps per SM, and its blocks no longer hold their part of the
+// boundary table.  A plate with holes gains with any number (its interior pass
+// looks at node types).  Measured, many-step over separate launches, FP32 / FP16 /
+// BFP13 / FP64 (points, boundary points): 100 000, 12528 0.78 / 0.82 / 0.83 / 0.82 (16
+// wide), 300 000, 12592 0.80 / 0.98 / 0.90 / 0.88 (48 wide) and 0.90 / 1.05 / 1.02 / 0.81
+// (48 high); 480 000, 9796 0.89 / 1.11 / 1.00 / 0.94 (100 wide), 15124 0.96 / 1.17 / 1.05 /
+// 0.89 (64 wide) and 0.97 / 1.33 / 1.14 / 0.90 (64 high); 300 000, 25044 1.26 / 1.58 / 1.39
+// / 1.02 (24 high); 1 100 000, 91710 1.24 / 1.35 / 1.30 / 1.10 (24 high); plates with
+// 28892 .. 133956 boundary points 0.94 .. 1.00 / 0.84 .. 1.11 / 0.90 .. 1.05 / 0.85 .. 0.96.
+bool many_boundary_points(const lbps_lattice* lat) {
+    const bool pairs16 = lat->p.storage != LBPS_STORAGE_F32 && lat->p.storage != LBPS_STORAGE_F64;
+    const bool few = (int64_t)lat->L.g.nx * lat->L.g.ny <= (1 << 17);
+    return !lat->L.g.general && lat->L.nb > (pairs16 && !few ? 8192 : 16384);
+}
+
 // n: the steps asked for.
 bool fused_ok(const lbps_lattice* lat, int64_t n) {
     const int64_t points = (int64_t)lat->L.g.nx * lat->L.g.ny;
@@ -819,7 +839,8 @@ bool fused_ok(const lbps_lattice* lat, int64_t n) {
     const int64_t most = streams <= 1             ? kFusedMaxPoints
                          : streams == 2 || n == 1 ? kFusedSharedPoints1
                                                   : kFusedSharedPoints;
-    return !lat->fused_off && !lat->prof && !lat->tuned && !pair_ok(lat) && !periodic_pairs(lat) && points <= most;
+    return !lat->fused_off && !lat->prof && !lat->tuned && !pair_ok(lat) && !periodic_pairs(lat) && points <= most &&
+           !many_boundary_points(lat);
 }
 
 // The mapped host words of many-step launches: pairs out of one page that the

@@ -15,6 +15,7 @@ def L():
     (708, 708, "f64", {}, "NONE"), (708, 708, "f32", dict(sync_every=1), "NONE"),
     (708, 708, "f32", dict(sync_every=2), "EXACT"), (708, 708, "f32", dict(periodic_x=1), "NONE"),
     (9000, 63, "f32", {}, "NONE"), (9000, 64, "f32", {}, "EXACT"),
+    (127, 9000, "f16", {}, "NONE"), (128, 9000, "f16", {}, "EXACT"), (64, 46874, "f32", {}, "NONE"),
     (1733, 1732, "f32", {}, "FOUR"), (1733, 1732, "bfp13", {}, "TWO"), (1733, 1732, "f64", {}, "NONE"),
     (60000, 63, "f32", {}, "TWO"), (200000, 15, "f32", {}, "NONE"), (1733, 1732, "f32", dict(periodic_y=1), "NONE")])
 def test_default_sweeps(L, nx, ny, storage, kw, want):
