@@ -101,3 +101,19 @@ def test_energy_call_order(L):
     k0, s0, t0 = lat.energy()
     assert k0 == 0.0 and s0 > 0 and t0 == s0     # initial state at rest
     lat.close()
+
+
+@pytest.mark.parametrize("size", [(2047, 3), (2048, 3), (20000, 20), (100003, 16), (9001, 300), (5000, 1030)])
+def test_energy_of_flat_lattices(L, size):
+    """Rows split over blocks: the sum still equals that of the densities (FP64
+    summation in another order: within points x 2^-53 of it, all terms >= 0)."""
+    nx, ny = size
+    lat = L.Lattice.rectangle(nx, ny, 1.5, 1.0, (2, 1, 1, 2), np.zeros(8), a0_phi=0.99)
+    rng = np.random.default_rng(nx)
+    lat.init(*(1e-3 * rng.standard_normal((4, ny, nx)))).step(2)
+    e = lat.energy()
+    for q, k in enumerate(("kinetic_energy", "strain_energy")):
+        want = lat.read(k).sum()
+        assert want > 0 and abs(e[q] - want) <= nx * ny * 2.0**-53 * want, k
+    assert e[2] == e[0] + e[1]
+    lat.close()
