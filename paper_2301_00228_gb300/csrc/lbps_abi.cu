@@ -10,6 +10,8 @@
 #include <new>
 #include <vector>
 
+#include <cuda.h>
+
 #include "lbps.h"
 #include "lbps_launch.h"
 #include "lbps_state.h"
@@ -843,37 +845,59 @@ bool fused_ok(const lbps_lattice* lat, int64_t n) {
            !many_boundary_points(lat);
 }
 
-// The mapped host words of many-step launches: pairs out of one page that the
-// process keeps, as freeing page-locked memory waits for the whole device (a
-// lattice closed beside 628 ms of other work: 30 us against those 628 ms).
+// The mapped host words of many-step launches: pairs out of one page per CUDA
+// context that the process keeps, as freeing page-locked memory waits for the
+// whole device (a lattice closed beside 628 ms of other work: 30 us against
+// those 628 ms).  A page is gone with its context: after a device reset the
+// context has another id, and a new page.
 class HostWords {
   public:
-    unsigned* take() {
+    static constexpr size_t kPairs = 2048;
+    // null where no words can be had; *page is for give_back
+    unsigned* take(int* page) {
+        unsigned long long id = 0;
+        if (!context_id(&id)) return nullptr;
         const std::lock_guard<std::mutex> lock(m_);
-        if (!page_) {
-            if (cudaHostAlloc(reinterpret_cast<void**>(&page_), kPage, cudaHostAllocMapped | cudaHostAllocPortable) !=
-                cudaSuccess) {
+        size_t q = 0;
+        while (q < pages_.size() && pages_[q].context != id) ++q;
+        if (q == pages_.size()) {
+            unsigned* base = nullptr;
+            if (cudaHostAlloc(reinterpret_cast<void**>(&base), kPairs * 2 * sizeof(unsigned),
+                              cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
                 cudaGetLastError();
-                page_ = nullptr;
                 return nullptr;
             }
-            for (size_t q = kPage / kPair; q-- > 0;) free_.push_back(page_ + q * (kPair / sizeof(unsigned)));
+            pages_.push_back(Page{id, {}});
+            for (size_t w = kPairs; w-- > 0;) pages_[q].free.push_back(base + 2 * w);
         }
-        if (free_.empty()) return nullptr;
-        unsigned* w = free_.back();
-        free_.pop_back();
+        if (pages_[q].free.empty()) return nullptr;
+        unsigned* w = pages_[q].free.back();
+        pages_[q].free.pop_back();
+        *page = (int)q;
         return w;
     }
-    void give_back(unsigned* w) {
+    void give_back(int page, unsigned* w) {
         const std::lock_guard<std::mutex> lock(m_);
-        free_.push_back(w);
+        pages_[(size_t)page].free.push_back(w);
     }
 
   private:
-    static constexpr size_t kPage = 16384, kPair = 2 * sizeof(unsigned);   // 2048 lattices
+    struct Page {
+        unsigned long long context;
+        std::vector<unsigned*> free;
+    };
+    static bool context_id(unsigned long long* id) {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        return found == cudaDriverEntryPointSuccess &&
+               reinterpret_cast<CUresult (*)(CUcontext, unsigned long long*)>(fn)(nullptr, id) == CUDA_SUCCESS;
+    }
     std::mutex m_;
-    unsigned* page_ = nullptr;
-    std::vector<unsigned*> free_;
+    std::vector<Page> pages_;
 };
 
 HostWords& host_words() {
@@ -1255,8 +1279,6 @@ int lbps_create_cells(const lbps_params* params, const uint8_t* node_type, const
         if (params->storage == LBPS_STORAGE_BFP13) lat->tuning.variant = 4;
     }
     streams_in_use().add(lat->st);
-    // (without the words lbps_check copies the flag)
-    if ((int64_t)params->nx * params->ny <= kFusedMaxPoints) lat->host_flag = host_words().take();
     // the side stream of the boundary Newmark pass; if it cannot be had, the
     // pass runs on the lattice's stream (same results, no overlap).  It has
     // the greatest priority: its short dependent launches then take SM slots
@@ -1277,6 +1299,8 @@ int lbps_create_cells(const lbps_params* params, const uint8_t* node_type, const
         lat->side = nullptr;
         lat->fork = lat->join = nullptr;
     }
+    // (without the words lbps_check copies the flag; the streams above made the context)
+    if ((int64_t)params->nx * params->ny <= kFusedMaxPoints) lat->host_flag = host_words().take(&lat->host_page);
     if (L.g.general) {
         lat->L.g.type = reinterpret_cast<const uint8_t*>(lat->mem + L.off_type);
         lat->L.g.gap = reinterpret_cast<const int*>(lat->mem + L.off_gap);
@@ -1873,7 +1897,7 @@ void lbps_destroy(lbps_lattice* lat) {
         // no launch may write the words once they are another lattice's; where
         // none is known to be over (the stream may be gone by now), wait for all
         if (lat->unchecked) cudaDeviceSynchronize();
-        host_words().give_back(lat->host_flag);
+        host_words().give_back(lat->host_page, lat->host_flag);
     }
     if (lat->owns && lat->mem) {
         cudaStreamSynchronize(lat->st);

@@ -101,6 +101,7 @@ struct lbps_lattice {
     // mapped host words that launch_fused sets beside the flag (null: none), and
     // whether anything else may have set the flag since the initialisation
     unsigned* host_flag = nullptr;
+    int host_page = 0;       // the page they are from
     bool unchecked = false;  // many-step launches may be under way,
     bool moved = false;      // some of them on a stream the lattice has left
     bool flag_other = true;

@@ -56,3 +56,36 @@ def test_more_lattices_than_host_words(L):
     assert [lat.check() for lat in more] == [L.LBPS_ERR_NONFINITE if q % 3 == 1 else 0 for q in range(len(more))]
     for lat in more + lats[1::2]:
         lat.close()
+
+
+def test_lattices_after_a_device_reset():
+    """The page of host words goes with its context; lattices made after a reset
+    get one of their own.  In a child process, the library's own memory."""
+    import subprocess
+    import sys
+    from pathlib import Path
+
+    root = Path(__file__).resolve().parents[1]
+    code = f"import sys; sys.path.insert(0, {str(root)!r})" + r"""
+import ctypes
+import numpy as np
+from paper_2301_00228_gb300 import lbps as L
+
+def run():
+    nt, bv = L.lbps_rect_bc(32, 24, False, False, 1.0, (2, 1, 1, 2), np.zeros(8))
+    h = L.lbps_create(L.lbps_params(32, 24, 1.5, 1.0, 1.0, 1.0, 0.99, 0, 0, 0, 0, 0, 0, None), nt, bv, 0, 0)
+    u = 1e-3 * np.random.default_rng(1).standard_normal((24, 32))
+    L.lbps_init(h, u, u)
+    assert L._lib.lbps_step(h, 20) == 0
+    out = np.zeros((24, 32))
+    L.lbps_read(h, L.LBPS_UX, out)
+    L.lbps_destroy(h)
+    return out
+
+a = run()
+assert ctypes.CDLL("libcuda.so.1").cuDevicePrimaryCtxReset_v2(0) == 0
+assert np.array_equal(a, run()) and np.array_equal(a, run())
+print("OK")
+"""
+    out = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert out.returncode == 0 and out.stdout.strip().endswith("OK"), out.stdout + out.stderr
