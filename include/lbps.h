@@ -500,7 +500,7 @@ int lbps_set_graph_steps(lbps_lattice* lat, int32_t k);
  * The sweep runs beside a chain
  * of boundary and frame launches on a second stream of greatest priority.
  * It pays from about 800^2 points (FP32, us a step against single steps:
- * 8192^2 567 / 1562; 4096^2 162 / 400; 2047 x 1533 36 / 85). */
+ * 8192^2 554 / 1565; 4096^2 156 / 400; 2047 x 1533 37 / 85). */
 int lbps_set_step_pairs(lbps_lattice* lat, int32_t on);
 
 /* The sweeps lbps_step takes on a lattice, and the scratch state copies (beside

@@ -7,10 +7,10 @@
 // 5000 where every thread has stores on the way).  Every block keeps its tasks
 // and its boundary table for all steps, and one warp takes one strip of a few
 // rows, so that a phase is one wave.  Against graphs of 32 steps (three
-// launches a step): 64^2 FP64 storage 10.9 us a step against 15.7, 300^2 FP32
-// 8.7 against 10.2, 389 x 1171 15.7 against 18.1, 1024^2 with a hole 41.8
-// against 45.7; a single step through lbps_step on 128 x 96 26.8 us against
-// 32.5.
+// launches a step): 64^2 FP64 storage 10.6 us a step against 15.7, 300^2 FP32
+// 8.9 against 10.3, 389 x 1171 15.6 against 20.0, 1024^2 with a hole 39.4
+// against 45.7; a single step through lbps_step on 128 x 96 19.8 us against
+// 32.1.
 #include <algorithm>
 
 #include "lbps_steps.cuh"

@@ -310,13 +310,13 @@ __device__ __forceinline__ void init_ring(unsigned long long* bars) {
 }
 
 // What bounds it: K = 4 in FP32, the FP64 pipe (12 instructions of 64 cycles a
-// row and warp; 79 % busy on 3072^2, issue 54 %, DRAM 53 %, 320 us for 4 steps);
-// K = 2 in the 16-bit formats, the issue slots their codec takes (BFP13 76 %,
-// FP64 49 %, DRAM 69 %, 220 us for 2 steps; K = 4 takes 556 us for 4).  The
+// row and warp; 75 % busy on 3072^2, issue 49 %, DRAM 46 %, 363 us for 4 steps);
+// K = 2 in the 16-bit formats, the issue slots their codec takes (BFP13 77 %,
+// FP64 52 %, DRAM 73 %, 208 us for 2 steps; K = 4 takes 556 us for 4).  The
 // rows come by TMA, two at a time and DEPTH pairs ahead, so no registers hold
 // rows in flight: the kernel this replaced loaded them through registers, one
 // row ahead, and waited on them (8192^2, two steps: FP32 1784 us, FP16 1632;
-// now FP32 two steps 1626, four steps 2304; FP16 1443).  Blocks per SM: what
+// now FP32 two steps 1626, four steps 2214; FP16 1398).  Blocks per SM: what
 // the registers allow without spilling in earnest (K = 4 at 128 registers
 // spills 314 bytes and takes 3340 us).
 template <typename P, int K, int MINB, bool EXACT>
@@ -478,10 +478,12 @@ cudaError_t encode(CUtensorMap* m, CUtensorMapDataType type, int elem, void* bas
 
 // Rows per chunk.  Tall chunks recompute fewer rows around them; short ones
 // end more often, so that the boundary launches beside the sweep find room
-// on the SMs, and fill the last wave.  Measured, us a step: K = 4 FP32 2047
-// x 1533 41.8 / 43.0 / 35.6 / 46.1 with 32 / 64 / 96 / 128 rows, 8192^2
-// 601 / 578 / 576 / 578; K = 2 FP16 2047 x 1533 48.1 / 49.2 / 71.1 with 16 /
-// 32 / 64 rows, 4096^2 204 / 201 / -, BFP13 4096^2 206 / 201 / 211.
+// on the SMs, and fill the last wave.  Measured, us a step: K = 4 FP32 8192^2
+// 601 / 578 / 576 / 578 with 32 / 64 / 96 / 128 rows: any height from 64 on, so 96,
+// which fills the last wave of 2047 x 1533 (41.8 / 43.0 / 35.6 / 46.1) but not of
+// every size (2048^2 58 us, 1.2 times the time a point); K = 2 FP16 2047 x 1533
+// 48.1 / 49.2 / 71.1 with 16 / 32 / 64 rows, 4096^2 204 / 201 / -, BFP13 4096^2
+// 206 / 201 / 211.
 // Below 6 M points a K = 2 launch is a few waves of blocks: the height of 16 .. 32
 // rows whose waves cost least, a chunk costing its rows and 8 around them
 // (1024^2 BF16: 16 rows are 640 blocks on 608 places). free: places left to the

@@ -376,7 +376,7 @@ def lbps_set_origin(h, row0):
 # ---- convenience wrapper --------------------------------------------------
 
 # From this many points a lattice takes composed sweeps by default (FP32: four
-# steps per sweep; us a step against single ones, 8192^2 567 / 1562, 4096^2 162 /
+# steps per sweep; us a step against single ones, 8192^2 554 / 1565, 4096^2 156 /
 # 400); smaller ones take exact sweeps or many steps in one launch.  FP64 storage
 # is bound by its FP64 population arithmetic, so not there.
 PAIRS_AUTO_POINTS = 3_000_000
